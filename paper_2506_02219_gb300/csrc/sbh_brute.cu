@@ -1,203 +1,407 @@
-// sbh_brute.cu -- the exact kernel sum F(q) = sum_i m_i f(p_i, q) (Madan et al. 2025, Eq. 1) by
-// tiled brute force: each block stages a tile of sources in shared memory and every thread sums
-// the tile for its query (the classic all-pairs layout the paper uses for ground truth, Sec. 4.3).
-// With fp64_accum each tile's FP32 partial sum is added into an FP64 accumulator, which keeps
-// the rounding error of million-term sums at the level of one tile; this is the error reference.
+// sbh_brute.cu -- the exact kernel sum F(q) = sum_i m_i f(p_i, q) (Madan et al. 2025, Eq. 1) and its
+// query gradient by tiled brute force (the paper's ground truth, Sec. 4.3).
+//
+// A block of eight warps works on one group of 32 x QPT queries, QPT to a lane, and every warp of it on
+// another eighth of each source tile; a cluster of up to eight blocks splits the sources further. So
+// a few thousand queries fill the chip (5,001 queries: 79 groups of 64 make 632 blocks instead of
+// the 20 that one query per thread makes), and a source read from shared memory serves QPT queries.
+// Partial sums meet in shared memory, then across the cluster's distributed shared memory, always in
+// the same order: no scratch memory, no atomics, results reproducible.
+//
+// Sources are staged two by two, so that the packed FP32 instructions take both of a pair at once.
+// What bounds it: the FP32 pipe's register reads. A winding term is 12 FMA-pipe operations, most of them on
+// three different registers, which this chip runs at 1.6 cycles per warp and scheduler (1.1 with a
+// repeated operand; measured, packed or scalar alike): 19 cycles a term, of which the reciprocal root's 8.4
+// run beside. The Coulomb term takes 9.7 cycles, near the root's own rate.
+// 65,536 queries against 2^20 sources, winding: 49.1 -> 32.2 ms; smooth distance and gradient, 5,001
+// queries against 2^19 sources: 47.3 -> 2.5 ms (one query per thread ran on 20 of 152 SMs, and the FP64
+// sums were rescaled with every new smallest distance).
+//
+// With fp64_accum every FP32 partial sum of at most 256 terms is added into an FP64 accumulator, which
+// keeps the rounding error of million-term sums at the level of one such partial.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "sbh_eval.cuh"
+#include "sbh_f32x2.cuh"
 
 namespace sbh {
 
-constexpr int kBruteThreads = 256;
-constexpr int kBruteTile = 256;
+namespace {
 
-template <int KIND, bool FP64>
+namespace cg = cooperative_groups;
+
+constexpr int kBruteWarps = 8;
+constexpr int kBruteThreads = 32 * kBruteWarps;
+constexpr int kWarpTile = 128;                       // sources of a tile that one warp takes
+constexpr int kBruteTile = kWarpTile * kBruteWarps;  // sources staged at a time
+constexpr int kFlushTiles = 2;                       // tiles per FP32 partial: 256 terms at most
+constexpr int kMaxCluster = 8;
+
+__device__ __forceinline__ float ex2_ftz(float x)
+{
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// A pair of staged sources: (x0 x1 y0 y1)(z0 z1 s0 s1) with s the mass, or for the winding kernel
+// z of the dipole m n, whose x and y follow: (nx0 nx1 ny0 ny1)
+template <int KIND>
+struct Pair {
+    static constexpr int kQuads = KIND == SBH_WINDING ? 3 : 2;
+    f2 x, y, z, s, nx, ny;
+    __device__ __forceinline__ void load(const float4* t)
+    {
+        const float4 a = t[0], b = t[1];
+        x = f2_make(a.x, a.y); y = f2_make(a.z, a.w);
+        z = f2_make(b.x, b.y); s = f2_make(b.z, b.w);
+        if constexpr (KIND == SBH_WINDING) {
+            const float4 c = t[2];
+            nx = f2_make(c.x, c.y); ny = f2_make(c.z, c.w);
+        }
+    }
+};
+
+// Running sums of one query: FP32 partials by pair half, and what they are flushed into. The smooth
+// distance keeps the partials in the frame exp(-alpha ref), ref the smallest distance so far, and what
+// they are flushed into in the frame of aref, the ref of the last flush (an FP64 product costs 20
+// cycles of the SM, so the frame of the FP64 sums moves once a flush and not with every new ref).
+// The winding sums leave out 1 / (4 pi), the smooth distance's gradient alpha.
+template <int KIND, bool FP64, bool GRAD>
+struct Sums {
+    using Acc = typename std::conditional<FP64, double, float>::type;
+    f2 nqx, nqy, nqz;  // minus the query, in both halves
+    f2 v, g[GRAD ? 3 : 1];
+    Acc av, ag[GRAD ? 3 : 1];
+    float ref, aref;
+
+    __device__ __forceinline__ void init(float3 q)
+    {
+        nqx = f2_dup(-q.x); nqy = f2_dup(-q.y); nqz = f2_dup(-q.z);
+        v = f2_dup(0.0f);
+        av = 0;
+        if constexpr (GRAD)
+            for (int c = 0; c < 3; ++c) { g[c] = f2_dup(0.0f); ag[c] = 0; }
+        ref = aref = 3.0e38f;
+    }
+    __device__ __forceinline__ void flush(float c2)
+    {
+        if constexpr (KIND == SBH_SMOOTHDIST) {
+            if (ref < aref) {
+                const Acc f = (Acc)ex2_ftz(c2 * (aref - ref));
+                av *= f;
+                if constexpr (GRAD)
+                    for (int c = 0; c < 3; ++c) ag[c] *= f;
+                aref = ref;
+            }
+        }
+        av += (Acc)(f2_lo(v) + f2_hi(v));
+        v = f2_dup(0.0f);
+        if constexpr (GRAD)
+            for (int c = 0; c < 3; ++c) { ag[c] += (Acc)(f2_lo(g[c]) + f2_hi(g[c])); g[c] = f2_dup(0.0f); }
+    }
+    // the frame moves down to distance d (rare: about ln n times a query)
+    __device__ __forceinline__ void lower(float d, float c2)
+    {
+        const float f = ex2_ftz(c2 * (ref - d));
+        const f2 f22 = f2_dup(f);
+        v = v * f22;
+        if constexpr (GRAD)
+            for (int c = 0; c < 3; ++c) g[c] = g[c] * f22;
+        ref = d;
+    }
+    // add a pair's terms (BOTH false: the second source is padding)
+    template <bool BOTH>
+    __device__ __forceinline__ void add(const Pair<KIND>& p, const KernelParams& kp, float c2)
+    {
+        const f2 dx = p.x + nqx, dy = p.y + nqy, dz = p.z + nqz;
+        if constexpr (KIND == SBH_COULOMB) {
+            const f2 e = f2_fma(dx, dx, f2_fma(dy, dy, f2_fma(dz, dz, f2_dup(kp.eps2))));
+            const f2 ir = f2_make(rsqrt_ftz(f2_lo(e)), rsqrt_ftz(f2_hi(e)));
+            if constexpr (GRAD) {
+                f2 t = p.s * ir, c = t * (ir * ir);
+                if (!BOTH) { t = f2_make(f2_lo(t), 0.0f); c = f2_make(f2_lo(c), 0.0f); }
+                v = v + t;
+                add_grad<BOTH>(c, dx, dy, dz);
+            } else if (BOTH) {
+                v = f2_fma(p.s, ir, v);
+            } else {
+                v = v + f2_make(f2_lo(p.s) * f2_lo(ir), 0.0f);
+            }
+        } else if constexpr (KIND == SBH_WINDING) {
+            // 4 pi times the term, ((p - q).N) / r^3; 0 where r^2 is below the smallest normal float. The
+            // root's argument is clamped there, so that its powers stay finite and the select can sit
+            // before the last FMA (a select of the product cost an addition, 8% of the FMA pipe's work)
+            const f2 r2 = f2_fma(dx, dx, f2_fma(dy, dy, dz * dz));
+            const f2 dn = f2_fma(dx, p.nx, f2_fma(dy, p.ny, dz * p.s));
+            const float r2l = f2_lo(r2), r2h = f2_hi(r2);
+            const f2 ir = f2_make(rsqrt_ftz(fmaxf(r2l, kMinNormal)), rsqrt_ftz(fmaxf(r2h, kMinNormal)));
+            const f2 ir2 = ir * ir, u = dn * ir;
+            const bool l = r2l >= kMinNormal, h = BOTH && r2h >= kMinNormal;
+            const f2 us = f2_make(l ? f2_lo(u) : 0.0f, h ? f2_hi(u) : 0.0f);
+            v = f2_fma(us, ir2, v);
+            if constexpr (GRAD) {  // 3 ((p - q).N) (p - q) / r^5 - N / r^3
+                f2 x = dx, y = dy, z = dz, mx = p.nx, my = p.ny, mz = p.s;
+                f2 c = (us * ir2) * (ir2 * f2_dup(3.0f));
+                f2 b = ir * ir2 * f2_dup(-1.0f);
+                if (!(l && h)) {  // coincident, NaN or padding: the half adds nothing (0 times NaN is not 0)
+                    const auto mask = [&](f2 a) { return f2_make(l ? f2_lo(a) : 0.0f, h ? f2_hi(a) : 0.0f); };
+                    x = mask(x); y = mask(y); z = mask(z); mx = mask(mx); my = mask(my); mz = mask(mz);
+                    c = mask(c); b = mask(b);
+                }
+                g[0] = f2_fma(c, x, f2_fma(b, mx, g[0]));
+                g[1] = f2_fma(c, y, f2_fma(b, my, g[1]));
+                g[2] = f2_fma(c, z, f2_fma(b, mz, g[2]));
+            }
+        } else if constexpr (KIND == SBH_SMOOTHDIST) {
+            const f2 r2 = f2_fma(dx, dx, f2_fma(dy, dy, dz * dz));
+            const float r2l = f2_lo(r2), r2h = f2_hi(r2);
+            const f2 ir = f2_make(rsqrt_ftz(fmaxf(r2l, 1e-37f)), rsqrt_ftz(fmaxf(r2h, 1e-37f)));
+            const f2 d = r2 * ir;
+            const float dm = BOTH ? fminf(f2_lo(d), f2_hi(d)) : f2_lo(d);
+            if (dm < ref) lower(dm, c2);
+            const f2 x = (d + f2_dup(-ref)) * f2_dup(c2);
+            f2 t = p.s * f2_make(ex2_ftz(f2_lo(x)), ex2_ftz(f2_hi(x)));
+            if (!BOTH) t = f2_make(f2_lo(t), 0.0f);
+            v = v + t;
+            if constexpr (GRAD) {
+                const f2 c0 = t * ir;
+                add_grad<BOTH>(f2_make(r2l > 0.0f ? f2_lo(c0) : 0.0f, BOTH && r2h > 0.0f ? f2_hi(c0) : 0.0f), dx, dy,
+                               dz);
+            }
+        } else {
+            const f2 h = f2_fma(f2_dup(kp.g[0]), dx, f2_fma(f2_dup(kp.g[1]), dy, f2_dup(kp.g[2]) * dz));
+            f2 t = p.s * (f2_dup(1.0f) + h);
+            if (!BOTH) t = f2_make(f2_lo(t), 0.0f);
+            v = v + t;
+            if constexpr (GRAD) {
+                const f2 m = BOTH ? p.s : f2_make(f2_lo(p.s), 0.0f);
+                for (int c = 0; c < 3; ++c) g[c] = f2_fma(m, f2_dup(-kp.g[c]), g[c]);
+            }
+        }
+    }
+    template <bool BOTH>
+    __device__ __forceinline__ void add_grad(f2 c, f2 dx, f2 dy, f2 dz)
+    {
+        if constexpr (!BOTH) {  // the padding's difference is not used (0 times it could be NaN)
+            dx = f2_make(f2_lo(dx), 0.0f); dy = f2_make(f2_lo(dy), 0.0f); dz = f2_make(f2_lo(dz), 0.0f);
+        }
+        g[0] = f2_fma(c, dx, g[0]); g[1] = f2_fma(c, dy, g[1]); g[2] = f2_fma(c, dz, g[2]);
+    }
+};
+
+// what a warp, a block and then the cluster hand on about one query
+template <bool FP64, bool GRAD>
+struct Part {
+    typename std::conditional<FP64, double, float>::type v, g[GRAD ? 3 : 1];
+    float ref;
+};
+
+// sum of parts 0 .. count - 1 (get(k)), in that order; smooth distance: in the frame of the smallest
+template <int KIND, bool FP64, bool GRAD, class Get>
+__device__ __forceinline__ Part<FP64, GRAD> sum_parts(int count, float alpha, Get get)
+{
+    using P = Part<FP64, GRAD>;
+    P s = get(0);
+    if constexpr (KIND == SBH_SMOOTHDIST) {
+        for (int k = 1; k < count; ++k) s.ref = fminf(s.ref, get(k).ref);
+        s.v = 0;
+        if (GRAD) for (int c = 0; c < 3; ++c) s.g[c] = 0;
+    }
+    for (int k = KIND == SBH_SMOOTHDIST ? 0 : 1; k < count; ++k) {
+        const P p = get(k);
+        if constexpr (KIND == SBH_SMOOTHDIST) {
+            using A = decltype(s.v);
+            A f;
+            if constexpr (FP64) f = exp(-(double)alpha * ((double)p.ref - (double)s.ref));
+            else f = __expf(-alpha * (p.ref - s.ref));
+            s.v += p.v * f;
+            if (GRAD) for (int c = 0; c < 3; ++c) s.g[c] += p.g[c] * f;
+        } else {
+            s.v += p.v;
+            if (GRAD) for (int c = 0; c < 3; ++c) s.g[c] += p.g[c];
+        }
+    }
+    return s;
+}
+
+template <int KIND, bool FP64, bool GRAD, int QPT>
 __global__ void __launch_bounds__(kBruteThreads) k_brute(const float* __restrict__ P, const float* __restrict__ W,
                                                          const float* __restrict__ N, int64_t n,
                                                          const float* __restrict__ Q, int64_t nq, KernelParams kp,
-                                                         float* __restrict__ out)
+                                                         float* __restrict__ out, float* __restrict__ grad)
 {
-    __shared__ float4 spm[kBruteTile];
-    __shared__ float4 sdp[KIND == SBH_WINDING ? kBruteTile : 1];
-    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const bool active = j < nq;
-    const float3 q = active ? make_float3(Q[3 * j], Q[3 * j + 1], Q[3 * j + 2]) : make_float3(0.f, 0.f, 0.f);
-    double acc64 = 0.0;
-    float acc32 = 0.0f;
-    // smooth distance: sum = (acc64 + part) * exp(-alpha * ref), ref = smallest distance so far
-    float ref = 3.0e38f;
-    for (int64_t t0 = 0; t0 < n; t0 += kBruteTile) {
-        const int cnt = (n - t0) < kBruteTile ? (int)(n - t0) : kBruteTile;
-        __syncthreads();
-        if (threadIdx.x < cnt) {
-            const int64_t i = t0 + threadIdx.x;
-            spm[threadIdx.x] = make_float4(P[3 * i], P[3 * i + 1], P[3 * i + 2], W[i]);
-            if constexpr (KIND == SBH_WINDING) {
-                const float w = W[i];
-                sdp[threadIdx.x] = make_float4(w * N[3 * i], w * N[3 * i + 1], w * N[3 * i + 2], 0.0f);
-            }
-        }
-        __syncthreads();
-        float part = 0.0f;
-        if constexpr (KIND == SBH_SMOOTHDIST) {
-            for (int k = 0; k < cnt; ++k) {
-                const float4 p = spm[k];
-                const float d = dist_fast(p, q);
-                if (d < ref) {
-                    const float f = __expf(-kp.alpha * (ref - d));
-                    part *= f;
-                    if (FP64) acc64 *= (double)f; else acc32 *= f;
-                    ref = d;
-                }
-                part = fmaf(p.w, __expf(-kp.alpha * (d - ref)), part);
-            }
-        } else {
-#pragma unroll 8
-            for (int k = 0; k < cnt; ++k) {
-                const float4 p = spm[k];
-                if constexpr (KIND == SBH_COULOMB) part += term_coulomb(p, q, kp.eps2);
-                else if constexpr (KIND == SBH_WINDING) part += term_winding(p, sdp[k], q);
-                else part += term_affine(p, q, kp.g);
-            }
-        }
-        if (FP64) acc64 += (double)part; else acc32 += part;
-    }
-    if (!active) return;
-    const double total = FP64 ? acc64 : (double)acc32;
-    if constexpr (KIND == SBH_SMOOTHDIST)
-        out[j] = total > 0.0 ? (float)((double)ref - log(total) / (double)kp.alpha) : __int_as_float(0x7F800000);
-    else out[j] = (float)total;
-}
+    constexpr int kQuads = Pair<KIND>::kQuads;
+    constexpr int kGroup = 32 * QPT;
+    using PartT = Part<FP64, GRAD>;
+    constexpr size_t kTileBytes = (size_t)(kBruteTile / 2) * kQuads * sizeof(float4);
+    constexpr size_t kPartBytes = sizeof(PartT) * kGroup * kBruteWarps;
+    __shared__ __align__(16) unsigned char s_buf[kTileBytes > kPartBytes ? kTileBytes : kPartBytes];
+    __shared__ PartT s_block[kGroup];
+    float4* tile = reinterpret_cast<float4*>(s_buf);
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank(), ranks = (int)cluster.num_blocks();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t q0 = (int64_t)(blockIdx.x / ranks) * kGroup;
+    // this block's sources: whole tiles, as evenly as they go
+    const int64_t tiles = (n + kBruteTile - 1) / kBruteTile;
+    const int64_t t_lo = tiles * rank / ranks, t_hi = tiles * (rank + 1) / ranks;
 
-// The exact sum and its query gradient: per tile FP32 partials of the value and of the three
-// gradient components, added into FP64 accumulators (the smooth distance in the frame
-// exp(-alpha ref) of the smallest distance so far, as above). Outputs follow sbh_eval_grad:
-// the smooth distance returns d = ref - log(acc) / alpha and grad d = -grad acc / (alpha acc).
-template <int KIND>
-__global__ void __launch_bounds__(kBruteThreads) k_brute_grad(const float* __restrict__ P, const float* __restrict__ W,
-                                                              const float* __restrict__ N, int64_t n,
-                                                              const float* __restrict__ Q, int64_t nq, KernelParams kp,
-                                                              float* __restrict__ out, float* __restrict__ grad)
-{
-    __shared__ float4 spm[kBruteTile];
-    __shared__ float4 sdp[KIND == SBH_WINDING ? kBruteTile : 1];
-    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const bool active = j < nq;
-    const float3 q = active ? make_float3(Q[3 * j], Q[3 * j + 1], Q[3 * j + 2]) : make_float3(0.f, 0.f, 0.f);
-    double a64 = 0.0, g64[3] = {0.0, 0.0, 0.0};
-    float ref = 3.0e38f;
-    for (int64_t t0 = 0; t0 < n; t0 += kBruteTile) {
-        const int cnt = (n - t0) < kBruteTile ? (int)(n - t0) : kBruteTile;
+    Sums<KIND, FP64, GRAD> S[QPT];
+#pragma unroll
+    for (int k = 0; k < QPT; ++k) {
+        const int64_t j = q0 + 32 * k + lane;
+        S[k].init(j < nq ? make_float3(Q[3 * j], Q[3 * j + 1], Q[3 * j + 2]) : make_float3(0.f, 0.f, 0.f));
+    }
+    const float c2 = -kp.alpha * 1.44269504088896341f;  // exp(-alpha x) = 2^(c2 x)
+    for (int64_t t = t_lo; t < t_hi; ++t) {
+        const int64_t base = t * kBruteTile;
+        const int cnt = (n - base) < kBruteTile ? (int)(n - base) : kBruteTile;
         __syncthreads();
-        if (threadIdx.x < cnt) {
-            const int64_t i = t0 + threadIdx.x;
-            spm[threadIdx.x] = make_float4(P[3 * i], P[3 * i + 1], P[3 * i + 2], W[i]);
+        for (int k = threadIdx.x; k < (cnt + 1) / 2; k += kBruteThreads) {
+            const int64_t i = base + 2 * k, i1 = i + 1 < n ? i + 1 : i;
+            float4* d = tile + kQuads * k;
+            const float w0 = W[i], w1 = W[i1];
+            d[0] = make_float4(P[3 * i], P[3 * i1], P[3 * i + 1], P[3 * i1 + 1]);
             if constexpr (KIND == SBH_WINDING) {
-                const float w = W[i];
-                sdp[threadIdx.x] = make_float4(w * N[3 * i], w * N[3 * i + 1], w * N[3 * i + 2], 0.0f);
-            }
-        }
-        __syncthreads();
-        float v = 0.0f, g[3] = {0.0f, 0.0f, 0.0f};
-        for (int k = 0; k < cnt; ++k) {
-            const float4 pm = spm[k];
-            const float dx = pm.x - q.x, dy = pm.y - q.y, dz = pm.z - q.z;
-            if constexpr (KIND == SBH_COULOMB) {
-                const float e = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, kp.eps2)));
-                const float ir = rsqrt_ftz(e);
-                const float t = pm.w * ir;
-                const float c = t * ir * ir;
-                v += t;
-                g[0] = fmaf(c, dx, g[0]); g[1] = fmaf(c, dy, g[1]); g[2] = fmaf(c, dz, g[2]);
-            } else if constexpr (KIND == SBH_WINDING) {
-                const float4 D = sdp[k];
-                const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                if (r2 >= kMinNormal) {
-                    const float ir = rsqrt_ftz(r2);
-                    const float ir3 = ir * ir * ir;
-                    const float dn = fmaf(dx, D.x, fmaf(dy, D.y, dz * D.z));
-                    v = fmaf(kInv4Pi * dn, ir3, v);
-                    const float c = 3.0f * kInv4Pi * dn * ir3 * ir * ir;
-                    const float b = -kInv4Pi * ir3;
-                    g[0] += fmaf(b, D.x, c * dx); g[1] += fmaf(b, D.y, c * dy); g[2] += fmaf(b, D.z, c * dz);
-                }
-            } else if constexpr (KIND == SBH_SMOOTHDIST) {
-                const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                const float ir = rsqrt_ftz(fmaxf(r2, 1e-37f));
-                const float r = r2 * ir;
-                if (r < ref) {
-                    const float f = __expf(-kp.alpha * (ref - r));
-                    const double f64 = (double)f;
-                    v *= f; g[0] *= f; g[1] *= f; g[2] *= f;
-                    a64 *= f64; g64[0] *= f64; g64[1] *= f64; g64[2] *= f64;
-                    ref = r;
-                }
-                const float t = pm.w * __expf(-kp.alpha * (r - ref));
-                v += t;
-                if (r2 > 0.0f) {
-                    const float c = kp.alpha * t * ir;
-                    g[0] = fmaf(c, dx, g[0]); g[1] = fmaf(c, dy, g[1]); g[2] = fmaf(c, dz, g[2]);
-                }
+                d[1] = make_float4(P[3 * i + 2], P[3 * i1 + 2], w0 * N[3 * i + 2], w1 * N[3 * i1 + 2]);
+                d[2] = make_float4(w0 * N[3 * i], w1 * N[3 * i1], w0 * N[3 * i + 1], w1 * N[3 * i1 + 1]);
             } else {
-                v = fmaf(pm.w, 1.0f + fmaf(kp.g[0], dx, fmaf(kp.g[1], dy, kp.g[2] * dz)), v);
-                g[0] -= pm.w * kp.g[0]; g[1] -= pm.w * kp.g[1]; g[2] -= pm.w * kp.g[2];
+                d[1] = make_float4(P[3 * i + 2], P[3 * i1 + 2], w0, w1);
             }
         }
-        a64 += (double)v;
-        g64[0] += (double)g[0]; g64[1] += (double)g[1]; g64[2] += (double)g[2];
+        __syncthreads();
+        // the warp's eighth of the tile, in whole pairs; only the last pair of all may hold padding
+        const int per = cnt == kBruteTile ? kWarpTile / 2 : ((cnt + 1) / 2 + kBruteWarps - 1) / kBruteWarps;
+        const int lo = warp * per, full = cnt / 2;
+        const int hi = lo + per < full ? lo + per : full;
+        // measured per kernel: 20.3 / 18.9 cycles a winding term at 2 / 4, 21.7 / 21.0 / 23.7 a smooth-distance
+        // one at 2 / 1 / 4, its gradient 2.51 / 2.58 ms (5,001 queries, 2^19 sources) at 2 / 1
+        constexpr int kUnroll = GRAD ? 2 : (KIND == SBH_SMOOTHDIST ? 1 : 4);
+#pragma unroll kUnroll
+        for (int k = lo; k < hi; ++k) {
+            Pair<KIND> p;
+            p.load(tile + kQuads * k);
+#pragma unroll
+            for (int u = 0; u < QPT; ++u) S[u].template add<true>(p, kp, c2);
+        }
+        if ((cnt & 1) && full >= lo && full < lo + per) {
+            Pair<KIND> p;
+            p.load(tile + kQuads * full);
+#pragma unroll
+            for (int u = 0; u < QPT; ++u) S[u].template add<false>(p, kp, c2);
+        }
+        if (((t - t_lo) % kFlushTiles) == kFlushTiles - 1) {
+#pragma unroll
+            for (int u = 0; u < QPT; ++u) S[u].flush(c2);
+        }
     }
-    if (!active) return;
-    if constexpr (KIND == SBH_SMOOTHDIST) {
-        const bool pos = a64 > 0.0;
-        out[j] = pos ? (float)((double)ref - log(a64) / (double)kp.alpha) : __int_as_float(0x7F800000);
-        const double c = pos ? -1.0 / ((double)kp.alpha * a64) : 0.0;
-        for (int a = 0; a < 3; ++a) grad[3 * j + a] = pos ? (float)(c * g64[a]) : __int_as_float(0x7FC00000);
-    } else {
-        out[j] = (float)a64;
-        for (int a = 0; a < 3; ++a) grad[3 * j + a] = (float)g64[a];
+    __syncthreads();  // the tile's memory becomes the warps' parts
+    PartT* parts = reinterpret_cast<PartT*>(s_buf);
+#pragma unroll
+    for (int u = 0; u < QPT; ++u) {
+        S[u].flush(c2);
+        PartT p;
+        p.v = S[u].av;
+        if (GRAD) for (int c = 0; c < 3; ++c) p.g[c] = S[u].ag[c];
+        p.ref = S[u].ref;
+        parts[warp * kGroup + 32 * u + lane] = p;
     }
+    __syncthreads();
+    if (threadIdx.x < kGroup)
+        s_block[threadIdx.x] = sum_parts<KIND, FP64, GRAD>(kBruteWarps, kp.alpha,
+                                                           [&](int k) { return parts[k * kGroup + threadIdx.x]; });
+    cluster.sync();
+    const int64_t j = q0 + threadIdx.x;
+    if (rank == 0 && threadIdx.x < kGroup && j < nq) {
+        const PartT s = sum_parts<KIND, FP64, GRAD>(
+            ranks, kp.alpha, [&](int k) { return *cluster.map_shared_rank(&s_block[threadIdx.x], k); });
+        const double v = (double)s.v;
+        if constexpr (KIND == SBH_SMOOTHDIST) {
+            const bool pos = v > 0.0;
+            out[j] = pos ? (float)((double)s.ref - log(v) / (double)kp.alpha) : __int_as_float(0x7F800000);
+            if constexpr (GRAD)  // d = ref - log(acc) / alpha: grad d = -grad acc / (alpha acc); alpha cancels
+                for (int c = 0; c < 3; ++c)
+                    grad[3 * j + c] = pos ? (float)(-(double)s.g[c] / v) : __int_as_float(0x7FC00000);
+        } else {
+            const double f = KIND == SBH_WINDING ? 0.07957747154594766788 : 1.0;  // 1 / (4 pi)
+            out[j] = (float)(v * f);
+            if constexpr (GRAD)
+                for (int c = 0; c < 3; ++c) grad[3 * j + c] = (float)((double)s.g[c] * f);
+        }
+    }
+    cluster.sync();  // no block leaves while its sums are being read
 }
 
-template <int KIND>
-static void launch_brute_kind(const float* P, const float* W, const float* N, int64_t n, const float* Q, int64_t nq,
-                              const KernelParams& kp, int fp64, float* out, cudaStream_t s)
+template <int KIND, bool FP64, bool GRAD, int QPT>
+cudaError_t launch_group(const float* P, const float* W, const float* N, int64_t n, const float* Q, int64_t nq,
+                         const KernelParams& kp, float* out, float* grad, cudaStream_t s)
 {
-    const unsigned blocks = (unsigned)((nq + kBruteThreads - 1) / kBruteThreads);
-    if (fp64) k_brute<KIND, true><<<blocks, kBruteThreads, 0, s>>>(P, W, N, n, Q, nq, kp, out);
-    else k_brute<KIND, false><<<blocks, kBruteThreads, 0, s>>>(P, W, N, n, Q, nq, kp, out);
-    note_launch();
+    // as many blocks to a cluster as there are tiles for, at most eight
+    int ranks = kMaxCluster;
+    while (ranks > 1 && (int64_t)ranks * kBruteTile > n) ranks /= 2;
+    const int64_t groups = (nq + 32 * QPT - 1) / (32 * QPT);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(groups * ranks));
+    cfg.blockDim = dim3(kBruteThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)ranks;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_brute<KIND, FP64, GRAD, QPT>, P, W, N, n, Q, nq, kp, out, grad);
+    if (e == cudaSuccess) note_launch();
+    return e;
 }
+
+// Queries to a lane: four (the shared-memory reads of a source then cost a quarter each) where that
+// still leaves several blocks to every SM, else two; the gradient's sums have registers for two
+template <int KIND, bool FP64, bool GRAD>
+cudaError_t launch_kind(const float* P, const float* W, const float* N, int64_t n, const float* Q, int64_t nq,
+                        const KernelParams& kp, float* out, float* grad, cudaStream_t s)
+{
+    if constexpr (!GRAD) {
+        if (nq >= (int64_t)128 * device_sm_count())
+            return launch_group<KIND, FP64, GRAD, 4>(P, W, N, n, Q, nq, kp, out, grad, s);
+    }
+    return launch_group<KIND, FP64, GRAD, 2>(P, W, N, n, Q, nq, kp, out, grad, s);
+}
+
+template <bool FP64, bool GRAD>
+cudaError_t launch_any(const float* P, const float* W, const float* N, int64_t n, const float* Q, int64_t nq,
+                       const KernelParams& kp, float* out, float* grad, cudaStream_t s)
+{
+    if (nq <= 0) return cudaSuccess;
+    cudaError_t e;
+    switch (kp.kind) {
+    case SBH_COULOMB: e = launch_kind<SBH_COULOMB, FP64, GRAD>(P, W, N, n, Q, nq, kp, out, grad, s); break;
+    case SBH_WINDING: e = launch_kind<SBH_WINDING, FP64, GRAD>(P, W, N, n, Q, nq, kp, out, grad, s); break;
+    case SBH_SMOOTHDIST: e = launch_kind<SBH_SMOOTHDIST, FP64, GRAD>(P, W, N, n, Q, nq, kp, out, grad, s); break;
+    case SBH_AFFINE: e = launch_kind<SBH_AFFINE, FP64, GRAD>(P, W, N, n, Q, nq, kp, out, grad, s); break;
+    default: return cudaErrorInvalidValue;
+    }
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+}  // namespace
 
 cudaError_t launch_brute(const float* P, const float* W, const float* N, int64_t n, const float* Q, int64_t nq,
                          const KernelParams& kp, int fp64_accum, float* out, cudaStream_t s)
 {
-    if (nq <= 0) return cudaSuccess;
-    switch (kp.kind) {
-    case SBH_COULOMB: launch_brute_kind<SBH_COULOMB>(P, W, N, n, Q, nq, kp, fp64_accum, out, s); break;
-    case SBH_WINDING: launch_brute_kind<SBH_WINDING>(P, W, N, n, Q, nq, kp, fp64_accum, out, s); break;
-    case SBH_SMOOTHDIST: launch_brute_kind<SBH_SMOOTHDIST>(P, W, N, n, Q, nq, kp, fp64_accum, out, s); break;
-    case SBH_AFFINE: launch_brute_kind<SBH_AFFINE>(P, W, N, n, Q, nq, kp, fp64_accum, out, s); break;
-    default: return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
+    return fp64_accum ? launch_any<true, false>(P, W, N, n, Q, nq, kp, out, nullptr, s)
+                      : launch_any<false, false>(P, W, N, n, Q, nq, kp, out, nullptr, s);
 }
 
 cudaError_t launch_brute_grad(const float* P, const float* W, const float* N, int64_t n, const float* Q, int64_t nq,
                               const KernelParams& kp, float* out, float* grad, cudaStream_t s)
 {
-    if (nq <= 0) return cudaSuccess;
-    const unsigned b = (unsigned)((nq + kBruteThreads - 1) / kBruteThreads);
-    switch (kp.kind) {
-    case SBH_COULOMB: k_brute_grad<SBH_COULOMB><<<b, kBruteThreads, 0, s>>>(P, W, N, n, Q, nq, kp, out, grad); break;
-    case SBH_WINDING: k_brute_grad<SBH_WINDING><<<b, kBruteThreads, 0, s>>>(P, W, N, n, Q, nq, kp, out, grad); break;
-    case SBH_SMOOTHDIST: k_brute_grad<SBH_SMOOTHDIST><<<b, kBruteThreads, 0, s>>>(P, W, N, n, Q, nq, kp, out, grad); break;
-    case SBH_AFFINE: k_brute_grad<SBH_AFFINE><<<b, kBruteThreads, 0, s>>>(P, W, N, n, Q, nq, kp, out, grad); break;
-    default: return cudaErrorInvalidValue;
-    }
-    note_launch();
-    return cudaGetLastError();
+    return launch_any<true, true>(P, W, N, n, Q, nq, kp, out, grad, s);
 }
 
 }  // namespace sbh
