@@ -152,15 +152,10 @@ sbh_status sbh_build(const float* points, const float* weights, const float* nor
         release(T, s);
         return cuda_fail(e, "sbh_build allocation");
     }
-    int bad_p = 0, bad_w = 0;
-    e = sbh::build_sorted(T, points, weights, normals, s, &bad_p, &bad_w);
+    e = sbh::build_sorted(T, points, weights, normals, s);
     if (e != cudaSuccess) {
         release(T, s);
         return cuda_fail(e, "sbh_build sort");
-    }
-    if (bad_p || bad_w) {
-        release(T, s);
-        return fail(SBH_EINVAL, "sbh_build: %d non-finite coordinates, %d weights not finite and > 0", bad_p, bad_w);
     }
     e = sbh::build_tree(T, T->t4, T->lcp4, sbh::kMaxLevel4, 2, false, s);
     if (e != cudaSuccess) {
@@ -173,8 +168,16 @@ sbh_status sbh_build(const float* points, const float* weights, const float* nor
         release(T, s);
         return cuda_fail(e, "sbh_build");
     }
-    if (T->host_ctrl4.error) {
+    const sbh::TreeCtrl& c = T->host_ctrl4;
+    if (c.bad_points || c.bad_weights) {
+        const int bad_p = c.bad_points, bad_w = c.bad_weights;
         release(T, s);
+        return fail(SBH_EINVAL, "sbh_build: %d non-finite coordinates, %d weights not finite and > 0", bad_p, bad_w);
+    }
+    if (c.error) {
+        const int32_t why = c.error;
+        release(T, s);
+        if (why == sbh::kErrorTimeout) return fail(SBH_ETIMEOUT, "sbh_build: a wait of the sort gave up");
         return fail(SBH_EUNSUPPORTED, "sbh_build: more than 2^24 - 1 points share one deepest-level cell");
     }
     *out = T;

@@ -4,7 +4,7 @@
 //   1. bounds + validation   per-axis min/max of the points (the root cube), counts of NaN/Inf
 //                            coordinates and of non-positive weights
 //   2. Morton codes          20-bit FP32 quantisation per axis, interleaved to 60 bits
-//   3. stable LSD radix sort (code, index), 8 passes of 8 bits, block-local split sort
+//   3. stable LSD radix sort (code, index), 8 passes of 8 bits, one kernel each
 //   4. gather                points, weights and normals into Morton order
 //   5. topology              generation by generation: a node whose points span several cells one
 //                            level down has those runs as children; a run that stays inside one
@@ -28,6 +28,7 @@ namespace sbh {
 
 namespace {
 constexpr int kThreads = 256;
+constexpr int kMortonThreads = 1024;
 // blocks for n items, at most 16 per SM of the current device (grid-stride loops do the rest)
 inline unsigned grid_for(int64_t n, int per_block = kThreads, unsigned cap = 0)
 {
@@ -146,89 +147,84 @@ __device__ __forceinline__ int ordered_int(float f)
 }
 __device__ __forceinline__ float from_ordered(int i) { return __int_as_float(i >= 0 ? i : (i ^ 0x7FFFFFFF)); }
 
-// scratch: [0..2] min (ordered int), [3..5] max, [6] bad coordinates, [7] bad weights
-__global__ void k_bounds_init(int* scratch)
+// The float order as unsigned integers, so that a maximum taken by atomicMax can start from zero
+__device__ __forceinline__ uint32_t ordered_uint(float f) { return (uint32_t)ordered_int(f) ^ 0x80000000u; }
+__device__ __forceinline__ float from_ordered_uint(uint32_t u) { return from_ordered((int)(u ^ 0x80000000u)); }
+
+// Whether the calling block is the last of the grid to come here (every thread gets the answer):
+// what the other blocks wrote before is then visible to it. *done starts at zero.
+__device__ __forceinline__ bool last_block(unsigned* done)
 {
-    if (threadIdx.x < 3) { scratch[threadIdx.x] = INT32_MAX; scratch[3 + threadIdx.x] = INT32_MIN; }
-    if (threadIdx.x == 6 || threadIdx.x == 7) scratch[threadIdx.x] = 0;
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (last) __threadfence();
+    return last;
 }
 
-__global__ void k_bounds(const float* __restrict__ pts, const float* __restrict__ w, int64_t n,
-                         int* __restrict__ scratch)
+// Per-axis extremes and the counts of bad inputs, then (the last block) the root cube: lo = per-axis
+// min, side = largest extent (1 if every point coincides), and the cell diagonal table |B|(level) =
+// sqrt(3) * side * 2^-(shift * level) for each branching
+__global__ void __launch_bounds__(kThreads) k_bounds(const float* __restrict__ pts, const float* __restrict__ w,
+                                                     int64_t n, SortHead* __restrict__ H, TreeCtrl* c4, TreeCtrl* c2)
 {
-    int mn[3] = {INT32_MAX, INT32_MAX, INT32_MAX}, mx[3] = {INT32_MIN, INT32_MIN, INT32_MIN};
+    uint32_t mx[6] = {0, 0, 0, 0, 0, 0};  // of the negated order (the minima), of the order
     int bad_p = 0, bad_w = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             const float v = pts[3 * i + a];
             if (!isfinite(v)) { ++bad_p; continue; }
-            const int o = ordered_int(v);
-            mn[a] = min(mn[a], o);
-            mx[a] = max(mx[a], o);
+            const uint32_t o = ordered_uint(v);
+            mx[a] = max(mx[a], ~o);
+            mx[3 + a] = max(mx[3 + a], o);
         }
         const float m = w[i];
         if (!(m > 0.0f) || !isfinite(m)) ++bad_w;
     }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            mn[a] = min(mn[a], __shfl_xor_sync(0xFFFFFFFFu, mn[a], off));
-            mx[a] = max(mx[a], __shfl_xor_sync(0xFFFFFFFFu, mx[a], off));
-        }
-        bad_p += __shfl_xor_sync(0xFFFFFFFFu, bad_p, off);
-        bad_w += __shfl_xor_sync(0xFFFFFFFFu, bad_w, off);
-    }
-    // then across the block's warps, so that each block adds one set of atomics (not one per warp)
-    __shared__ int s_red[kThreads / 32][8];
+    // across the warp, then across the block's warps, so that each block adds one set of atomics
+    __shared__ uint32_t s_red[kThreads / 32][8];
     const int warp = threadIdx.x >> 5;
-    if ((threadIdx.x & 31) == 0) {
+    uint32_t r[8];
 #pragma unroll
-        for (int a = 0; a < 3; ++a) { s_red[warp][a] = mn[a]; s_red[warp][3 + a] = mx[a]; }
-        s_red[warp][6] = bad_p;
-        s_red[warp][7] = bad_w;
+    for (int a = 0; a < 6; ++a) r[a] = __reduce_max_sync(0xFFFFFFFFu, mx[a]);
+    r[6] = __reduce_add_sync(0xFFFFFFFFu, (unsigned)bad_p);
+    r[7] = __reduce_add_sync(0xFFFFFFFFu, (unsigned)bad_w);
+    if ((threadIdx.x & 31) < 8) {
+#pragma unroll
+        for (int a = 0; a < 8; ++a)
+            if ((int)(threadIdx.x & 31) == a) s_red[warp][a] = r[a];
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int k = 1; k < (int)(blockDim.x >> 5); ++k) {
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                mn[a] = min(mn[a], s_red[k][a]);
-                mx[a] = max(mx[a], s_red[k][3 + a]);
-            }
-            bad_p += s_red[k][6];
-            bad_w += s_red[k][7];
-        }
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            atomicMin(&scratch[a], mn[a]);
-            atomicMax(&scratch[3 + a], mx[a]);
-        }
-        if (bad_p) atomicAdd(&scratch[6], bad_p);
-        if (bad_w) atomicAdd(&scratch[7], bad_w);
+    if (threadIdx.x < 8) {
+        uint32_t t = s_red[0][threadIdx.x];
+        for (int k = 1; k < (int)(blockDim.x >> 5); ++k)
+            t = threadIdx.x < 6 ? max(t, s_red[k][threadIdx.x]) : t + s_red[k][threadIdx.x];
+        if (threadIdx.x < 6) atomicMax(&H->bounds[threadIdx.x], t);
+        else if (t) atomicAdd(&H->bounds[threadIdx.x], t);
     }
-}
-
-// root cube: lo = per-axis min, side = largest extent (1 if every point coincides); the cell
-// diagonal table |B|(level) = sqrt(3) * side * 2^-(shift * level) for each branching
-__global__ void k_root_cube(const int* __restrict__ scratch, TreeCtrl* c4, TreeCtrl* c2)
-{
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+    if (!last_block(&H->done[0])) return;
     float lo[3], side = 0.0f;
     for (int a = 0; a < 3; ++a) {
-        lo[a] = from_ordered(scratch[a]);
-        const float ext = __fsub_rn(from_ordered(scratch[3 + a]), lo[a]);
+        lo[a] = from_ordered_uint(~__ldcg(&H->bounds[a]));
+        const float ext = __fsub_rn(from_ordered_uint(__ldcg(&H->bounds[3 + a])), lo[a]);
         side = ext > side ? ext : side;
     }
     if (side == 0.0f) side = 1.0f;
     const float diam0 = __fmul_rn(1.7320508075688772f, side);
-    for (int a = 0; a < 3; ++a) { c4->lo[a] = lo[a]; c2->lo[a] = lo[a]; }
-    c4->side = side;
-    c2->side = side;
-    for (int l = 0; l < kDiamLevels; ++l) {
-        c4->diam[l] = ldexpf(diam0, -2 * l);
-        c2->diam[l] = ldexpf(diam0, -l);
+    if (threadIdx.x < kDiamLevels) {
+        c4->diam[threadIdx.x] = ldexpf(diam0, -2 * (int)threadIdx.x);
+        c2->diam[threadIdx.x] = ldexpf(diam0, -(int)threadIdx.x);
+    }
+    if (threadIdx.x == 0) {
+        for (int a = 0; a < 3; ++a) { c4->lo[a] = lo[a]; c2->lo[a] = lo[a]; }
+        c4->side = side;
+        c2->side = side;
+        c4->error = c2->error = 0;
+        c4->bad_points = (int32_t)__ldcg(&H->bounds[6]);
+        c4->bad_weights = (int32_t)__ldcg(&H->bounds[7]);
     }
 }
 
@@ -255,18 +251,58 @@ __device__ __forceinline__ uint32_t quantise(float x, float lo, float scale)
     return c > 1048575u ? 1048575u : c;
 }
 
-__global__ void k_morton(const float* __restrict__ pts, int64_t n, const TreeCtrl* __restrict__ c4,
-                         uint64_t* __restrict__ code, int32_t* __restrict__ idx)
+// The codes, and the histogram of each of their eight digits: counted per block in shared memory, added
+// up, and made exclusive sums (where each digit's run starts in its pass) by the last block. Lanes
+// that share a digit add once together in the top one, which has 16 values.
+__global__ void __launch_bounds__(kMortonThreads) k_morton(const float* __restrict__ pts, int64_t n,
+                                                           const TreeCtrl* __restrict__ c4, uint64_t* __restrict__ code,
+                                                           SortHead* __restrict__ H)
 {
+    __shared__ int s_hist[kPasses][256];
+    for (int k = threadIdx.x; k < kPasses * 256; k += blockDim.x) (&s_hist[0][0])[k] = 0;
+    __syncthreads();
     const float lx = c4->lo[0], ly = c4->lo[1], lz = c4->lo[2];
     const float scale = __fdiv_rn(1048576.0f, c4->side);
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    for (int64_t b = blockIdx.x * (int64_t)blockDim.x; b < n; b += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t i = b + threadIdx.x;
+        const unsigned live = __ballot_sync(0xFFFFFFFFu, i < n);
+        if (i >= n) continue;
         const uint32_t cx = quantise(pts[3 * i], lx, scale);
         const uint32_t cy = quantise(pts[3 * i + 1], ly, scale);
         const uint32_t cz = quantise(pts[3 * i + 2], lz, scale);
-        code[i] = (spread3(cx) << 2) | (spread3(cy) << 1) | spread3(cz);
-        idx[i] = (int32_t)i;
+        const uint64_t c = (spread3(cx) << 2) | (spread3(cy) << 1) | spread3(cz);
+        code[i] = c;
+#pragma unroll
+        for (int p = 0; p < kPasses; ++p) {
+            const int d = (int)(c >> (8 * p)) & 0xFF;
+            if (p < kPasses - 1) {
+                atomicAdd(&s_hist[p][d], 1);
+            } else {
+                const unsigned peers = __match_any_sync(live, d);
+                if ((threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&s_hist[p][d], __popc(peers));
+            }
+        }
     }
+    __syncthreads();
+    for (int k = threadIdx.x; k < kPasses * 256; k += blockDim.x) {
+        const int v = (&s_hist[0][0])[k];
+        if (v) atomicAdd(&H->hist[0][0] + k, v);
+    }
+    if (!last_block(&H->done[1])) return;
+    const int p = threadIdx.x >> 5, lane = threadIdx.x & 31;  // a warp to a digit, eight values to a lane
+    if (p >= kPasses) return;
+    int v[8], sum = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) { v[k] = __ldcg(&H->hist[p][8 * lane + k]); sum += v[k]; }
+    int x = sum;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int y = __shfl_up_sync(0xFFFFFFFFu, x, off);
+        if (lane >= off) x += y;
+    }
+    x -= sum;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) { H->hist[p][8 * lane + k] = x; x += v[k]; }
 }
 
 // ----------------------------------------------------------------------------------------------
@@ -370,87 +406,196 @@ void scan_exclusive(const int* in, int* out, int64_t n, int* temp, cudaStream_t 
 }
 
 // ----------------------------------------------------------------------------------------------
-// 3. stable LSD radix sort of (code, index) pairs, 8-bit digits
-//    hist: per-tile digit counts, stored digit-major so that one exclusive scan gives every
-//    (digit, tile) output offset. scatter: a stable local sort of the tile by the digit (nine
-//    one-bit splits of (digit, slot) words in shared memory; the ninth moves padding last),
-//    then each key goes to offset[digit][tile] + its rank among the tile's keys of that digit.
+// 3. stable LSD radix sort of (code, index) pairs, 8-bit digits, one kernel per pass: each tile
+//    ranks its keys by digit (warp by warp, lanes of equal digit found by a match, so the order is
+//    kept), learns from the tiles before it how many keys of each digit they hold, and writes its keys
+//    in runs. The tiles' counts pass along by decoupled look-back (Merrill and Garland, "Single-pass
+//    Parallel Prefix Scan with Decoupled Look-back", 2016; as a sort: Adinets and Merrill,
+//    "Onesweep", 2022): a status word per (tile, digit) says nothing yet, the tile's own count, or
+//    the count of it and all before it. A tile number is drawn when a block starts, so every tile
+//    waited for is already running; each wait is bounded all the same, and one that runs out sets
+//    H->error, which ends the build with SBH_ETIMEOUT.
+//    What bounds it: the latency of a tile's steps (load, rank, look back, write) with two blocks of
+//    512 threads to an SM; the 24 bytes a key moves take a quarter of the time. It replaces a count, a
+//    scan of up to three kernels and a scatter that sorted its tile by nine one-bit splits: 40 kernels
+//    and 650 us for 2^22 keys, now 8 and 307 us (2^20: 230 -> 106 us), and the histograms of all
+//    digits come with the codes.
 // ----------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint64_t* __restrict__ keys, int64_t n,
-                                                             int shift, int ntiles, int* __restrict__ hist)
+constexpr uint32_t kStatusOwn = 1u << 30, kStatusAll = 2u << 30, kStatusMask = (1u << 30) - 1;
+constexpr int kSpinLimit = 1 << 22;  // polls before a wait gives up (seconds)
+constexpr int kLook = 4;             // status words a digit's thread has in flight
+
+// The lanes of the warp whose 8-bit digit equals the caller's, by one ballot per bit: about 40 cycles
+// whatever the digits are. (A match instruction takes 9 cycles where few digits occur, but grows with
+// their number: a pass over 2^22 keys took 60 us with it where the digits are random.)
+__device__ __forceinline__ unsigned same_digit(int d)
 {
-    __shared__ int cnt[256];
-    cnt[threadIdx.x] = 0;
-    __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * kSortTile;
+    unsigned peers = 0xFFFFFFFFu;
 #pragma unroll
-    for (int k = 0; k < kSortItems; ++k) {
-        const int64_t i = base + (int64_t)k * kSortThreads + threadIdx.x;
-        if (i < n) atomicAdd(&cnt[(keys[i] >> shift) & 0xFF], 1);
+    for (int b = 0; b < 8; ++b) {
+        const bool on = (d >> b) & 1;
+        const unsigned m = __ballot_sync(0xFFFFFFFFu, on);
+        peers &= on ? m : ~m;
     }
-    __syncthreads();
-    hist[(int64_t)threadIdx.x * ntiles + blockIdx.x] = cnt[threadIdx.x];
+    return peers;
 }
 
-__global__ void __launch_bounds__(kSortThreads) k_radix_scatter(const uint64_t* __restrict__ kin,
-                                                                const int32_t* __restrict__ vin, int64_t n,
-                                                                int shift, int ntiles,
-                                                                const int* __restrict__ offsets,
-                                                                uint64_t* __restrict__ kout,
-                                                                int32_t* __restrict__ vout)
+template <int ITEMS>
+__global__ void __launch_bounds__(kSortThreads, 2) k_radix_pass(const uint64_t* __restrict__ kin,
+                                                             const int32_t* __restrict__ vin, int64_t n, int pass,
+                                                             SortHead* __restrict__ H, uint32_t* status,
+                                                             uint32_t* __restrict__ next_status,
+                                                             uint64_t* __restrict__ kout, int32_t* __restrict__ vout)
 {
-    __shared__ uint64_t skey[kSortTile];
-    __shared__ int32_t sval[kSortTile];
-    __shared__ uint32_t ord[2][kSortTile];  // digit << 16 | slot
-    __shared__ int dstart[257];
-    __shared__ int ws[32];
-    const int64_t base = (int64_t)blockIdx.x * kSortTile;
-    const int count = (n - base) < kSortTile ? (int)(n - base) : kSortTile;
-    for (int i = threadIdx.x; i < kSortTile; i += kSortThreads) {
-        if (i < count) {
-            const uint64_t k = kin[base + i];
-            skey[i] = k;
-            sval[i] = vin[base + i];
-            ord[0][i] = ((uint32_t)((k >> shift) & 0xFF) << 16) | (uint32_t)i;
-        } else {
-            ord[0][i] = (256u << 16) | (uint32_t)i;  // padding sorts last
-        }
+    constexpr int kTile = kSortThreads * ITEMS, kWarps = kSortThreads / 32;
+    extern __shared__ __align__(16) unsigned char s_sort[];
+    uint64_t* s_key = reinterpret_cast<uint64_t*>(s_sort);
+    int32_t* s_val = reinterpret_cast<int32_t*>(s_key + kTile);
+    uint16_t(*s_cnt)[256] = reinterpret_cast<uint16_t(*)[256]>(s_val + kTile);  // per warp and digit
+    __shared__ int s_start[256];   // first place of a digit in the sorted tile
+    __shared__ int s_out[256];     // where that place goes, minus it
+    __shared__ int s_warp[kWarps];
+    __shared__ int s_tile;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    if (t == 0) s_tile = (int)atomicAdd(&H->next_tile[pass], 1u);
+    for (int k = t; k < kWarps * 128; k += kSortThreads) reinterpret_cast<uint32_t*>(s_cnt)[k] = 0u;
+    __syncthreads();
+    const int tile = s_tile;
+    const int64_t base = (int64_t)tile * kTile;
+    const int count = (n - base) < kTile ? (int)(n - base) : kTile;
+    const int shift = 8 * pass;
+    // a warp takes consecutive keys; what lies past the end ranks behind every key (digit 255, last)
+    uint64_t key[ITEMS];
+    const int w0 = warp * 32 * ITEMS + lane;
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k) key[k] = w0 + 32 * k < count ? kin[base + w0 + 32 * k] : ~0ull;
+    if (t < 256) next_status[(int64_t)tile * 256 + t] = 0u;  // the next pass's words (read last in the pass before)
+    // a key's rank among the warp's keys of its digit; keys of equal digit in a row of 32 find each other
+    uint32_t rank[ITEMS / 2];  // two 16-bit ranks to a word
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k) {
+        const int d = (int)(key[k] >> shift) & 0xFF;
+        const unsigned peers = same_digit(d);
+        const uint32_t r = s_cnt[warp][d] + __popc(peers & ((1u << lane) - 1u));
+        __syncwarp();
+        if (lane == 31 - __clz(peers)) s_cnt[warp][d] = (uint16_t)(r + 1u);
+        __syncwarp();
+        if (k & 1) rank[k / 2] |= r << 16;
+        else rank[k / 2] = r;
     }
     __syncthreads();
-    int cur = 0;
-    for (int bit = 16; bit < 25; ++bit) {
-        uint32_t e[kSortItems];
-        int zeros = 0;
+    // thread t < 256: digit t
+    volatile uint32_t* st = status;
+    int own = 0, real = 0;
+    if (t < 256) {
 #pragma unroll
-        for (int k = 0; k < kSortItems; ++k) {
-            e[k] = ord[cur][threadIdx.x * kSortItems + k];
-            zeros += ((e[k] >> bit) & 1u) ? 0 : 1;
-        }
-        int total_zeros;
-        int zb = block_exclusive_scan(zeros, ws, &total_zeros);
-        int pos = threadIdx.x * kSortItems;
-#pragma unroll
-        for (int k = 0; k < kSortItems; ++k, ++pos) {
-            const bool one = (e[k] >> bit) & 1u;
-            const int dst = one ? total_zeros + (pos - zb) : zb;
-            if (!one) ++zb;
-            ord[cur ^ 1][dst] = e[k];
-        }
-        cur ^= 1;
-        __syncthreads();
+        for (int k = 0; k < kWarps; ++k) { const int c = s_cnt[k][t]; s_cnt[k][t] = (uint16_t)own; own += c; }
+        real = t == 255 ? own - (kTile - count) : own;
+        st[(int64_t)tile * 256 + t] = (tile == 0 ? kStatusAll : kStatusOwn) | (uint32_t)real;
     }
-    for (int i = threadIdx.x; i < count; i += kSortThreads) {
-        const uint32_t d = ord[cur][i] >> 16;
-        if (i == 0 || (ord[cur][i - 1] >> 16) != d) dstart[d] = i;
+    int x = own;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int y = __shfl_up_sync(0xFFFFFFFFu, x, off);
+        if (lane >= off) x += y;
+    }
+    if (lane == 31) s_warp[warp] = x;
+    __syncthreads();
+    if (t < 256) {
+        int add = x - own;
+#pragma unroll
+        for (int k = 0; k < 7; ++k) add += k < warp ? s_warp[k] : 0;
+        s_start[t] = add;
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < count; i += kSortThreads) {
-        const uint32_t e = ord[cur][i];
-        const uint32_t d = e >> 16, slot = e & 0xFFFFu;
-        const int64_t dst = (int64_t)offsets[(int64_t)d * ntiles + blockIdx.x] + (i - dstart[d]);
-        kout[dst] = skey[slot];
-        vout[dst] = sval[slot];
+    // into digit order in shared memory, while the first status words come in
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k) {
+        const int i = w0 + 32 * k;
+        const int d = (int)(key[k] >> shift) & 0xFF;
+        const int at = s_start[d] + s_cnt[warp][d] + (int)((rank[k / 2] >> (16 * (k & 1))) & 0xFFFFu);
+        s_key[at] = key[k];
+        s_val[at] = i < count ? (vin ? vin[base + i] : (int32_t)(base + i)) : 0;
     }
+    // look back, kLook tiles at a time
+    uint32_t before = 0;
+    if (tile > 0 && t < 256) {
+        int spin = 0;
+        for (int p = tile - 1; p >= 0;) {
+            uint32_t v[kLook];
+#pragma unroll
+            for (int k = 0; k < kLook; ++k) v[k] = p - k >= 0 ? st[(int64_t)(p - k) * 256 + t] : (uint32_t)kStatusAll;
+            bool wait = false;
+#pragma unroll
+            for (int k = 0; k < kLook; ++k) {
+                if (p < 0 || wait) continue;
+                if (v[k] == 0u) { wait = true; continue; }
+                before += v[k] & kStatusMask;
+                p = (v[k] & kStatusAll) ? -1 : p;
+            }
+            if (p >= 0) {
+                // how many of the words were there: step over them
+                int got = 0;
+#pragma unroll
+                for (int k = 0; k < kLook; ++k) got += (got == k && v[k] != 0u) ? 1 : 0;
+                p -= got;
+                if (got == 0 && ++spin > kSpinLimit) { H->error = 1; break; }
+            }
+        }
+        st[(int64_t)tile * 256 + t] = kStatusAll | ((before + (uint32_t)real) & kStatusMask);
+    }
+    if (t < 256) s_out[t] = H->hist[pass][t] + (int)before - s_start[t];
+    __syncthreads();
+    for (int i = t; i < count; i += kSortThreads) {
+        const uint64_t k = s_key[i];
+        const uint32_t dst = (uint32_t)(s_out[(int)(k >> shift) & 0xFF] + i);
+        if (dst < (uint32_t)n) {  // always, unless a wait gave up
+            kout[dst] = k;
+            vout[dst] = s_val[i];
+        }
+    }
+}
+
+int64_t sort_tiles(int64_t n) { return (n + kSortTile - 1) / kSortTile; }
+
+size_t sort_status_bytes(int64_t n) { return (size_t)sort_tiles(n) * 256 * sizeof(uint32_t); }
+
+__global__ void k_sort_error(const SortHead* __restrict__ H, TreeCtrl* ctrl)
+{
+    if (threadIdx.x == 0 && blockIdx.x == 0 && H->error) ctrl->error = kErrorTimeout;
+}
+
+template <int ITEMS>
+static cudaError_t radix_passes(uint64_t* const k[2], int32_t* const v[2], int64_t n, SortHead* H, uint32_t* status,
+                                cudaStream_t s)
+{
+    constexpr int kTile = kSortThreads * ITEMS;
+    constexpr size_t kBytes = (size_t)kTile * (sizeof(uint64_t) + sizeof(int32_t)) + (kSortThreads / 32) * 256 * sizeof(uint16_t);
+    const cudaError_t e = cudaFuncSetAttribute(k_radix_pass<ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBytes);
+    if (e != cudaSuccess) return e;
+    const unsigned tiles = (unsigned)((n + kTile - 1) / kTile);
+    const size_t words = (size_t)sort_tiles(n) * 256;
+    for (int pass = 0; pass < kPasses; ++pass) {
+        const int a = pass & 1;
+        k_radix_pass<ITEMS><<<tiles, kSortThreads, kBytes, s>>>(k[a], pass ? v[a] : nullptr, n, pass, H,
+                                                                status + a * words, status + (a ^ 1) * words, k[a ^ 1],
+                                                                v[a ^ 1]);
+        note_launch();
+    }
+    return cudaGetLastError();
+}
+
+cudaError_t sort_codes(const float* pts, const float* w, int64_t n, uint64_t* const k[2], int32_t* const v[2],
+                       SortHead* H, uint32_t* status, TreeCtrl* c4, TreeCtrl* c2, cudaStream_t s)
+{
+    cudaError_t e = cudaMemsetAsync(H, 0, sizeof(SortHead), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(status, 0, sort_status_bytes(n), s);  // the first pass's half
+    if (e != cudaSuccess) return e;
+    k_bounds<<<grid_for(n, kThreads, 4u * (unsigned)device_sm_count()), kThreads, 0, s>>>(pts, w, n, H, c4, c2);
+    note_launch();
+    k_morton<<<grid_for(n, kMortonThreads, 2u * (unsigned)device_sm_count()), kMortonThreads, 0, s>>>(pts, n, c4, k[0], H);
+    note_launch();
+    return radix_passes<kSortItems>(k, v, n, H, status, s);
 }
 
 // ----------------------------------------------------------------------------------------------
@@ -558,7 +703,6 @@ __global__ void k_topo_root(BuildArrays B, const int* __restrict__ root_min)
     for (int g = 0; g < kMaxDepth + 2; ++g) B.ctrl->depth_base[g] = 1;
     B.ctrl->depth_base[0] = 0;
     B.ctrl->max_depth = 0;
-    B.ctrl->error = 0;
 }
 
 __global__ void k_topo_seed(BuildArrays B)
@@ -632,7 +776,7 @@ __global__ void k_topo_classify(BuildArrays B, int gen)
         const uint32_t pm = B.meta[v];
         if (i + 1 == B.ne[v]) {  // parent's last point: its last child is c
             const uint32_t nc = (uint32_t)(c - B.fc[v] + 1);
-            if (nc > kMaxChildren) B.ctrl->error = 1;
+            if (nc > kMaxChildren) B.ctrl->error = kErrorChildren;
             B.meta[v] = meta_pack(nc, meta_level(pm), meta_kind(pm));
         }
         if (!B.flag[i]) continue;
@@ -849,55 +993,27 @@ void free_tree(DeviceTree& D, cudaStream_t s)
     D = DeviceTree();
 }
 
-cudaError_t build_sorted(sbh_tree* T, const float* pts, const float* w, const float* nrm, cudaStream_t s,
-                         int* bad_points, int* bad_weights)
+cudaError_t build_sorted(sbh_tree* T, const float* pts, const float* w, const float* nrm, cudaStream_t s)
 {
     const int64_t n = T->n;
     ScratchSet guard(s);
-    int* scratch = nullptr;
-    SBH_TRY(guard.alloc(&scratch, 8 * sizeof(int)));
-    k_bounds_init<<<1, 32, 0, s>>>(scratch);
-    note_launch();
-    k_bounds<<<grid_for(n), kThreads, 0, s>>>(pts, w, n, scratch);
-    note_launch();
-    int host[8];
-    SBH_TRY(cudaMemcpyAsync(host, scratch, sizeof(host), cudaMemcpyDeviceToHost, s));
-    SBH_TRY(cudaStreamSynchronize(s));
-    *bad_points = host[6];
-    *bad_weights = host[7];
-    if (host[6] || host[7]) return cudaSuccess;
-    k_root_cube<<<1, 32, 0, s>>>(scratch, T->t4.ctrl, T->t2.ctrl);
-    note_launch();
-    SBH_TRY(cudaGetLastError());
-
-    uint64_t *k0 = nullptr, *k1 = nullptr;
-    int32_t *v0 = nullptr, *v1 = nullptr;
-    const int ntiles = (int)((n + kSortTile - 1) / kSortTile);
-    const int64_t nhist = (int64_t)256 * ntiles;
-    int *hist = nullptr, *tmp = nullptr;
-    SBH_TRY(guard.alloc(&k0, n * sizeof(uint64_t)));
-    SBH_TRY(guard.alloc(&k1, n * sizeof(uint64_t)));
-    SBH_TRY(guard.alloc(&v0, n * sizeof(int32_t)));
-    SBH_TRY(guard.alloc(&v1, n * sizeof(int32_t)));
-    SBH_TRY(guard.alloc(&hist, nhist * sizeof(int)));
-    SBH_TRY(guard.alloc(&tmp, scan_temp_ints(nhist) * sizeof(int)));
-    k_morton<<<grid_for(n), kThreads, 0, s>>>(pts, n, T->t4.ctrl, k0, v0);
-    note_launch();
-    for (int pass = 0; pass < 8; ++pass) {
-        const int shift = 8 * pass;
-        k_radix_hist<<<ntiles, kSortThreads, 0, s>>>(k0, n, shift, ntiles, hist);
-        note_launch();
-        scan_exclusive(hist, hist, nhist, tmp, s);
-        k_radix_scatter<<<ntiles, kSortThreads, 0, s>>>(k0, v0, n, shift, ntiles, hist, k1, v1);
-        note_launch();
-        uint64_t* tk = k0; k0 = k1; k1 = tk;
-        int32_t* tv = v0; v0 = v1; v1 = tv;
+    uint64_t* k[2] = {nullptr, nullptr};
+    int32_t* v[2] = {nullptr, nullptr};
+    SortHead* head = nullptr;
+    uint32_t* status = nullptr;
+    SBH_TRY(guard.alloc(&head, sizeof(SortHead)));
+    SBH_TRY(guard.alloc(&status, 2 * sort_status_bytes(n)));
+    for (int a = 0; a < 2; ++a) {
+        SBH_TRY(guard.alloc(&k[a], n * sizeof(uint64_t)));
+        SBH_TRY(guard.alloc(&v[a], n * sizeof(int32_t)));
     }
-    SBH_TRY(cudaGetLastError());
-    T->code = k0;
-    T->perm = v0;
-    guard.keep(k0);
-    guard.keep(v0);
+    SBH_TRY(sort_codes(pts, w, n, k, v, head, status, T->t4.ctrl, T->t2.ctrl, s));
+    T->code = k[0];  // an even number of passes ends where it began
+    T->perm = v[0];
+    guard.keep(k[0]);
+    guard.keep(v[0]);
+    k_sort_error<<<1, 32, 0, s>>>(head, T->t4.ctrl);
+    note_launch();
 
     SBH_TRY(dalloc((void**)&T->spw, n * sizeof(float4), s));
     if (nrm) SBH_TRY(dalloc((void**)&T->snrm, n * sizeof(float4), s));

@@ -72,9 +72,9 @@ namespace sbh {
 // Enqueue the topology, aggregate and packing steps of one tree on `s`.
 cudaError_t build_tree(sbh_tree* T, DeviceTree& D, const uint8_t* lcp, int max_level, int level_shift,
                        bool with_skip, cudaStream_t s);
-// Enqueue validation (sets *bad on the host after a sync), root cube, codes, sort and gather.
-cudaError_t build_sorted(sbh_tree* T, const float* pts, const float* w, const float* nrm, cudaStream_t s,
-                         int* bad_points, int* bad_weights);
+// Enqueue validation (t4.ctrl gets the counts of bad inputs), root cube, codes, sort and gather. Bad
+// inputs do no harm to what follows: every coordinate quantises to a code.
+cudaError_t build_sorted(sbh_tree* T, const float* pts, const float* w, const float* nrm, cudaStream_t s);
 cudaError_t alloc_tree(DeviceTree& D, int64_t n, bool with_dip, bool with_skip, bool with_rec, cudaStream_t s);
 void free_tree(DeviceTree& D, cudaStream_t s);
 }  // namespace sbh

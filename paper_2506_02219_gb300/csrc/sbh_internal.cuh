@@ -57,8 +57,12 @@ struct TreeCtrl {
     float lo[3];
     float side;
     float diam[kDiamLevels];  // |B| at each level: sqrt(3) * side * d^-level (FP32, exact scaling)
-    int32_t error;        // nonzero if a build step detected an inconsistency
+    int32_t error;        // kErrorChildren, kErrorTimeout: a build step failed
+    int32_t bad_points;   // non-finite coordinates among the points
+    int32_t bad_weights;  // weights not finite or not > 0
 };
+constexpr int32_t kErrorChildren = 1;  // a node with more than kMaxChildren children
+constexpr int32_t kErrorTimeout = 2;   // a bounded wait gave up
 
 // Structure-of-arrays node storage of one tree (device pointers). Children of node v are the
 // contiguous ids fc[v] .. fc[v] + nchild - 1, in Morton order; generations are contiguous.

@@ -32,14 +32,11 @@ constexpr int kNoAllocMaxTiles = (int)((kNoAllocMaxPoints + kSortTile - 1) / kSo
 constexpr size_t round256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // layout of the scratch array
-constexpr size_t kOffKeys = 0;                                                            // u64 [max]
-constexpr size_t kOffVals = kOffKeys + round256(sizeof(uint64_t) * kNoAllocMaxPoints);    // i32 [max]
-constexpr size_t kOffHist = kOffVals + round256(sizeof(int32_t) * kNoAllocMaxPoints);     // i32 [256 x tiles]
-constexpr size_t kHistInts = (size_t)256 * kNoAllocMaxTiles;
-constexpr size_t kScanTempInts = kHistInts / 2048 + 16;                                   // >= scan_temp_ints
-constexpr size_t kOffScan = kOffHist + round256(sizeof(int) * kHistInts);
-constexpr size_t kOffBounds = kOffScan + round256(sizeof(int) * kScanTempInts);          // i32 [8]
-constexpr size_t kOffCtrl = kOffBounds + round256(sizeof(int) * 8);                       // TreeCtrl [2]
+constexpr size_t kOffKeys = 0;                                                          // u64 [max]
+constexpr size_t kOffVals = kOffKeys + round256(sizeof(uint64_t) * kNoAllocMaxPoints);  // i32 [max]
+constexpr size_t kOffStatus = kOffVals + round256(sizeof(int32_t) * kNoAllocMaxPoints); // u32 [2][tiles][256]
+constexpr size_t kOffHead = kOffStatus + round256(2 * 256 * sizeof(uint32_t) * kNoAllocMaxTiles);
+constexpr size_t kOffCtrl = kOffHead + round256(sizeof(SortHead));                      // TreeCtrl [2]
 constexpr size_t kScratchBytes = kOffCtrl + round256(2 * sizeof(TreeCtrl));
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
@@ -71,41 +68,14 @@ sbh_status sbh_morton_sort_noalloc(const float* points, int64_t n, uint64_t* cod
     }
     unsigned char* base = (unsigned char*)p;
     cudaStream_t s = (cudaStream_t)stream;
-    uint64_t* keys_tmp = (uint64_t*)(base + kOffKeys);
-    int32_t* vals_tmp = (int32_t*)(base + kOffVals);
-    int* hist = (int*)(base + kOffHist);
-    int* scan_tmp = (int*)(base + kOffScan);
-    int* bounds = (int*)(base + kOffBounds);
     TreeCtrl* ctrl = (TreeCtrl*)(base + kOffCtrl);
-
-    const unsigned grid = (unsigned)((n + 255) / 256 < 2432 ? (n + 255) / 256 : 2432);
-    k_bounds_init<<<1, 32, 0, s>>>(bounds);  // every call starts the min/max from scratch
-    note_launch();
-    // the weight count of k_bounds is not used here; the points array stands in for the weights
+    // the sort goes back and forth between the caller's outputs and the scratch copy and ends in the
+    // outputs. The count of bad weights is not used here; the points array stands in for the weights
     // (it has 3n floats, so the n reads stay inside it)
-    k_bounds<<<grid, 256, 0, s>>>(points, points, n, bounds);
-    note_launch();
-    k_root_cube<<<1, 32, 0, s>>>(bounds, ctrl, ctrl + 1);
-    note_launch();
-    // ping-pong between the caller's outputs and the scratch copy: 8 passes end in the outputs
-    uint64_t* k0 = codes;
-    int32_t* v0 = perm;
-    uint64_t* k1 = keys_tmp;
-    int32_t* v1 = vals_tmp;
-    k_morton<<<grid, 256, 0, s>>>(points, n, ctrl, k0, v0);
-    note_launch();
-    const int ntiles = (int)((n + kSortTile - 1) / kSortTile);
-    const int64_t nhist = (int64_t)256 * ntiles;
-    for (int pass = 0; pass < 8; ++pass) {
-        k_radix_hist<<<ntiles, kSortThreads, 0, s>>>(k0, n, 8 * pass, ntiles, hist);
-        note_launch();
-        scan_exclusive(hist, hist, nhist, scan_tmp, s);
-        k_radix_scatter<<<ntiles, kSortThreads, 0, s>>>(k0, v0, n, 8 * pass, ntiles, hist, k1, v1);
-        note_launch();
-        uint64_t* tk = k0; k0 = k1; k1 = tk;
-        int32_t* tv = v0; v0 = v1; v1 = tv;
-    }
-    e = cudaGetLastError();
+    uint64_t* const k[2] = {codes, (uint64_t*)(base + kOffKeys)};
+    int32_t* const v[2] = {perm, (int32_t*)(base + kOffVals)};
+    e = sort_codes(points, points, n, k, v, (SortHead*)(base + kOffHead), (uint32_t*)(base + kOffStatus), ctrl,
+                   ctrl + 1, s);
     if (e != cudaSuccess) {
         set_error_message("sbh_morton_sort_noalloc: kernel launch failed: %s", cudaGetErrorString(e));
         return SBH_ECUDA;

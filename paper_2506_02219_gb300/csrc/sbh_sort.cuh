@@ -1,5 +1,5 @@
-// sbh_sort.cuh -- the Morton-code and radix-sort kernels of the tree build (defined in
-// sbh_build.cu), declared for the other translation units that launch them.
+// sbh_sort.cuh -- the Morton-code and radix-sort step of the tree build (defined in sbh_build.cu),
+// declared for the other translation unit that runs it.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -9,21 +9,26 @@
 
 namespace sbh {
 
-constexpr int kSortThreads = 256;
+constexpr int kSortThreads = 512;
 constexpr int kSortItems = 8;
 constexpr int kSortTile = kSortThreads * kSortItems;
+constexpr int kPasses = 8;  // of 8 bits: an even number, so that the sort ends in the buffers it began in
 
-// scratch: [0..2] per-axis min (ordered int), [3..5] max, [6] bad coordinates, [7] bad weights
-__global__ void k_bounds_init(int* scratch);
-__global__ void k_bounds(const float* __restrict__ pts, const float* __restrict__ w, int64_t n,
-                         int* __restrict__ scratch);
-__global__ void k_root_cube(const int* __restrict__ scratch, TreeCtrl* c4, TreeCtrl* c2);
-__global__ void k_morton(const float* __restrict__ pts, int64_t n, const TreeCtrl* __restrict__ c4,
-                         uint64_t* __restrict__ code, int32_t* __restrict__ idx);
-__global__ void k_radix_hist(const uint64_t* __restrict__ keys, int64_t n, int shift, int ntiles,
-                             int* __restrict__ hist);
-__global__ void k_radix_scatter(const uint64_t* __restrict__ kin, const int32_t* __restrict__ vin, int64_t n,
-                                int shift, int ntiles, const int* __restrict__ offsets,
-                                uint64_t* __restrict__ kout, int32_t* __restrict__ vout);
+// Zeroed before each sort
+struct SortHead {
+    uint32_t bounds[8];          // ordered-integer maxima of -x, -y, -z, x, y, z; bad coordinates, bad weights
+    unsigned done[2];            // blocks of k_bounds, k_morton that are through
+    uint32_t next_tile[kPasses]; // tiles drawn in each pass
+    int32_t error;               // nonzero: a bounded wait gave up
+    int32_t hist[kPasses][256];  // counts of each digit, then where its run starts
+};
+
+// bytes of one of the two status arrays that a sort of n keys needs
+size_t sort_status_bytes(int64_t n);
+
+// Enqueue the root cube (c4, c2), the codes and their stable sort: k[0], v[0] get the sorted codes and
+// the input index of each; k[1], v[1] are scratch of the same size, status 2 x sort_status_bytes(n).
+cudaError_t sort_codes(const float* pts, const float* w, int64_t n, uint64_t* const k[2], int32_t* const v[2],
+                       SortHead* H, uint32_t* status, TreeCtrl* c4, TreeCtrl* c2, cudaStream_t s);
 
 }  // namespace sbh
