@@ -306,106 +306,6 @@ __global__ void __launch_bounds__(kMortonThreads) k_morton(const float* __restri
 }
 
 // ----------------------------------------------------------------------------------------------
-// Device-wide exclusive scan of int32 (reduce, scan the block sums, add): no inter-block waits.
-// ----------------------------------------------------------------------------------------------
-constexpr int kScanThreads = 256;
-constexpr int kScanItems = 8;
-constexpr int kScanTile = kScanThreads * kScanItems;
-
-// exclusive scan of one value per thread across the block; *total (if given) gets the sum
-__device__ __forceinline__ int block_exclusive_scan(int v, int* warp_sums, int* total)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int x = v;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const int y = __shfl_up_sync(0xFFFFFFFFu, x, off);
-        if (lane >= off) x += y;
-    }
-    if (lane == 31) warp_sums[warp] = x;
-    __syncthreads();
-    if (warp == 0) {
-        const int nw = blockDim.x >> 5;
-        int s = lane < nw ? warp_sums[lane] : 0;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const int y = __shfl_up_sync(0xFFFFFFFFu, s, off);
-            if (lane >= off) s += y;
-        }
-        if (lane < nw) warp_sums[lane] = s;
-    }
-    __syncthreads();
-    const int before = (warp > 0 ? warp_sums[warp - 1] : 0) + x - v;
-    if (total) *total = warp_sums[(blockDim.x >> 5) - 1];
-    __syncthreads();
-    return before;
-}
-
-__global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const int* __restrict__ in, int64_t n,
-                                                              int* __restrict__ sums)
-{
-    __shared__ int ws[32];
-    const int64_t base = (int64_t)blockIdx.x * kScanTile;
-    int s = 0;
-#pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
-        const int64_t i = base + (int64_t)k * kScanThreads + threadIdx.x;
-        if (i < n) s += in[i];
-    }
-    int total;
-    block_exclusive_scan(s, ws, &total);
-    if (threadIdx.x == 0) sums[blockIdx.x] = total;
-}
-
-// exclusive scan of each tile plus a per-tile offset (offsets may be nullptr); in may alias out
-__global__ void __launch_bounds__(kScanThreads) k_scan_tile(const int* in, int64_t n,
-                                                            const int* __restrict__ offsets, int* out)
-{
-    __shared__ int ws[32];
-    const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
-    int v[kScanItems];
-    int s = 0;
-#pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
-        v[k] = (base + k < n) ? in[base + k] : 0;
-        s += v[k];
-    }
-    int run = block_exclusive_scan(s, ws, nullptr) + (offsets ? offsets[blockIdx.x] : 0);
-#pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
-        if (base + k < n) out[base + k] = run;
-        run += v[k];
-    }
-}
-
-int64_t scan_temp_ints(int64_t n)
-{
-    int64_t total = 0;
-    while (n > kScanTile) {
-        n = (n + kScanTile - 1) / kScanTile;
-        total += n;
-    }
-    return total + 1;
-}
-
-void scan_exclusive(const int* in, int* out, int64_t n, int* temp, cudaStream_t s)
-{
-    if (n <= 0) return;
-    if (n <= kScanTile) {
-        k_scan_tile<<<1, kScanThreads, 0, s>>>(in, n, nullptr, out);
-        note_launch();
-        return;
-    }
-    const int64_t nb = (n + kScanTile - 1) / kScanTile;
-    int* sums = temp;
-    k_scan_reduce<<<(unsigned)nb, kScanThreads, 0, s>>>(in, n, sums);
-    note_launch();
-    scan_exclusive(sums, sums, nb, temp + nb, s);
-    k_scan_tile<<<(unsigned)nb, kScanThreads, 0, s>>>(in, n, sums, out);
-    note_launch();
-}
-
-// ----------------------------------------------------------------------------------------------
 // 3. stable LSD radix sort of (code, index) pairs, 8-bit digits, one kernel per pass: each tile
 //    ranks its keys by digit (warp by warp, lanes of equal digit found by a match, so the order is
 //    kept), learns from the tiles before it how many keys of each digit they hold, and writes its keys
@@ -600,197 +500,413 @@ cudaError_t sort_codes(const float* pts, const float* w, int64_t n, uint64_t* co
 
 // ----------------------------------------------------------------------------------------------
 // 4. gather into Morton order; shared code digits of neighbouring codes
+//    lcp[i] = leading code digits (6 bits for d = 4, 3 bits for d = 2) shared by sorted codes i-1 and
+//    i, capped at the deepest level; lcp[0] is not used
 // ----------------------------------------------------------------------------------------------
-__global__ void k_gather(const float* __restrict__ pts, const float* __restrict__ w,
-                         const float* __restrict__ nrm, const int32_t* __restrict__ perm, int64_t n,
-                         float4* __restrict__ spw, float4* __restrict__ snrm)
+constexpr int kTopoThreads = 512;
+constexpr int kTopoWarps = kTopoThreads / 32;
+constexpr int kTopoTile = 8 * kTopoThreads;  // positions to a block, eight to a thread
+inline int64_t topo_tiles(int64_t n) { return (n + kTopoTile - 1) / kTopoTile; }
+
+// What a run of boundaries tells a scan from one side: bit L (L < 24) says whether the last boundary
+// with lcp <= L had lcp = L; bits 24..28 hold the smallest lcp. No boundary at all: kNoRun.
+constexpr uint32_t kNoRun = 31u << 24;
+__device__ __forceinline__ uint32_t run_one(int l) { return (1u << l) | ((uint32_t)l << 24); }
+// the run `far` followed by the run `near`: a boundary of near with lcp l settles every level >= l
+__device__ __forceinline__ uint32_t run_join(uint32_t far, uint32_t near)
+{
+    const uint32_t mf = far >> 24, mn = near >> 24;
+    const uint32_t keep = mn < 24u ? (1u << mn) - 1u : 0xFFFFFFu;
+    return (far & keep) | (near & 0xFFFFFFu) | (min(mf, mn) << 24);
+}
+
+// A thread's eight boundaries (bytes of l8; b of them exist, the first is position 0's if `first`) as
+// runs from the left and from the right, joined over the block: the tile's runs for both sides
+__device__ __forceinline__ void tile_runs(uint64_t l8, int b, bool first, uint32_t* __restrict__ from_left,
+                                          uint32_t* __restrict__ from_right, uint32_t (*s_run)[kTopoWarps])
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t f = kNoRun, r = kNoRun;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        if (k >= b || (k == 0 && first)) continue;
+        const uint32_t o = run_one((int)(l8 >> (8 * k)) & 0xFF);
+        f = run_join(f, o);
+        r = run_join(o, r);
+    }
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t g = __shfl_down_sync(0xFFFFFFFFu, f, off), q = __shfl_down_sync(0xFFFFFFFFu, r, off);
+        f = run_join(f, g);  // lane 0 ends with the whole warp, in order
+        r = run_join(q, r);
+    }
+    if (lane == 0) { s_run[0][warp] = f; s_run[1][warp] = r; }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        f = r = kNoRun;
+        for (int k = 0; k < kTopoWarps; ++k) f = run_join(f, s_run[0][k]);
+        for (int k = kTopoWarps - 1; k >= 0; --k) r = run_join(r, s_run[1][k]);
+        from_left[blockIdx.x] = f;
+        from_right[blockIdx.x] = r;
+    }
+}
+
+// the runs from the right are joined far to near too: the boundaries further right are `far`
+__global__ void __launch_bounds__(kTopoThreads) k_gather(const float* __restrict__ pts, const float* __restrict__ w,
+                                                         const float* __restrict__ nrm,
+                                                         const int32_t* __restrict__ perm,
+                                                         const uint64_t* __restrict__ code, int64_t n,
+                                                         float4* __restrict__ spw, float4* __restrict__ snrm,
+                                                         uint8_t* __restrict__ lcp4, uint8_t* __restrict__ lcp2)
 {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t j = perm[i];
         spw[i] = make_float4(pts[3 * j], pts[3 * j + 1], pts[3 * j + 2], w[j]);
         if (nrm) snrm[i] = make_float4(nrm[3 * j], nrm[3 * j + 1], nrm[3 * j + 2], 0.0f);
-    }
-}
-
-// lcp[i] = leading code digits (6 bits for d = 4, 3 bits for d = 2) shared by sorted codes i-1
-// and i, capped at the deepest level; lcp[0] is unused
-__global__ void k_lcp(const uint64_t* __restrict__ code, int64_t n, uint8_t* __restrict__ lcp4,
-                      uint8_t* __restrict__ lcp2)
-{
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        if (i == 0) { lcp4[0] = 0; lcp2[0] = 0; continue; }
-        const int same_bits = __clzll((long long)(code[i] ^ code[i - 1])) - 4;  // codes use 60 bits
-        lcp4[i] = (uint8_t)min(same_bits / 6, kMaxLevel4);
-        lcp2[i] = (uint8_t)min(same_bits / 3, kMaxLevel2);
+        const int same = i ? __clzll((long long)(code[i] ^ code[i - 1])) - 4 : 0;  // codes use 60 bits
+        lcp4[i] = (uint8_t)min(same / 6, kMaxLevel4);
+        lcp2[i] = (uint8_t)min(same / 3, kMaxLevel2);
     }
 }
 
 // ----------------------------------------------------------------------------------------------
-// 5. topology, one generation at a time
-//    cid[i] is the node of the newest generation holding sorted point i (-1 once the point has
-//    left the frontier). A child of an expandable node v starts at point i when i is v's first
-//    point, when v is a multi-point leaf (every point is a child), or when lcp[i] equals v's
-//    level (points i-1 and i differ in the digit just below v). Child id = generation base +
-//    inclusive scan of those flags - 1, so children of one parent are contiguous.
+// 5. topology, all generations at once
+//    The levels at which the nodes above point i split are a set A_i: level L is in it when the
+//    L-digit cell of i holds a boundary with lcp = L, that is when the nearest boundary with lcp <= L
+//    to the left of i, or to the right, has lcp = L. Both sides are scans of the boundaries (run_join).
+//    The generation of the node that splits at L is the number of smaller levels in A_i, the point's own
+//    is |A_i|, and the nodes whose first point is i are those that split below the boundary on its
+//    left, L > lcp[i], and the point: consecutive generations g0 .. g1. A node's id is its generation's
+//    base plus the number of nodes of that generation that start before it, so one scan of counts per
+//    (generation, tile) gives every id, and a node's first child, parent, last child and end are
+//    ids at the same position. With leaf_size > 1 the levels below the first ancestor with at most that
+//    many points are dropped from A_i (kSmallLeaf marks that ancestor).
+//    What bounds it: a few passes over the positions, one for each generation in the last kernel. It
+//    replaces seven kernels over all positions for every generation: 84 kernels and 1,180 us for 2^22
+//    points, now 5 and 174 us (2^20: 470 -> 58 us)
 // ----------------------------------------------------------------------------------------------
+constexpr uint32_t kSmallLeaf = 1u << 31;  // in a mask: its last level is a leaf for its size
+
 struct BuildArrays {
     int32_t* nb;
     int32_t* ne;
     int32_t* fc;
     int32_t* parent;
     uint32_t* meta;
-    int32_t* minl;    // smallest lcp strictly inside a new node (its split level)
-    int32_t* cid;
-    int32_t* flag;
-    int32_t* scan;
+    int32_t* skip;        // depth-first successors, or nullptr
+    int32_t* last_child;  // scratch, per node
+    uint32_t* mask;       // scratch, per position: A_i
+    int32_t* count;       // scratch, [generation][tile]
+    uint32_t* from_left;  // scratch, per tile
+    uint32_t* from_right;
     const uint8_t* lcp;
     TreeCtrl* ctrl;
     int64_t n;
     int leaf_size;
     int max_level;
+    int tiles;
 };
 
-// expandable node of the newest generation that holds point i, or -1
-__device__ __forceinline__ int32_t frontier_of(const BuildArrays& B, int64_t i)
+// eight lcp bytes from position i on (i a multiple of eight), and how many of them exist
+__device__ __forceinline__ uint64_t lcp8(const BuildArrays& B, int64_t i, int& have)
 {
-    const int32_t c = B.cid[i];
-    if (c < 0) return -1;
-    return meta_kind(B.meta[c]) != kPoint ? c : -1;
+    have = B.n - i >= 8 ? 8 : (B.n > i ? (int)(B.n - i) : 0);
+    if (have == 8) return *reinterpret_cast<const uint64_t*>(B.lcp + i);
+    uint64_t x = 0;
+    for (int k = 0; k < have; ++k) x |= (uint64_t)B.lcp[i + k] << (8 * k);
+    return x;
 }
 
-__device__ __forceinline__ int child_flag(const BuildArrays& B, int64_t i, int32_t v)
+__global__ void __launch_bounds__(kTopoThreads) k_topo_runs(BuildArrays B)
 {
-    if (v < 0) return 0;
-    const uint32_t m = B.meta[v];
-    if (meta_kind(m) == kMultiLeaf) return 1;
-    return (i == B.nb[v] || (int)B.lcp[i] == (int)meta_level(m)) ? 1 : 0;
+    __shared__ uint32_t s_run[2][kTopoWarps];
+    const int64_t i = (int64_t)blockIdx.x * kTopoTile + 8 * threadIdx.x;
+    int have;
+    const uint64_t l8 = lcp8(B, i, have);
+    tile_runs(l8, have, i == 0, B.from_left, B.from_right, s_run);
 }
 
-__global__ void k_min_u8(const uint8_t* __restrict__ lcp, int64_t n, int* __restrict__ out_min)
+// The run of all tiles before tile t (dir = -1) or after it (+1), by one warp, nearest tiles first:
+// it stops where level 0 is settled, which settles every level
+__device__ __forceinline__ uint32_t carry_run(const uint32_t* __restrict__ runs, int t, int dir, int tiles)
 {
-    int m = 255;
-    for (int64_t i = 1 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        m = min(m, (int)lcp[i]);
+    const int lane = threadIdx.x & 31;
+    uint32_t carry = kNoRun;
+    for (int p = t + dir; p >= 0 && p < tiles; p += 32 * dir) {
+        const int k = p + lane * dir;
+        uint32_t x = k >= 0 && k < tiles ? runs[k] : kNoRun;
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) m = min(m, __shfl_xor_sync(0xFFFFFFFFu, m, off));
-    if ((threadIdx.x & 31) == 0 && m < 255) atomicMin(out_min, m);
-}
-
-__global__ void k_set_int(int* p, int v)
-{
-    if (threadIdx.x == 0 && blockIdx.x == 0) *p = v;
-}
-
-// the root: point, multi-point leaf (n <= leaf_size, or every code equal), or internal at its
-// split level (collapsed down to the first level at which its points separate)
-__global__ void k_topo_root(BuildArrays B, const int* __restrict__ root_min)
-{
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    const int64_t n = B.n;
-    uint32_t kind, level;
-    if (n == 1) { kind = kPoint; level = 0; }
-    else if (n <= B.leaf_size) { kind = kMultiLeaf; level = 0; }
-    else {
-        const int L = *root_min;
-        if (L >= B.max_level) { kind = kMultiLeaf; level = (uint32_t)B.max_level; }
-        else { kind = kInternal; level = (uint32_t)L; }
-    }
-    B.nb[0] = 0;
-    B.ne[0] = (int32_t)n;
-    B.parent[0] = -1;
-    B.fc[0] = -1;
-    B.meta[0] = meta_pack(0, level, kind);
-    for (int g = 0; g < kMaxDepth + 2; ++g) B.ctrl->depth_base[g] = 1;
-    B.ctrl->depth_base[0] = 0;
-    B.ctrl->max_depth = 0;
-}
-
-__global__ void k_topo_seed(BuildArrays B)
-{
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < B.n; i += (int64_t)gridDim.x * blockDim.x)
-        B.cid[i] = 0;
-}
-
-__global__ void k_topo_flags(BuildArrays B)
-{
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < B.n; i += (int64_t)gridDim.x * blockDim.x)
-        B.flag[i] = child_flag(B, i, frontier_of(B, i));
-}
-
-// after the scan: ranges and parent links of generation gen + 1
-__global__ void k_topo_children(BuildArrays B, int gen)
-{
-    const int32_t base = B.ctrl->depth_base[gen + 1];
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < B.n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int f = B.flag[i];
-        if (i == B.n - 1) {
-            const int32_t total = B.scan[i] + f;
-            B.ctrl->depth_base[gen + 2] = base + total;
-            if (total > 0) B.ctrl->max_depth = gen + 1;
+        for (int off = 1; off < 32; off <<= 1) {
+            const uint32_t y = __shfl_down_sync(0xFFFFFFFFu, x, off);  // higher lanes are further away
+            x = run_join(lane + off < 32 ? y : kNoRun, x);
         }
-        const int32_t v = frontier_of(B, i);
-        if (v < 0) continue;
-        const int32_t c = base + B.scan[i] + f - 1;  // child holding point i
-        if (f) {
-            B.nb[c] = (int32_t)i;
-            B.parent[c] = v;
-            B.minl[c] = 255;
-            B.fc[c] = -1;
-        }
-        if (i == B.nb[v]) B.fc[v] = c;
-        if (i + 1 == B.ne[v] || B.flag[i + 1]) B.ne[c] = (int32_t)(i + 1);
+        carry = run_join(__shfl_sync(0xFFFFFFFFu, x, 0), carry);
+        if ((carry >> 24) == 0u) break;
     }
+    return carry;
 }
 
-// smallest lcp strictly inside each new child, then the cid map of the new generation
-__global__ void k_topo_minlcp(BuildArrays B, int gen)
+// the levels of mask A that split at or above the boundary with lcp l on a node's left: g0 of them
+__device__ __forceinline__ int first_gen(uint32_t A, int l) { return __popc(A & ((2u << l) - 1u) & ~kSmallLeaf); }
+__device__ __forceinline__ int point_gen(uint32_t A) { return __popc(A & ~kSmallLeaf); }
+
+// A_i of every position, and the nodes of each generation that start in the tile
+__global__ void __launch_bounds__(kTopoThreads) k_topo_masks(BuildArrays B)
 {
-    const int32_t base = B.ctrl->depth_base[gen + 1];
-    for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x; i0 < B.n; i0 += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = i0 + threadIdx.x;
-        int32_t c = -1;
-        int val = 255;
-        if (i < B.n) {
-            const int32_t v = frontier_of(B, i);
-            if (v >= 0) {
-                const int f = B.flag[i];
-                c = base + B.scan[i] + f - 1;
-                if (!f) val = B.lcp[i];
+    __shared__ uint32_t s_run[2][kTopoWarps];
+    __shared__ uint32_t s_carry[2];
+    __shared__ int s_count[kMaxDepth + 1];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t i0 = (int64_t)blockIdx.x * kTopoTile + 8 * threadIdx.x;
+    int have;
+    const uint64_t l8 = lcp8(B, i0, have);
+    if (threadIdx.x <= kMaxDepth) s_count[threadIdx.x] = 0;
+    // runs of the thread, then inclusive over the lanes before (after) it
+    uint32_t f = kNoRun, r = kNoRun;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        if (k >= have || (k == 0 && i0 == 0)) continue;
+        const uint32_t o = run_one((int)(l8 >> (8 * k)) & 0xFF);
+        f = run_join(f, o);
+        r = run_join(o, r);
+    }
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t g = __shfl_up_sync(0xFFFFFFFFu, f, off), q = __shfl_down_sync(0xFFFFFFFFu, r, off);
+        if (lane >= off) f = run_join(g, f);
+        if (lane + off < 32) r = run_join(q, r);
+    }
+    if (lane == 31) s_run[0][warp] = f;
+    if (lane == 0) s_run[1][warp] = r;
+    if (warp == 0) {
+        const uint32_t c = carry_run(B.from_left, (int)blockIdx.x, -1, B.tiles);
+        if (lane == 0) s_carry[0] = c;
+    }
+    if (warp == 1) {
+        const uint32_t c = carry_run(B.from_right, (int)blockIdx.x, 1, B.tiles);
+        if (lane == 0) s_carry[1] = c;
+    }
+    f = __shfl_up_sync(0xFFFFFFFFu, f, 1);
+    r = __shfl_down_sync(0xFFFFFFFFu, r, 1);
+    if (lane == 0) f = kNoRun;
+    if (lane == 31) r = kNoRun;
+    __syncthreads();
+    uint32_t left = s_carry[0], right = s_carry[1];
+    for (int k = 0; k < warp; ++k) left = run_join(left, s_run[0][k]);
+    for (int k = kTopoWarps - 1; k > warp; --k) right = run_join(right, s_run[1][k]);
+    left = run_join(left, f);
+    right = run_join(right, r);
+    // each position: the boundaries up to its own from the left, those after it from the right
+    uint32_t A[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        if (k < have && !(k == 0 && i0 == 0)) left = run_join(left, run_one((int)(l8 >> (8 * k)) & 0xFF));
+        A[k] = left & 0xFFFFFFu;
+    }
+#pragma unroll
+    for (int k = 7; k >= 0; --k) {
+        A[k] |= right & 0xFFFFFFu;
+        if (k < have && !(k == 0 && i0 == 0)) right = run_join(right, run_one((int)(l8 >> (8 * k)) & 0xFF));
+    }
+    if (B.leaf_size > 1) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            if (k >= have) continue;
+            // widen the point's run level by level, deepest first, while it is small enough for a leaf
+            int64_t a = i0 + k, b = a + 1;
+            uint32_t rest = A[k], keep = A[k];
+            while (rest) {
+                const int L = 31 - __clz(rest);
+                while (a > 0 && b - a <= B.leaf_size && (int)B.lcp[a] >= L) --a;
+                while (b < B.n && b - a <= B.leaf_size && (int)B.lcp[b] >= L) ++b;
+                if (b - a > B.leaf_size) break;
+                keep = (A[k] & ((2u << L) - 1u)) | kSmallLeaf;
+                rest &= ~(1u << L);
+            }
+            A[k] = keep;
+        }
+    }
+    if (have == 8) {
+        uint4* d = reinterpret_cast<uint4*>(B.mask + i0);
+        d[0] = make_uint4(A[0], A[1], A[2], A[3]);
+        d[1] = make_uint4(A[4], A[5], A[6], A[7]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            if (k < have) B.mask[i0 + k] = A[k];
+    }
+    // bit g of gens: a node of generation g starts here
+    uint32_t gens[8], any = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const int l = i0 + k == 0 ? -1 : (int)(l8 >> (8 * k)) & 0xFF;
+        gens[k] = k < have ? (2u << point_gen(A[k])) - (1u << (l < 0 ? 0 : first_gen(A[k], l))) : 0u;
+        any |= gens[k];
+    }
+    any = __reduce_or_sync(0xFFFFFFFFu, any);
+    for (int g = 0; any >> g; ++g) {
+        int c = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) c += (int)(gens[k] >> g) & 1;
+        c = __reduce_add_sync(0xFFFFFFFFu, c);
+        if (lane == 0) atomicAdd(&s_count[g], c);
+    }
+    __syncthreads();
+    if (threadIdx.x <= kMaxDepth) B.count[(int64_t)threadIdx.x * B.tiles + blockIdx.x] = s_count[threadIdx.x];
+}
+
+// Exclusive sums of the counts along the tiles, a warp to a generation, and the control block
+__global__ void __launch_bounds__(1024) k_topo_scan(BuildArrays B)
+{
+    __shared__ int s_total[32];
+    const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+    int run = 0;
+    if (g <= kMaxDepth) {
+        int32_t* c = B.count + (int64_t)g * B.tiles;
+        for (int b = 0; b < B.tiles; b += 128) {
+            int v[4], sum = 0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int i = b + 4 * lane + k;
+                v[k] = i < B.tiles ? c[i] : 0;
+                sum += v[k];
+            }
+            int x = sum;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int y = __shfl_up_sync(0xFFFFFFFFu, x, off);
+                if (lane >= off) x += y;
+            }
+            int at = run + x - sum;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int i = b + 4 * lane + k;
+                if (i < B.tiles) c[i] = at;
+                at += v[k];
+            }
+            run += __shfl_sync(0xFFFFFFFFu, x, 31);
+        }
+    }
+    if (lane == 0) s_total[g] = run;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    int base = 0, deepest = 0;
+    for (int k = 0; k <= kMaxDepth; ++k) {
+        B.ctrl->depth_base[k] = base;
+        base += s_total[k];
+        if (s_total[k]) deepest = k;
+    }
+    B.ctrl->depth_base[kMaxDepth + 1] = base;
+    B.ctrl->max_depth = deepest;
+    B.ctrl->n_nodes = base;
+    B.ctrl->first_sub = deepest > 0 ? 1 : 0;  // the root's children, or a lone point
+    B.ctrl->n_sub = s_total[deepest > 0 ? 1 : 0];
+}
+
+// The nodes' ranges, links, levels and kinds. A warp takes 256 positions, 32 at a time; for each
+// generation a ballot says at which of them a node starts.
+__global__ void __launch_bounds__(kTopoThreads) k_topo_emit(BuildArrays B)
+{
+    __shared__ int32_t s_base[kTopoWarps][kMaxDepth + 1];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned below = (1u << lane) - 1u;
+    const int64_t i0 = (int64_t)blockIdx.x * kTopoTile + warp * 256;
+    const int top = B.ctrl->max_depth;
+    {
+        uint32_t gens[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int64_t i = i0 + 32 * k + lane;
+            gens[k] = 0u;
+            if (i < B.n) {
+                const uint32_t A = B.mask[i];
+                gens[k] = (2u << point_gen(A)) - (1u << (i ? first_gen(A, B.lcp[i]) : 0));
             }
         }
-        const unsigned peers = __match_any_sync(0xFFFFFFFFu, c);
-        const int m = (int)__reduce_min_sync(peers, (unsigned)val);
-        if (c >= 0 && m < 255 && (threadIdx.x & 31) == __ffs(peers) - 1) atomicMin(&B.minl[c], m);
-        if (i < B.n) B.cid[i] = c;
+        for (int g = 0; g <= top; ++g) {
+            int c = 0;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) c += (int)(gens[k] >> g) & 1;
+            c = __reduce_add_sync(0xFFFFFFFFu, c);
+            if (lane == 0) s_base[warp][g] = c;
+        }
+    }
+    __syncthreads();
+    if ((int)threadIdx.x <= top) {  // where each warp's nodes of a generation begin
+        int at = B.ctrl->depth_base[threadIdx.x] + B.count[(int64_t)threadIdx.x * B.tiles + blockIdx.x];
+        for (int k = 0; k < kTopoWarps; ++k) {
+            const int c = s_base[k][threadIdx.x];
+            s_base[k][threadIdx.x] = at;
+            at += c;
+        }
+    }
+    __syncthreads();
+    for (int k = 0; k < 8; ++k) {
+        const int64_t i = i0 + 32 * k + lane;
+        const bool live = i < B.n;
+        if (!__any_sync(0xFFFFFFFFu, live)) break;
+        const uint32_t A = live ? B.mask[i] : 0u;
+        const int l = live && i ? (int)B.lcp[i] : -1;
+        const int g1 = live ? point_gen(A) : -1;
+        const int g0 = live ? (l < 0 ? 0 : first_gen(A, l)) : kMaxDepth + 1;
+        int gp = __shfl_up_sync(0xFFFFFFFFu, g1, 1);  // the generation of the point before
+        if (lane == 0) gp = i0 + 32 * k > 0 ? point_gen(B.mask[i0 + 32 * k - 1]) : -1;
+        const bool end = live && i == B.n - 1;
+        const bool small = (A & kSmallLeaf) != 0u;
+        uint32_t rest = A & ~kSmallLeaf;
+        int level = -1;       // of the generation before
+        int32_t before = 0;   // nodes of the generation before that start before this position (as ids)
+        int32_t first = -1;   // the first node that starts here
+        int started = 0;      // whether one of the generation before starts here
+        for (int g = 0; g <= top; ++g) {
+            const int starts = g >= g0 && g <= g1 ? 1 : 0;
+            const unsigned bal = __ballot_sync(0xFFFFFFFFu, starts);
+            const int32_t id = s_base[warp][g] + __popc(bal & below);
+            __syncwarp();
+            if (lane == 0) s_base[warp][g] += __popc(bal);
+            __syncwarp();
+            if (g <= g1) {
+                uint32_t kind = kPoint;
+                const int split = __ffs(rest) - 1;
+                rest &= rest - 1u;
+                if (g == g1) level = level + 1;
+                else if (small && g == g1 - 1) { kind = kMultiLeaf; level = level + 1; }
+                else { kind = split >= B.max_level ? kMultiLeaf : kInternal; level = split; }
+                if (starts) {
+                    if (g == g0) first = id;
+                    B.nb[id] = (int32_t)i;
+                    B.parent[id] = g ? before + started - 1 : -1;
+                    B.meta[id] = meta_pack(0, (uint32_t)level, kind);
+                    if (kind == kPoint) B.fc[id] = -1;
+                    if (started) B.fc[before] = id;
+                }
+            }
+            if (live && i > 0 && g >= g0 && g <= gp) {  // the node before this position ends here
+                B.ne[id - 1] = (int32_t)i;
+                if (B.skip) B.skip[id - 1] = first;
+            }
+            if (live && i > 0 && g > g0 && g <= gp) B.last_child[before - 1] = id - 1;
+            if (end && g <= g1) {
+                B.ne[id + starts - 1] = (int32_t)B.n;
+                if (B.skip) B.skip[id + starts - 1] = -1;
+                if (g) B.last_child[before + started - 1] = id + starts - 1;
+            }
+            before = id;
+            started = starts;
+        }
     }
 }
 
-// kind and level of each new child; child counts of the parents
-__global__ void k_topo_classify(BuildArrays B, int gen)
+// child counts, once the first and last children are known
+__global__ void k_topo_children(BuildArrays B)
 {
-    const int32_t base = B.ctrl->depth_base[gen + 1];
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < B.n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t c = B.cid[i];
-        if (c < base) continue;  // not in the new generation
-        const int32_t v = B.parent[c];
-        const uint32_t pm = B.meta[v];
-        if (i + 1 == B.ne[v]) {  // parent's last point: its last child is c
-            const uint32_t nc = (uint32_t)(c - B.fc[v] + 1);
-            if (nc > kMaxChildren) B.ctrl->error = kErrorChildren;
-            B.meta[v] = meta_pack(nc, meta_level(pm), meta_kind(pm));
-        }
-        if (!B.flag[i]) continue;
-        const int32_t cnt = B.ne[c] - B.nb[c];
-        const uint32_t L1 = meta_level(pm) + 1;
-        uint32_t kind, level;
-        if (meta_kind(pm) == kMultiLeaf || cnt == 1) { kind = kPoint; level = L1; }
-        else if (cnt <= B.leaf_size) { kind = kMultiLeaf; level = L1; }
-        else {
-            const int m = B.minl[c];
-            if (m >= B.max_level) { kind = kMultiLeaf; level = (uint32_t)B.max_level; }
-            else { kind = kInternal; level = (uint32_t)m; }
-        }
-        B.meta[c] = meta_pack(0, level, kind);
+    const int32_t N = B.ctrl->n_nodes;
+    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < N; v += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t m = B.meta[v];
+        if (meta_kind(m) == kPoint) continue;
+        const uint32_t nc = (uint32_t)(B.last_child[v] - B.fc[v] + 1);
+        if (nc > kMaxChildren) B.ctrl->error = kErrorChildren;
+        B.meta[v] = m | (nc & kMaxChildren);
     }
 }
 
@@ -900,34 +1016,6 @@ __global__ void k_guide(const int32_t* __restrict__ fc, const uint32_t* __restri
     }
 }
 
-__global__ void k_finalize(TreeCtrl* ctrl, const int32_t* __restrict__ fc, const uint32_t* __restrict__ meta)
-{
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    ctrl->n_nodes = ctrl->depth_base[ctrl->max_depth + 1];
-    const uint32_t m = meta[0];
-    if (meta_nchild(m) > 0) {
-        ctrl->first_sub = fc[0];
-        ctrl->n_sub = (int32_t)meta_nchild(m);
-    } else {
-        ctrl->first_sub = 0;
-        ctrl->n_sub = 1;
-    }
-}
-
-// depth-first successor after a node's subtree: its next sibling, else its parent's successor
-__global__ void k_skip(const int32_t* __restrict__ parent, const int32_t* __restrict__ fc,
-                       const uint32_t* __restrict__ meta, const TreeCtrl* __restrict__ ctrl, int gen,
-                       int32_t* __restrict__ skip)
-{
-    const int32_t lo = ctrl->depth_base[gen], hi = ctrl->depth_base[gen + 1];
-    for (int64_t v = lo + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < hi; v += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t p = parent[v];
-        if (p < 0) { skip[v] = -1; continue; }
-        const int32_t last = fc[p] + (int32_t)meta_nchild(meta[p]) - 1;
-        skip[v] = (v < last) ? (int32_t)(v + 1) : skip[p];
-    }
-}
-
 // ----------------------------------------------------------------------------------------------
 // host orchestration
 // ----------------------------------------------------------------------------------------------
@@ -980,7 +1068,6 @@ cudaError_t alloc_tree(DeviceTree& D, int64_t n, bool with_dip, bool with_skip, 
     SBH_TRY(dalloc((void**)&D.ne, cap * sizeof(int32_t), s));
     SBH_TRY(dalloc((void**)&D.parent, cap * sizeof(int32_t), s));
     if (with_skip) SBH_TRY(dalloc((void**)&D.skip, cap * sizeof(int32_t), s));
-    SBH_TRY(dalloc((void**)&D.minl, cap * sizeof(int32_t), s));
     SBH_TRY(dalloc((void**)&D.agg, cap * 8 * sizeof(double), s));
     if (!D.ctrl) SBH_TRY(dalloc((void**)&D.ctrl, sizeof(TreeCtrl), s));
     return cudaSuccess;
@@ -989,7 +1076,7 @@ cudaError_t alloc_tree(DeviceTree& D, int64_t n, bool with_dip, bool with_skip, 
 void free_tree(DeviceTree& D, cudaStream_t s)
 {
     dfree(D.pm, s); dfree(D.dip, s); dfree(D.pmd, s); dfree(D.cdf, s); dfree(D.gd, s); dfree(D.fc, s); dfree(D.meta, s); dfree(D.nb, s);
-    dfree(D.ne, s); dfree(D.parent, s); dfree(D.skip, s); dfree(D.minl, s); dfree(D.agg, s); dfree(D.ctrl, s);
+    dfree(D.ne, s); dfree(D.parent, s); dfree(D.skip, s); dfree(D.agg, s); dfree(D.ctrl, s);
     D = DeviceTree();
 }
 
@@ -1019,9 +1106,8 @@ cudaError_t build_sorted(sbh_tree* T, const float* pts, const float* w, const fl
     if (nrm) SBH_TRY(dalloc((void**)&T->snrm, n * sizeof(float4), s));
     SBH_TRY(dalloc((void**)&T->lcp4, n, s));
     SBH_TRY(dalloc((void**)&T->lcp2, n, s));
-    k_gather<<<grid_for(n), kThreads, 0, s>>>(pts, w, nrm, T->perm, n, T->spw, T->snrm);
-    note_launch();
-    k_lcp<<<grid_for(n), kThreads, 0, s>>>(T->code, n, T->lcp4, T->lcp2);
+    k_gather<<<grid_for(n, kTopoThreads, 8u * (unsigned)device_sm_count()), kTopoThreads, 0, s>>>(
+        pts, w, nrm, T->perm, T->code, n, T->spw, T->snrm, T->lcp4, T->lcp2);
     note_launch();
     return cudaGetLastError();
 }
@@ -1033,39 +1119,28 @@ cudaError_t build_tree(sbh_tree* T, DeviceTree& D, const uint8_t* lcp, int max_l
     D.max_level = max_level;
     D.level_shift = level_shift;
     ScratchSet guard(s);
-    int32_t *cid = nullptr, *flag = nullptr, *scan = nullptr, *tmp = nullptr, *rmin = nullptr;
-    SBH_TRY(guard.alloc(&cid, n * sizeof(int32_t)));
-    SBH_TRY(guard.alloc(&flag, n * sizeof(int32_t)));
-    SBH_TRY(guard.alloc(&scan, n * sizeof(int32_t)));
-    SBH_TRY(guard.alloc(&tmp, scan_temp_ints(n) * sizeof(int32_t)));
-    SBH_TRY(guard.alloc(&rmin, sizeof(int32_t)));
-
+    const int64_t tiles = topo_tiles(n);
     BuildArrays B;
-    B.nb = D.nb; B.ne = D.ne; B.fc = D.fc; B.parent = D.parent; B.meta = D.meta; B.minl = D.minl;
-    B.cid = cid; B.flag = flag; B.scan = scan; B.lcp = lcp; B.ctrl = D.ctrl; B.n = n;
-    B.leaf_size = T->leaf_size; B.max_level = max_level;
+    B.nb = D.nb; B.ne = D.ne; B.fc = D.fc; B.parent = D.parent; B.meta = D.meta;
+    B.skip = with_skip ? D.skip : nullptr;
+    B.lcp = lcp; B.ctrl = D.ctrl; B.n = n; B.leaf_size = T->leaf_size; B.max_level = max_level; B.tiles = (int)tiles;
+    SBH_TRY(guard.alloc(&B.mask, n * sizeof(uint32_t)));
+    SBH_TRY(guard.alloc(&B.last_child, D.cap * sizeof(int32_t)));
+    SBH_TRY(guard.alloc(&B.count, (kMaxDepth + 1) * tiles * sizeof(int32_t)));
+    SBH_TRY(guard.alloc(&B.from_left, 2 * tiles * sizeof(uint32_t)));
+    B.from_right = B.from_left + tiles;
 
-    const unsigned g = grid_for(n);
-    k_set_int<<<1, 32, 0, s>>>(rmin, 255);
+    k_topo_runs<<<(unsigned)tiles, kTopoThreads, 0, s>>>(B);
     note_launch();
-    k_min_u8<<<g, kThreads, 0, s>>>(lcp, n, rmin);
+    k_topo_masks<<<(unsigned)tiles, kTopoThreads, 0, s>>>(B);
     note_launch();
-    k_topo_root<<<1, 32, 0, s>>>(B, rmin);
+    k_topo_scan<<<1, 1024, 0, s>>>(B);
     note_launch();
-    k_topo_seed<<<g, kThreads, 0, s>>>(B);
+    k_topo_emit<<<(unsigned)tiles, kTopoThreads, 0, s>>>(B);
+    note_launch();
+    k_topo_children<<<grid_for(2 * n), kThreads, 0, s>>>(B);
     note_launch();
     const int generations = max_level + 2;  // levels strictly increase; points end one below the deepest level
-    for (int gen = 0; gen < generations; ++gen) {
-        k_topo_flags<<<g, kThreads, 0, s>>>(B);
-        note_launch();
-        scan_exclusive(flag, scan, n, tmp, s);
-        k_topo_children<<<g, kThreads, 0, s>>>(B, gen);
-        note_launch();
-        k_topo_minlcp<<<g, kThreads, 0, s>>>(B, gen);
-        note_launch();
-        k_topo_classify<<<g, kThreads, 0, s>>>(B, gen);
-        note_launch();
-    }
     SBH_TRY(cudaGetLastError());
     for (int gen = generations; gen >= 0; --gen) {
         k_aggregate<<<grid_for(n), kThreads, 0, s>>>(D.fc, D.meta, D.nb, T->spw, T->snrm, D.ctrl, gen, D.agg);
@@ -1076,14 +1151,6 @@ cudaError_t build_tree(sbh_tree* T, DeviceTree& D, const uint8_t* lcp, int max_l
     note_launch();
     k_guide<<<grid_for(2 * n), kThreads, 0, s>>>(D.fc, D.meta, D.parent, D.cdf, D.ctrl, D.gd);
     note_launch();
-    k_finalize<<<1, 32, 0, s>>>(D.ctrl, D.fc, D.meta);
-    note_launch();
-    if (with_skip) {
-        for (int gen = 0; gen <= generations; ++gen) {
-            k_skip<<<grid_for(n), kThreads, 0, s>>>(D.parent, D.fc, D.meta, D.ctrl, gen, D.skip);
-            note_launch();
-        }
-    }
     SBH_TRY(cudaGetLastError());
     D.built = true;
     return cudaSuccess;

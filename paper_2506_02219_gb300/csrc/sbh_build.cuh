@@ -24,7 +24,6 @@ struct DeviceTree {
     int32_t* ne = nullptr;
     int32_t* parent = nullptr;
     int32_t* skip = nullptr;
-    int32_t* minl = nullptr;
     double* agg = nullptr;   // [cap][8] FP64: m, m p (3), m n (3), 0
     TreeCtrl* ctrl = nullptr;
     bool built = false;
@@ -44,9 +43,6 @@ void dfree(void* p, cudaStream_t s);
 void set_allocator(sbh_alloc_fn a, sbh_free_fn f, void* ctx);
 void set_memory_limit(uint64_t bytes);
 uint64_t memory_in_use();
-
-int64_t scan_temp_ints(int64_t n);
-void scan_exclusive(const int* in, int* out, int64_t n, int* temp, cudaStream_t s);
 
 }  // namespace sbh
 
