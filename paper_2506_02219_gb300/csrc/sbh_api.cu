@@ -702,12 +702,14 @@ sbh_status sbh_mlp_train(sbh_mlp* net, const sbh_tree* tree, const float* querie
         if (e == cudaSuccess) e = sbh::dalloc((void**)&feats, total * 6 * sizeof(float), s);
         if (e == cudaSuccess) e = sbh::dalloc((void**)&targets, total * sizeof(float), s);
         if (e == cudaSuccess) e = sbh::mlp_dataset(tree, queries, set_q, set_node, n_sets, doff, kp, feats, targets, s);
-        // 3. full-batch Adam steps
+        // 3. full-batch Adam steps. Their losses wait in dcount, which is done with, and are copied nq at
+        // a time: a copy to pageable host memory waits for the step before it.
+        float* dloss = reinterpret_cast<float*>(dcount);
         for (int32_t k = 0; k < steps && e == cudaSuccess; ++k) {
-            e = sbh::mlp_loss_grad(net->M, feats, targets, doff, n_sets, s);
-            if (e == cudaSuccess && losses)
-                e = cudaMemcpyAsync(&losses[k], net->M.loss, sizeof(float), cudaMemcpyDeviceToHost, s);
-            if (e == cudaSuccess) e = sbh::mlp_adam_step(net->M, lr, s);
+            const int32_t at = (int32_t)(k % nq);
+            e = sbh::mlp_train_step(net->M, feats, targets, doff, n_sets, lr, dloss + at, s);
+            if (e == cudaSuccess && losses && (at == nq - 1 || k == steps - 1))
+                e = cudaMemcpyAsync(&losses[k - at], dloss, (at + 1) * sizeof(float), cudaMemcpyDeviceToHost, s);
         }
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // the host copies of `losses` are complete
     }

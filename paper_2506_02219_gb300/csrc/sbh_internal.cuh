@@ -131,16 +131,26 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k)
 // 24 random bits as a float in [0, 1): exact in FP32
 __device__ __forceinline__ float unit24(uint32_t x) { return __uint2float_rn(x >> 8) * 5.9604644775390625e-8f; }
 
+// (double)f by integer operations: the conversion instruction runs at the FP64 rate, two lanes to an
+// SM and clock. Exact for every f (subnormals take the instruction).
+__device__ __forceinline__ double widen(float f)
+{
+    const uint32_t u = __float_as_uint(f);
+    if ((u & 0x7F800000u) - 0x00800000u >= 0x7F000000u)  // zero, subnormal, infinite or not a number
+        return (u << 1) == 0u ? __hiloint2double((int)u, 0) : (double)f;
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(u << 29));
+}
+
 // ----------------------------------------------------------------------------------------------
 // FP32 decision arithmetic. Every step is one IEEE round-to-nearest operation with no
 // contraction, in a fixed order, so that a CPU reference in FP32 reproduces it bit for bit.
 // ----------------------------------------------------------------------------------------------
-__device__ __forceinline__ float dist_rn(float px, float py, float pz, float3 q)
+__device__ __forceinline__ float dist2_rn(float px, float py, float pz, float3 q)
 {
     const float dx = __fsub_rn(px, q.x), dy = __fsub_rn(py, q.y), dz = __fsub_rn(pz, q.z);
-    const float s = __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
-    return __fsqrt_rn(s);
+    return __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
 }
+__device__ __forceinline__ float dist_rn(float px, float py, float pz, float3 q) { return __fsqrt_rn(dist2_rn(px, py, pz, q)); }
 
 // Eq. 5 for the step from node T into its child c with the draw u: continue iff u < p,
 // p = min(1, max(1, beta~_T) / beta~_c), beta~ = ||q - p~|| / |B|. The child's cell is exactly

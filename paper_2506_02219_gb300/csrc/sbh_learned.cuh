@@ -351,7 +351,9 @@ cudaError_t mlp_sync_half(MlpState& M, cudaStream_t s);
 cudaError_t mlp_scores(const MlpState& M, const float* feats, int64_t n, float* out, cudaStream_t s);
 cudaError_t mlp_loss_grad(MlpState& M, const float* feats, const float* targets, const int64_t* off, int64_t n_sets,
                           cudaStream_t s);
-cudaError_t mlp_adam_step(MlpState& M, float lr, cudaStream_t s);
+// one full-batch Adam step; *loss (device) is the loss before it
+cudaError_t mlp_train_step(MlpState& M, const float* feats, const float* targets, const int64_t* off, int64_t n_sets,
+                           float lr, float* loss, cudaStream_t s);
 // training sets visited by Algorithm 2's own paths: base == nullptr counts per query, else writes
 cudaError_t mlp_visit(const TreeView& T, const float* Q, int nq, int samples, uint64_t seed, float near,
                       int max_per_query, int32_t* count, const int64_t* base, int32_t* set_q, int32_t* set_node,
