@@ -798,6 +798,7 @@ sbh_status sbh_eval_bh(sbh_tree* tree, const float* queries, int64_t nq, sbh_ker
         // the root cube of t2.ctrl was written by sbh_build; alloc_tree keeps that block
         cudaError_t e = sbh::alloc_tree(tree->t2, tree->n, tree->has_normals != 0, true, false, s);
         if (e == cudaSuccess) e = sbh::build_tree(tree, tree->t2, tree->lcp2, sbh::kMaxLevel2, 1, true, s);
+        if (e == cudaSuccess) e = sbh::add_walk_records(tree->t2, s);
         if (e != cudaSuccess) {  // give back what was taken, keep the control block with the root cube
             sbh::TreeCtrl* ctrl = tree->t2.ctrl;
             tree->t2.ctrl = nullptr;
@@ -810,7 +811,7 @@ sbh_status sbh_eval_bh(sbh_tree* tree, const float* queries, int64_t nq, sbh_ker
     if (nq == 0) return SBH_OK;
     if (!device_ptr(queries) || !device_ptr(out)) return fail(SBH_EINVAL, "queries and out must be device memory");
     const float beta = theta > 0.0f ? 1.0f / theta : INFINITY;
-    cudaError_t e = sbh::launch_bh_eval(tree->t2.view(), queries, nq, kp, beta, warp_vote ? 1 : 0, out, s);
+    cudaError_t e = sbh::launch_bh_eval(tree->t2, queries, nq, kp, beta, warp_vote ? 1 : 0, out, s);
     if (e != cudaSuccess) return cuda_fail(e, "sbh_eval_bh launch");
     return SBH_OK;
 }

@@ -7,10 +7,26 @@
 // that node's subtree (its next sibling, else its parent's skip). With warp voting the 32 queries
 // of a warp walk together: a node is opened when any of them needs it, so every lane reads the
 // same node (one broadcast load) and no lane diverges; the sum only gets more accurate.
+//
+// What bounds the walk is the instructions of a step and the chain from one node's record to the
+// next one's address, so a step is kept short:
+//   - one 32-byte record per node holds its centre, mass, first child, skip and level
+//     (k_walk_records): one load, where position, meta word and link were three, the last of them
+//     behind the test;
+//   - the far-field ratio is a correctly rounded root and quotient, and monotone in the squared
+//     distance, so the test is one comparison with the smallest squared distance that passes it at
+//     the node's level (open_limit): the same decisions without either operation.
+// Without voting each lane walks for itself, so a warp takes as long as its lanes' paths differ; calls
+// of kSortFrom queries or more walk in the order of the queries' Morton codes (sort_queries), which
+// changes neither a query's walk nor its sum.
+//   2^20 winding sources, 2^21 grid queries, voting, theta 0.5: 8.04 -> 6.04 ms. 2^18 Coulomb sources,
+// 10^6 random queries, theta 0.8, no voting: 1.68 -> 0.67 ms with the sort.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "sbh_build.cuh"
 #include "sbh_eval.cuh"
+#include "sbh_sort.cuh"
 
 namespace sbh {
 
@@ -28,20 +44,56 @@ __device__ __forceinline__ void bh_add(const TreeView& T, int32_t v, float4 p, f
     }
 }
 
-template <int KIND, bool VOTE>
-__global__ void __launch_bounds__(256) k_bh_eval(TreeView T, const float* __restrict__ Q, int64_t nq, KernelParams kp,
-                                                 float beta, float* __restrict__ out)
+// The smallest squared distance s with sqrt(s) / B >= beta, both operations rounded to nearest: they
+// never decrease with s, so a bisection over the floats finds it, near (beta B)^2 when that is a
+// normal number. NaN (no s passes) when even infinity does not.
+__device__ __forceinline__ bool far_enough(uint32_t s, float B, float beta)
 {
-    __shared__ float sdiam[kDiamLevels];
-    if (threadIdx.x < kDiamLevels) sdiam[threadIdx.x] = T.ctrl->diam[threadIdx.x];
+    return __fdiv_rn(__fsqrt_rn(__uint_as_float(s)), B) >= beta;
+}
+__device__ float open_limit(float B, float beta)
+{
+    const uint32_t inf = 0x7F800000u;
+    const float t = beta * B;
+    const uint32_t g = min(__float_as_uint(t * t) & 0x7FFFFFFFu, inf);
+    uint32_t lo = g > 8u ? g - 8u : 0u, hi = min(g + 8u, inf);
+    if (far_enough(lo, B, beta)) {
+        if (far_enough(0u, B, beta)) return 0.0f;
+        hi = lo;
+        lo = 0u;
+    }
+    if (!far_enough(hi, B, beta)) {
+        if (!far_enough(inf, B, beta)) return __uint_as_float(0x7FC00000u);
+        lo = hi;
+        hi = inf;
+    }
+    while (hi - lo > 1u) {  // lo does not pass, hi does
+        const uint32_t mid = lo + (hi - lo) / 2u;
+        if (far_enough(mid, B, beta)) hi = mid;
+        else lo = mid;
+    }
+    return __uint_as_float(hi);
+}
+
+// REC: the walk records are there (without the memory for them a node is read from its three arrays)
+template <int KIND, bool VOTE, bool REC>
+__global__ void __launch_bounds__(256) k_bh_eval(TreeView T, const float4* __restrict__ rec,
+                                                 const float* __restrict__ Q, int64_t nq, KernelParams kp, float beta,
+                                                 const int32_t* __restrict__ order, const int32_t* sort_error,
+                                                 float* __restrict__ out)
+{
+    __shared__ float s_limit[kDiamLevels];
+    if (threadIdx.x < kDiamLevels) s_limit[threadIdx.x] = open_limit(T.ctrl->diam[threadIdx.x], beta);
     __syncthreads();
+    if (order && *sort_error) order = nullptr;  // a bounded wait of the sort gave up: the caller's order
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int32_t n_nodes = T.ctrl->n_nodes;
     // the loop bound is warp-uniform so that voting warps stay converged
     const int64_t warp_base = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31);
     for (int64_t jb = warp_base; jb < nq; jb += stride) {
-        const int64_t j = jb + (threadIdx.x & 31);
-        const bool active = j < nq;
+        const int64_t i = jb + (threadIdx.x & 31);
+        const bool active = i < nq;
+        const int64_t j = active && order ? (int64_t)order[i] : i;
         const float3 q = active ? make_float3(Q[3 * j], Q[3 * j + 1], Q[3 * j + 2]) : make_float3(0.f, 0.f, 0.f);
         float acc = 0.0f;
         ExpAcc ex;
@@ -51,16 +103,27 @@ __global__ void __launch_bounds__(256) k_bh_eval(TreeView T, const float* __rest
         int32_t budget = n_nodes + 1;
         if (VOTE || active) {
             while (v >= 0 && budget-- > 0) {
-                const float4 p = __ldg(&T.pm[v]);
-                const uint32_t m = __ldg(&T.meta[v]);
-                bool use = meta_kind(m) == kPoint;
-                if (!use) use = __fdiv_rn(dist_rn(p.x, p.y, p.z, q), sdiam[meta_level(m)]) >= beta;
+                float4 p;
+                int32_t first, skip = 0;
+                bool use;
+                if constexpr (REC) {
+                    float4 r;
+                    ld_pmd(rec, v, p, r);
+                    first = __float_as_int(r.x);
+                    skip = __float_as_int(r.y);
+                    use = first < 0 || dist2_rn(p.x, p.y, p.z, q) >= s_limit[__float_as_int(r.z)];
+                } else {
+                    p = __ldg(&T.pm[v]);
+                    const uint32_t m = __ldg(&T.meta[v]);
+                    use = meta_kind(m) == kPoint || dist2_rn(p.x, p.y, p.z, q) >= s_limit[meta_level(m)];
+                    first = 0;
+                }
                 if (VOTE) use = __all_sync(0xFFFFFFFFu, use || !active);
                 if (use) {
                     if (active) bh_add<KIND>(T, v, p, q, kp, acc, ex);
-                    v = __ldg(&T.skip[v]);
+                    v = REC ? skip : __ldg(&T.skip[v]);
                 } else {
-                    v = __ldg(&T.fc[v]);
+                    v = REC ? first : __ldg(&T.fc[v]);
                 }
             }
         }
@@ -73,30 +136,64 @@ __global__ void __launch_bounds__(256) k_bh_eval(TreeView T, const float* __rest
     }
 }
 
-template <int KIND>
-static void launch_bh_kind(const TreeView& T, const float* Q, int64_t nq, const KernelParams& kp, float beta,
-                           int vote, float* out, cudaStream_t s, unsigned blocks)
+namespace {
+// Queries from which a walk without voting is worth the sort: it takes 45 us of launches and 20 us
+// per million queries.
+constexpr int64_t kSortFrom = 1 << 16;
+
+struct BhLaunch {
+    TreeView T;
+    const float4* rec;
+    const float* Q;
+    int64_t nq;
+    KernelParams kp;
+    float beta;
+    const int32_t* order;
+    const int32_t* sort_error;
+    float* out;
+    cudaStream_t s;
+    unsigned blocks;
+};
+
+template <int KIND, bool VOTE, bool REC>
+void launch_bh(const BhLaunch& L)
 {
-    if (vote) k_bh_eval<KIND, true><<<blocks, 256, 0, s>>>(T, Q, nq, kp, beta, out);
-    else k_bh_eval<KIND, false><<<blocks, 256, 0, s>>>(T, Q, nq, kp, beta, out);
+    k_bh_eval<KIND, VOTE, REC><<<L.blocks, 256, 0, L.s>>>(L.T, L.rec, L.Q, L.nq, L.kp, L.beta, L.order, L.sort_error, L.out);
     note_launch();
 }
 
-cudaError_t launch_bh_eval(const TreeView& T, const float* Q, int64_t nq, const KernelParams& kp, float beta,
+template <int KIND>
+void launch_bh_kind(const BhLaunch& L, bool vote)
+{
+    if (L.rec) vote ? launch_bh<KIND, true, true>(L) : launch_bh<KIND, false, true>(L);
+    else vote ? launch_bh<KIND, true, false>(L) : launch_bh<KIND, false, false>(L);
+}
+}  // namespace
+
+cudaError_t launch_bh_eval(const DeviceTree& D, const float* Q, int64_t nq, const KernelParams& kp, float beta,
                            int warp_vote, float* out, cudaStream_t s)
 {
     if (nq <= 0) return cudaSuccess;
     int64_t blocks = (nq + 255) / 256;
     const int64_t cap = (int64_t)device_sm_count() * 64;
     if (blocks > cap) blocks = cap;
-    switch (kp.kind) {
-    case SBH_COULOMB: launch_bh_kind<SBH_COULOMB>(T, Q, nq, kp, beta, warp_vote, out, s, (unsigned)blocks); break;
-    case SBH_WINDING: launch_bh_kind<SBH_WINDING>(T, Q, nq, kp, beta, warp_vote, out, s, (unsigned)blocks); break;
-    case SBH_SMOOTHDIST: launch_bh_kind<SBH_SMOOTHDIST>(T, Q, nq, kp, beta, warp_vote, out, s, (unsigned)blocks); break;
-    case SBH_AFFINE: launch_bh_kind<SBH_AFFINE>(T, Q, nq, kp, beta, warp_vote, out, s, (unsigned)blocks); break;
-    default: return cudaErrorInvalidValue;
+    BhLaunch L = {D.view(), D.rec, Q, nq, kp, beta, nullptr, nullptr, out, s, (unsigned)blocks};
+    void* scratch = nullptr;
+    if (!warp_vote && nq >= kSortFrom) {
+        const cudaError_t e = sort_queries(Q, nq, D.ctrl, &scratch, &L.order, &L.sort_error, s);
+        if (e != cudaSuccess) return e;
     }
-    return cudaGetLastError();
+    cudaError_t e = cudaSuccess;
+    switch (kp.kind) {
+    case SBH_COULOMB: launch_bh_kind<SBH_COULOMB>(L, warp_vote); break;
+    case SBH_WINDING: launch_bh_kind<SBH_WINDING>(L, warp_vote); break;
+    case SBH_SMOOTHDIST: launch_bh_kind<SBH_SMOOTHDIST>(L, warp_vote); break;
+    case SBH_AFFINE: launch_bh_kind<SBH_AFFINE>(L, warp_vote); break;
+    default: e = cudaErrorInvalidValue;
+    }
+    if (e == cudaSuccess) e = cudaGetLastError();
+    dfree(scratch, s);
+    return e;
 }
 
 }  // namespace sbh

@@ -253,29 +253,35 @@ __device__ __forceinline__ uint32_t quantise(float x, float lo, float scale)
 
 // The codes, and the histogram of each of their eight digits: counted per block in shared memory, added
 // up, and made exclusive sums (where each digit's run starts in its pass) by the last block. Lanes
-// that share a digit add once together in the top one, which has 16 values.
+// that share a digit add once together in the top one, which has 16 values. PASSES = kQueryPasses: the
+// codes of queries, eight bits an axis over the cube of twice the side around the root cube (queries
+// further out are taken as on its border).
+template <int PASSES>
 __global__ void __launch_bounds__(kMortonThreads) k_morton(const float* __restrict__ pts, int64_t n,
                                                            const TreeCtrl* __restrict__ c4, uint64_t* __restrict__ code,
                                                            SortHead* __restrict__ H)
 {
-    __shared__ int s_hist[kPasses][256];
-    for (int k = threadIdx.x; k < kPasses * 256; k += blockDim.x) (&s_hist[0][0])[k] = 0;
+    __shared__ int s_hist[PASSES][256];
+    for (int k = threadIdx.x; k < PASSES * 256; k += blockDim.x) (&s_hist[0][0])[k] = 0;
     __syncthreads();
-    const float lx = c4->lo[0], ly = c4->lo[1], lz = c4->lo[2];
-    const float scale = __fdiv_rn(1048576.0f, c4->side);
+    constexpr bool kQuery = PASSES == kQueryPasses;
+    const float out = kQuery ? 0.5f * c4->side : 0.0f;
+    const float lx = c4->lo[0] - out, ly = c4->lo[1] - out, lz = c4->lo[2] - out;
+    const float scale = __fdiv_rn(kQuery ? 128.0f : 1048576.0f, c4->side);
+    constexpr uint32_t kTop = kQuery ? 255u : 1048575u;
     for (int64_t b = blockIdx.x * (int64_t)blockDim.x; b < n; b += (int64_t)gridDim.x * blockDim.x) {
         const int64_t i = b + threadIdx.x;
         const unsigned live = __ballot_sync(0xFFFFFFFFu, i < n);
         if (i >= n) continue;
-        const uint32_t cx = quantise(pts[3 * i], lx, scale);
-        const uint32_t cy = quantise(pts[3 * i + 1], ly, scale);
-        const uint32_t cz = quantise(pts[3 * i + 2], lz, scale);
+        const uint32_t cx = min(quantise(pts[3 * i], lx, scale), kTop);
+        const uint32_t cy = min(quantise(pts[3 * i + 1], ly, scale), kTop);
+        const uint32_t cz = min(quantise(pts[3 * i + 2], lz, scale), kTop);
         const uint64_t c = (spread3(cx) << 2) | (spread3(cy) << 1) | spread3(cz);
         code[i] = c;
 #pragma unroll
-        for (int p = 0; p < kPasses; ++p) {
+        for (int p = 0; p < PASSES; ++p) {
             const int d = (int)(c >> (8 * p)) & 0xFF;
-            if (p < kPasses - 1) {
+            if (p < PASSES - 1) {
                 atomicAdd(&s_hist[p][d], 1);
             } else {
                 const unsigned peers = __match_any_sync(live, d);
@@ -284,13 +290,13 @@ __global__ void __launch_bounds__(kMortonThreads) k_morton(const float* __restri
         }
     }
     __syncthreads();
-    for (int k = threadIdx.x; k < kPasses * 256; k += blockDim.x) {
+    for (int k = threadIdx.x; k < PASSES * 256; k += blockDim.x) {
         const int v = (&s_hist[0][0])[k];
         if (v) atomicAdd(&H->hist[0][0] + k, v);
     }
     if (!last_block(&H->done[1])) return;
     const int p = threadIdx.x >> 5, lane = threadIdx.x & 31;  // a warp to a digit, eight values to a lane
-    if (p >= kPasses) return;
+    if (p >= PASSES) return;
     int v[8], sum = 0;
 #pragma unroll
     for (int k = 0; k < 8; ++k) { v[k] = __ldcg(&H->hist[p][8 * lane + k]); sum += v[k]; }
@@ -466,8 +472,8 @@ __global__ void k_sort_error(const SortHead* __restrict__ H, TreeCtrl* ctrl)
 }
 
 template <int ITEMS>
-static cudaError_t radix_passes(uint64_t* const k[2], int32_t* const v[2], int64_t n, SortHead* H, uint32_t* status,
-                                cudaStream_t s)
+static cudaError_t radix_passes(uint64_t* const k[2], int32_t* const v[2], int64_t n, int passes, SortHead* H,
+                                uint32_t* status, cudaStream_t s)
 {
     constexpr int kTile = kSortThreads * ITEMS;
     constexpr size_t kBytes = (size_t)kTile * (sizeof(uint64_t) + sizeof(int32_t)) + (kSortThreads / 32) * 256 * sizeof(uint16_t);
@@ -475,7 +481,7 @@ static cudaError_t radix_passes(uint64_t* const k[2], int32_t* const v[2], int64
     if (e != cudaSuccess) return e;
     const unsigned tiles = (unsigned)((n + kTile - 1) / kTile);
     const size_t words = (size_t)sort_tiles(n) * 256;
-    for (int pass = 0; pass < kPasses; ++pass) {
+    for (int pass = 0; pass < passes; ++pass) {
         const int a = pass & 1;
         k_radix_pass<ITEMS><<<tiles, kSortThreads, kBytes, s>>>(k[a], pass ? v[a] : nullptr, n, pass, H,
                                                                 status + a * words, status + (a ^ 1) * words, k[a ^ 1],
@@ -493,9 +499,46 @@ cudaError_t sort_codes(const float* pts, const float* w, int64_t n, uint64_t* co
     if (e != cudaSuccess) return e;
     k_bounds<<<grid_for(n, kThreads, 4u * (unsigned)device_sm_count()), kThreads, 0, s>>>(pts, w, n, H, c4, c2);
     note_launch();
-    k_morton<<<grid_for(n, kMortonThreads, 2u * (unsigned)device_sm_count()), kMortonThreads, 0, s>>>(pts, n, c4, k[0], H);
+    k_morton<kPasses><<<grid_for(n, kMortonThreads, 2u * (unsigned)device_sm_count()), kMortonThreads, 0, s>>>(pts, n, c4, k[0], H);
     note_launch();
-    return radix_passes<kSortItems>(k, v, n, H, status, s);
+    return radix_passes<kSortItems>(k, v, n, kPasses, H, status, s);
+}
+
+cudaError_t sort_queries(const float* q, int64_t n, const TreeCtrl* ctrl, void** scratch, const int32_t** order,
+                         const int32_t** error, cudaStream_t s)
+{
+    if (n < 1 || n >= (1 << 28)) return cudaSuccess;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(s, &cap);
+    if (e != cudaSuccess) return e;
+    if (cap != cudaStreamCaptureStatusNone) return cudaSuccess;
+    const auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
+    const size_t kb = up(n * sizeof(uint64_t)), vb = up(n * sizeof(int32_t)), hb = up(sizeof(SortHead));
+    if (dalloc(scratch, 2 * kb + 2 * vb + hb + 2 * sort_status_bytes(n), s) != cudaSuccess) {
+        cudaGetLastError();  // no memory: the caller's order
+        *scratch = nullptr;
+        return cudaSuccess;
+    }
+    unsigned char* at = static_cast<unsigned char*>(*scratch);
+    SortHead* H = reinterpret_cast<SortHead*>(at);
+    uint64_t* const k[2] = {reinterpret_cast<uint64_t*>(at + hb), reinterpret_cast<uint64_t*>(at + hb + kb)};
+    int32_t* const v[2] = {reinterpret_cast<int32_t*>(at + hb + 2 * kb), reinterpret_cast<int32_t*>(at + hb + 2 * kb + vb)};
+    uint32_t* status = reinterpret_cast<uint32_t*>(at + hb + 2 * kb + 2 * vb);
+    e = cudaMemsetAsync(H, 0, sizeof(SortHead), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(status, 0, sort_status_bytes(n), s);
+    if (e == cudaSuccess) {
+        k_morton<kQueryPasses><<<grid_for(n, kMortonThreads, 2u * (unsigned)device_sm_count()), kMortonThreads, 0, s>>>(q, n, ctrl, k[0], H);
+        note_launch();
+        e = radix_passes<kSortItems>(k, v, n, kQueryPasses, H, status, s);
+    }
+    if (e != cudaSuccess) {
+        dfree(*scratch, s);
+        *scratch = nullptr;
+        return e;
+    }
+    *order = v[kQueryPasses & 1];
+    *error = &H->error;
+    return cudaSuccess;
 }
 
 // ----------------------------------------------------------------------------------------------
@@ -1076,7 +1119,7 @@ cudaError_t alloc_tree(DeviceTree& D, int64_t n, bool with_dip, bool with_skip, 
 void free_tree(DeviceTree& D, cudaStream_t s)
 {
     dfree(D.pm, s); dfree(D.dip, s); dfree(D.pmd, s); dfree(D.cdf, s); dfree(D.gd, s); dfree(D.fc, s); dfree(D.meta, s); dfree(D.nb, s);
-    dfree(D.ne, s); dfree(D.parent, s); dfree(D.skip, s); dfree(D.agg, s); dfree(D.ctrl, s);
+    dfree(D.ne, s); dfree(D.parent, s); dfree(D.skip, s); dfree(D.rec, s); dfree(D.agg, s); dfree(D.ctrl, s);
     D = DeviceTree();
 }
 
@@ -1154,6 +1197,31 @@ cudaError_t build_tree(sbh_tree* T, DeviceTree& D, const uint8_t* lcp, int max_l
     SBH_TRY(cudaGetLastError());
     D.built = true;
     return cudaSuccess;
+}
+
+// Node v's walk record: centre of mass and mass; first child (-1: a point), skip, level, nothing
+__global__ void __launch_bounds__(kThreads) k_walk_records(TreeView T, float4* __restrict__ rec)
+{
+    const int32_t N = T.ctrl->n_nodes;
+    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < N; v += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t m = T.meta[v];
+        const bool point = meta_kind(m) == kPoint;
+        rec[2 * v] = T.pm[v];
+        rec[2 * v + 1] = make_float4(__int_as_float(point ? -1 : T.fc[v]), __int_as_float(T.skip[v]),
+                                     __int_as_float((int)meta_level(m)), 0.0f);
+    }
+}
+
+cudaError_t add_walk_records(DeviceTree& D, cudaStream_t s)
+{
+    if (dalloc((void**)&D.rec, 2 * D.cap * sizeof(float4), s) != cudaSuccess) {
+        cudaGetLastError();
+        D.rec = nullptr;
+        return cudaSuccess;
+    }
+    k_walk_records<<<grid_for(D.cap), kThreads, 0, s>>>(D.view(), D.rec);
+    note_launch();
+    return cudaGetLastError();
 }
 
 }  // namespace sbh

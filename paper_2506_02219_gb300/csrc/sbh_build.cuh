@@ -24,6 +24,7 @@ struct DeviceTree {
     int32_t* ne = nullptr;
     int32_t* parent = nullptr;
     int32_t* skip = nullptr;
+    float4* rec = nullptr;   // [cap][2]: the walk records (8-ary tree; optional, see add_walk_records)
     double* agg = nullptr;   // [cap][8] FP64: m, m p (3), m n (3), 0
     TreeCtrl* ctrl = nullptr;
     bool built = false;
@@ -73,4 +74,7 @@ cudaError_t build_tree(sbh_tree* T, DeviceTree& D, const uint8_t* lcp, int max_l
 cudaError_t build_sorted(sbh_tree* T, const float* pts, const float* w, const float* nrm, cudaStream_t s);
 cudaError_t alloc_tree(DeviceTree& D, int64_t n, bool with_dip, bool with_skip, bool with_rec, cudaStream_t s);
 void free_tree(DeviceTree& D, cudaStream_t s);
+// Enqueue the records the Barnes-Hut walk reads. They are 64 bytes per source that the tree can do
+// without: if there is no memory for them nothing is done and the walk reads the tree's arrays.
+cudaError_t add_walk_records(DeviceTree& D, cudaStream_t s);
 }  // namespace sbh

@@ -49,7 +49,8 @@ cudaError_t launch_stoch_batched_grad(const TreeView& T, const TreeCtrl& host_ct
                                       const KernelParams& kp, int S, uint64_t seed, const sbh_eval_opts& o, float* out,
                                       float* grad, cudaStream_t s);
 
-cudaError_t launch_bh_eval(const TreeView& T, const float* Q, int64_t nq, const KernelParams& kp, float beta,
+struct DeviceTree;
+cudaError_t launch_bh_eval(const DeviceTree& D, const float* Q, int64_t nq, const KernelParams& kp, float beta,
                            int warp_vote, float* out, cudaStream_t s);
 
 cudaError_t launch_brute(const float* P, const float* W, const float* N, int64_t n, const float* Q, int64_t nq,

@@ -13,6 +13,7 @@ constexpr int kSortThreads = 512;
 constexpr int kSortItems = 8;
 constexpr int kSortTile = kSortThreads * kSortItems;
 constexpr int kPasses = 8;  // of 8 bits: an even number, so that the sort ends in the buffers it began in
+constexpr int kQueryPasses = 3;
 
 // Zeroed before each sort
 struct SortHead {
@@ -30,5 +31,13 @@ size_t sort_status_bytes(int64_t n);
 // the input index of each; k[1], v[1] are scratch of the same size, status 2 x sort_status_bytes(n).
 cudaError_t sort_codes(const float* pts, const float* w, int64_t n, uint64_t* const k[2], int32_t* const v[2],
                        SortHead* H, uint32_t* status, TreeCtrl* c4, TreeCtrl* c2, cudaStream_t s);
+
+// Order of n queries by their Morton codes in twice the tree's root cube (24 bits, three passes): order[i]
+// is the query to take at place i, unless *error is set when the sort has run. Both are in *scratch,
+// for the caller to dfree when the work that reads them is enqueued. Where there is no memory for it,
+// where the stream is being captured (the scratch would be the graph's) or n is beyond the sort's
+// counters, nothing is done and order stays null.
+cudaError_t sort_queries(const float* q, int64_t n, const TreeCtrl* ctrl, void** scratch, const int32_t** order,
+                         const int32_t** error, cudaStream_t s);
 
 }  // namespace sbh
