@@ -16,11 +16,13 @@
 //   - the far-field ratio is a correctly rounded root and quotient, and monotone in the squared
 //     distance, so the test is one comparison with the smallest squared distance that passes it at
 //     the node's level (open_limit): the same decisions without either operation.
-// Without voting each lane walks for itself, so a warp takes as long as its lanes' paths differ; calls
-// of kSortFrom queries or more walk in the order of the queries' Morton codes (sort_queries), which
-// changes neither a query's walk nor its sum.
-//   2^20 winding sources, 2^21 grid queries, voting, theta 0.5: 8.04 -> 6.04 ms. 2^18 Coulomb sources,
-// 10^6 random queries, theta 0.8, no voting: 1.68 -> 0.67 ms with the sort.
+// Without voting a warp takes as long as its lanes' paths differ, and each lane reads its own record. Calls
+// of kSortFrom queries or more are walked in the order of the queries' Morton codes (sort_queries), a
+// warp going through the nodes that any of its queries visits (kTogether): neither changes a query's
+// walk or its sum.
+//   2^20 winding sources, 2^21 grid queries, voting, theta 0.5: 8.04 -> 6.04 ms with the record and the
+// comparison, 5.06 ms with the term taken from the test's differences. 2^18 Coulomb sources, 10^6 random
+// queries, theta 0.8, no voting: 1.68 -> 0.67 ms sorted, lanes alone, 0.58 ms together.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -30,17 +32,26 @@
 
 namespace sbh {
 
+// The node's term from d = p - q; r2 is its squared length as the test has it (every operation rounded),
+// which the Coulomb term takes too. The other two are singular at a source, or alpha times as
+// sensitive, and take the fused sum. The winding term is times 4 pi (the sum is scaled once), with the
+// squared length clamped as in term_winding_4pi.
 template <int KIND>
-__device__ __forceinline__ void bh_add(const TreeView& T, int32_t v, float4 p, float3 q, const KernelParams& kp,
-                                       float& acc, ExpAcc& ex)
+__device__ __forceinline__ void bh_add(float4 p, float4 dp, float3 d, float r2, const KernelParams& kp, float& acc,
+                                       ExpAcc& ex)
 {
-    if constexpr (KIND == SBH_COULOMB) acc += term_coulomb(p, q, kp.eps2);
-    else if constexpr (KIND == SBH_WINDING) acc += term_winding(p, __ldg(&T.dip[v]), q);
-    else if constexpr (KIND == SBH_AFFINE) acc += term_affine(p, q, kp.g);
-    else {
-        const float d = dist_fast(p, q);
-        ex.lower(d, kp.alpha);
-        ex.acc = fmaf(p.w, ex.scale(d, kp.alpha), ex.acc);
+    if constexpr (KIND == SBH_COULOMB) {
+        acc = fmaf(p.w, rsqrt_ftz(__fadd_rn(r2, kp.eps2)), acc);
+    } else if constexpr (KIND == SBH_WINDING) {
+        const float ir = rsqrt_ftz(fmaxf(fmaf(d.x, d.x, fmaf(d.y, d.y, d.z * d.z)), kMinNormal));
+        acc = fmaf(fmaf(d.x, dp.x, fmaf(d.y, dp.y, d.z * dp.z)) * ir, ir * ir, acc);
+    } else if constexpr (KIND == SBH_AFFINE) {
+        acc = fmaf(p.w, 1.0f + fmaf(kp.g[0], d.x, fmaf(kp.g[1], d.y, kp.g[2] * d.z)), acc);
+    } else {
+        const float f2 = fmaf(d.x, d.x, fmaf(d.y, d.y, d.z * d.z));
+        const float r = f2 * rsqrt_ftz(fmaxf(f2, 1e-37f));
+        ex.lower(r, kp.alpha);
+        ex.acc = fmaf(p.w, ex.scale(r, kp.alpha), ex.acc);
     }
 }
 
@@ -75,8 +86,17 @@ __device__ float open_limit(float B, float beta)
     return __uint_as_float(hi);
 }
 
+// How the lanes of a warp walk:
+//   kAlone     each for itself;
+//   kVote      together, a node opened for all when one needs it;
+//   kTogether  each query's own walk, the warp going through the nodes that any lane visits: a lane that
+//              is through with a subtree the others enter waits at its skip. All lanes read one record
+//              where lanes walking alone read one each, as soon as their paths differ. For queries near
+//              each other (sorted), whose nodes are mostly the same.
+enum { kAlone = 0, kVote = 1, kTogether = 2 };
+
 // REC: the walk records are there (without the memory for them a node is read from its three arrays)
-template <int KIND, bool VOTE, bool REC>
+template <int KIND, int MODE, bool REC>
 __global__ void __launch_bounds__(256) k_bh_eval(TreeView T, const float4* __restrict__ rec,
                                                  const float* __restrict__ Q, int64_t nq, KernelParams kp, float beta,
                                                  const int32_t* __restrict__ order, const int32_t* sort_error,
@@ -87,7 +107,7 @@ __global__ void __launch_bounds__(256) k_bh_eval(TreeView T, const float4* __res
     __syncthreads();
     if (order && *sort_error) order = nullptr;  // a bounded wait of the sort gave up: the caller's order
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const int32_t n_nodes = T.ctrl->n_nodes;
+    const int32_t n_nodes = T.ctrl->error ? -1 : T.ctrl->n_nodes;
     // the loop bound is warp-uniform so that voting warps stay converged
     const int64_t warp_base = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31);
     for (int64_t jb = warp_base; jb < nq; jb += stride) {
@@ -99,28 +119,39 @@ __global__ void __launch_bounds__(256) k_bh_eval(TreeView T, const float4* __res
         ExpAcc ex;
         ex.init(3.0e38f);
         int32_t v = 0;
+        int32_t own = active ? 0 : -1;  // kTogether: the node the lane's own walk is at
         // a depth-first walk enters every node at most once; the bound only guards a damaged tree
         int32_t budget = n_nodes + 1;
-        if (VOTE || active) {
+        if (MODE != kAlone || active) {
             while (v >= 0 && budget-- > 0) {
                 float4 p;
-                int32_t first, skip = 0;
-                bool use;
+                int32_t first = 0, skip = 0;
+                float limit;
+                bool point;
                 if constexpr (REC) {
                     float4 r;
                     ld_pmd(rec, v, p, r);
                     first = __float_as_int(r.x);
                     skip = __float_as_int(r.y);
-                    use = first < 0 || dist2_rn(p.x, p.y, p.z, q) >= s_limit[__float_as_int(r.z)];
+                    limit = *reinterpret_cast<const float*>(reinterpret_cast<const char*>(s_limit) + __float_as_int(r.z));
+                    point = first < 0;
                 } else {
                     p = __ldg(&T.pm[v]);
                     const uint32_t m = __ldg(&T.meta[v]);
-                    use = meta_kind(m) == kPoint || dist2_rn(p.x, p.y, p.z, q) >= s_limit[meta_level(m)];
-                    first = 0;
+                    limit = s_limit[meta_level(m)];
+                    point = meta_kind(m) == kPoint;
                 }
-                if (VOTE) use = __all_sync(0xFFFFFFFFu, use || !active);
-                if (use) {
-                    if (active) bh_add<KIND>(T, v, p, q, kp, acc, ex);
+                // dist2_rn, its differences kept
+                const float3 d = make_float3(__fsub_rn(p.x, q.x), __fsub_rn(p.y, q.y), __fsub_rn(p.z, q.z));
+                const float r2 = __fadd_rn(__fadd_rn(__fmul_rn(d.x, d.x), __fmul_rn(d.y, d.y)), __fmul_rn(d.z, d.z));
+                bool use = point || r2 >= limit;
+                if (MODE == kVote) use = __all_sync(0xFFFFFFFFu, use || !active);
+                const bool mine = MODE == kTogether ? own == v : active;
+                if (use && mine) bh_add<KIND>(p, KIND == SBH_WINDING ? __ldg(&T.dip[v]) : p, d, r2, kp, acc, ex);
+                if constexpr (MODE == kTogether) {
+                    if (mine) own = use ? skip : first;
+                    v = __any_sync(0xFFFFFFFFu, mine && !use) ? first : skip;
+                } else if (use) {
                     v = REC ? skip : __ldg(&T.skip[v]);
                 } else {
                     v = REC ? first : __ldg(&T.fc[v]);
@@ -131,7 +162,7 @@ __global__ void __launch_bounds__(256) k_bh_eval(TreeView T, const float4* __res
         if (active) {
             if constexpr (KIND == SBH_SMOOTHDIST)
                 out[j] = ex.acc > 0.0f ? ex.ref - __logf(ex.acc) / kp.alpha : __int_as_float(0x7F800000);
-            else out[j] = acc;
+            else out[j] = KIND == SBH_WINDING ? acc * kInv4Pi : acc;
         }
     }
 }
@@ -155,18 +186,19 @@ struct BhLaunch {
     unsigned blocks;
 };
 
-template <int KIND, bool VOTE, bool REC>
+template <int KIND, int MODE, bool REC>
 void launch_bh(const BhLaunch& L)
 {
-    k_bh_eval<KIND, VOTE, REC><<<L.blocks, 256, 0, L.s>>>(L.T, L.rec, L.Q, L.nq, L.kp, L.beta, L.order, L.sort_error, L.out);
+    k_bh_eval<KIND, MODE, REC><<<L.blocks, 256, 0, L.s>>>(L.T, L.rec, L.Q, L.nq, L.kp, L.beta, L.order, L.sort_error, L.out);
     note_launch();
 }
 
 template <int KIND>
 void launch_bh_kind(const BhLaunch& L, bool vote)
 {
-    if (L.rec) vote ? launch_bh<KIND, true, true>(L) : launch_bh<KIND, false, true>(L);
-    else vote ? launch_bh<KIND, true, false>(L) : launch_bh<KIND, false, false>(L);
+    if (vote) L.rec ? launch_bh<KIND, kVote, true>(L) : launch_bh<KIND, kVote, false>(L);
+    else if (L.rec) L.order ? launch_bh<KIND, kTogether, true>(L) : launch_bh<KIND, kAlone, true>(L);
+    else launch_bh<KIND, kAlone, false>(L);
 }
 }  // namespace
 
@@ -179,7 +211,7 @@ cudaError_t launch_bh_eval(const DeviceTree& D, const float* Q, int64_t nq, cons
     if (blocks > cap) blocks = cap;
     BhLaunch L = {D.view(), D.rec, Q, nq, kp, beta, nullptr, nullptr, out, s, (unsigned)blocks};
     void* scratch = nullptr;
-    if (!warp_vote && nq >= kSortFrom) {
+    if (!warp_vote && D.rec && nq >= kSortFrom) {
         const cudaError_t e = sort_queries(Q, nq, D.ctrl, &scratch, &L.order, &L.sort_error, s);
         if (e != cudaSuccess) return e;
     }

@@ -1199,7 +1199,7 @@ cudaError_t build_tree(sbh_tree* T, DeviceTree& D, const uint8_t* lcp, int max_l
     return cudaSuccess;
 }
 
-// Node v's walk record: centre of mass and mass; first child (-1: a point), skip, level, nothing
+// Node v's walk record: centre of mass and mass; first child (-1: a point), skip, level times 4, nothing
 __global__ void __launch_bounds__(kThreads) k_walk_records(TreeView T, float4* __restrict__ rec)
 {
     const int32_t N = T.ctrl->n_nodes;
@@ -1208,7 +1208,7 @@ __global__ void __launch_bounds__(kThreads) k_walk_records(TreeView T, float4* _
         const bool point = meta_kind(m) == kPoint;
         rec[2 * v] = T.pm[v];
         rec[2 * v + 1] = make_float4(__int_as_float(point ? -1 : T.fc[v]), __int_as_float(T.skip[v]),
-                                     __int_as_float((int)meta_level(m)), 0.0f);
+                                     __int_as_float(4 * (int)meta_level(m)), 0.0f);
     }
 }
 
