@@ -666,6 +666,7 @@ __global__ void __launch_bounds__(kTopoThreads) k_topo_runs(BuildArrays B)
     const int64_t i = (int64_t)blockIdx.x * kTopoTile + 8 * threadIdx.x;
     int have;
     const uint64_t l8 = lcp8(B, i, have);
+    if (i == 0) B.from_right[B.tiles] = 0u;  // k_aggregate's barrier
     tile_runs(l8, have, i == 0, B.from_left, B.from_right, s_run);
 }
 
@@ -940,98 +941,107 @@ __global__ void __launch_bounds__(kTopoThreads) k_topo_emit(BuildArrays B)
     }
 }
 
-// child counts, once the first and last children are known
-__global__ void k_topo_children(BuildArrays B)
+// ----------------------------------------------------------------------------------------------
+// 6. aggregates and records, children before parents: one kernel over the generations from the deepest
+//    up, with a barrier of the grid between them. A node gets the FP64 sums of m, m p, m n of its
+//    children in their order, its FP32 record (quotients rounded once to FP32) and its child count;
+//    its children get their prefix mass fractions and the slots of the child pick's guide table.
+//    What bounds it is the FP64 unit, two lanes to an SM: a warp's FP64 instruction holds it for 16
+//    clocks, however few lanes take part. So
+//      - eight lanes work on a node, one to each of the seven sums and the padding (a thread to a
+//        node issued seven additions a child, for the widest of 32 nodes);
+//      - the prefix sums are the running sum of m (each child summed them anew);
+//      - quotients are FP32 pairs (quotient_rn), and conversions integer operations;
+//      - points, three nodes of four, take a lane each and only the products m p, m n.
+//    2^22 points: 1,090 us in 16 kernels -> 534 us; 4,096 points: 137 -> 39 us; the 8-ary and 64-ary
+//    trees of 2^18: 434 us in 42 kernels -> 190 us.
+// ----------------------------------------------------------------------------------------------
+struct Split {
+    float h, l;
+    bool ok;  // h + l is the value to 2^-47 of it, and far from FP32's limits
+};
+__device__ __forceinline__ Split split(double x)
 {
-    const int32_t N = B.ctrl->n_nodes;
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < N; v += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t m = B.meta[v];
-        if (meta_kind(m) == kPoint) continue;
-        const uint32_t nc = (uint32_t)(B.last_child[v] - B.fc[v] + 1);
-        if (nc > kMaxChildren) B.ctrl->error = kErrorChildren;
-        B.meta[v] = m | (nc & kMaxChildren);
-    }
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const uint32_t e = (hi >> 20) & 0x7FFu, sign = hi & 0x80000000u;
+    Split r;
+    r.ok = e - 963u <= 120u;  // 2^-60 .. 2^60
+    r.h = __uint_as_float(sign | ((((hi & 0x7FFFFFFFu) - 0x38000000u) << 3) | lo >> 29));
+    r.l = (float)(lo & 0x1FFFFFFFu) * __uint_as_float(sign | ((e - 948u) << 23));  // 2^(e - 1023 - 52)
+    return r;
 }
 
-// ----------------------------------------------------------------------------------------------
-// 6. aggregates: FP64 sums of m, m p, m n, children before parents (generations in reverse)
-// ----------------------------------------------------------------------------------------------
-__global__ void k_aggregate(const int32_t* __restrict__ fc, const uint32_t* __restrict__ meta,
-                            const int32_t* __restrict__ nb, const float4* __restrict__ spw,
-                            const float4* __restrict__ snrm, const TreeCtrl* __restrict__ ctrl, int gen,
-                            double* __restrict__ agg)
+// __double2float_rn(a / b), B = split(b), y = 1 / B.h to a few roundings. The quotient to 2^-44 of it as
+// an FP32 pair decides the rounding unless it is that near to the middle of two floats: there, a
+// remainder of zero says that the quotient is the middle (the centre of two equal masses often is),
+// and anything else takes the division.
+__device__ __forceinline__ float quotient_rn(double a, double b, const Split& B, float y)
 {
-    const int32_t lo = ctrl->depth_base[gen], hi = ctrl->depth_base[gen + 1];
-    for (int64_t v = lo + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < hi; v += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t m = meta[v];
-        double a[7];
-        if (meta_kind(m) == kPoint) {
-            const float4 p = spw[nb[v]];
-            const double w = p.w;
-            a[0] = w; a[1] = w * (double)p.x; a[2] = w * (double)p.y; a[3] = w * (double)p.z;
-            if (snrm) {
-                const float4 q = snrm[nb[v]];
-                a[4] = w * (double)q.x; a[5] = w * (double)q.y; a[6] = w * (double)q.z;
-            } else {
-                a[4] = a[5] = a[6] = 0.0;
-            }
-        } else {
-            for (int k = 0; k < 7; ++k) a[k] = 0.0;
-            const int32_t f = fc[v];
-            const int nc = (int)meta_nchild(m);
-            for (int c = 0; c < nc; ++c) {
-                const double* s = agg + 8 * (int64_t)(f + c);
-                for (int k = 0; k < 7; ++k) a[k] += s[k];
-            }
-        }
-        double* d = agg + 8 * v;
-        for (int k = 0; k < 7; ++k) d[k] = a[k];
-        d[7] = 0.0;
-    }
+    const uint32_t ah = (uint32_t)__double2hiint(a);
+    if (((ah << 1) | (uint32_t)__double2loint(a)) == 0u) return __uint_as_float(ah);
+    const Split A = split(a);
+    if (!A.ok || !B.ok) return __double2float_rn(a / b);
+    const float q1 = __fmul_rn(A.h, y);
+    const float r = __fadd_rn(__fmaf_rn(-q1, B.l, __fmaf_rn(-q1, B.h, A.h)), A.l);
+    const float q2 = __fmul_rn(r, y);
+    const float s = __fadd_rn(q1, q2);
+    const float err = __fsub_rn(q2, __fsub_rn(s, q1)), ae = fabsf(err);
+    const float half = __uint_as_float((__float_as_uint(s) & 0x7F800000u) - (24u << 23));  // of the gap to the next float
+    const bool power = (__float_as_uint(s) & 0x7FFFFFu) == 0u;  // the gap below is half of it
+    if (ae <= half * (power ? 0.49999237f : 0.99999237f)) return s;
+    const float gap = power && ae < 0.75f * half && (err < 0.0f) != (s < 0.0f) ? 0.5f * half : half;
+    const double mid = (double)s + (double)copysignf(gap, err);
+    if (fma(-mid, b, a) == 0.0) return __double2float_rn(mid);
+    return __double2float_rn(a / b);
 }
 
-// FP32 node records and prefix mass fractions: FP64 quotients rounded once to FP32. FP64 division
-// is slow on this GPU, and a loop of them in one lane holds its whole warp, so each node computes
-// only its own: its centre of mass (a single point, whose quotient m x / m is x itself, copies its
-// own record) and its own fraction among its siblings, the prefix sum of their masses in sibling
-// order over the parent's mass (the same sum, in the same order, as k_aggregate's). (A product
-// with 1 / m is not a substitute for the quotient: small nodes of equal weights often sit exactly
-// on an FP32 rounding midpoint, where the product's last-bit error changes the rounding.)
-__global__ void k_pack(const double* __restrict__ agg, const int32_t* __restrict__ fc,
-                       const uint32_t* __restrict__ meta, const int32_t* __restrict__ nb,
-                       const int32_t* __restrict__ parent, const float4* __restrict__ spw,
-                       const float4* __restrict__ snrm, const TreeCtrl* __restrict__ ctrl, float4* __restrict__ pm,
-                       float4* __restrict__ dip, float4* __restrict__ pmd, float* __restrict__ cdf)
+// __double2float_rn(x) by integer operations
+__device__ __forceinline__ float narrow(double x)
 {
-    const int32_t N = ctrl->depth_base[ctrl->max_depth + 1];
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < N; v += (int64_t)gridDim.x * blockDim.x) {
-        if (meta_kind(meta[v]) == kPoint) {
-            const float4 p = spw[nb[v]];
-            pm[v] = p;
-            if (dip) {  // m n: one FP32 rounding of the exact product, as the FP64 sum rounded to FP32
-                const float4 q = snrm ? snrm[nb[v]] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                dip[v] = make_float4(__fmul_rn(p.w, q.x), __fmul_rn(p.w, q.y), __fmul_rn(p.w, q.z), 0.0f);
-            }
-        } else {
-            const double* a = agg + 8 * v;
-            const double m = a[0];
-            pm[v] = make_float4(__double2float_rn(a[1] / m), __double2float_rn(a[2] / m),
-                                __double2float_rn(a[3] / m), __double2float_rn(m));
-            if (dip) dip[v] = make_float4(__double2float_rn(a[4]), __double2float_rn(a[5]), __double2float_rn(a[6]), 0.0f);
-        }
-        if (pmd) {  // the same two records side by side, for one 32-byte load
-            pmd[2 * v] = pm[v];
-            pmd[2 * v + 1] = dip[v];
-        }
-        if (v == 0) { cdf[0] = 1.0f; continue; }
-        const int32_t par = parent[v];
-        const int32_t f = fc[par];
-        const int32_t last = f + (int32_t)meta_nchild(meta[par]) - 1;
-        if (v >= last) { cdf[v] = 1.0f; continue; }
-        double pre = 0.0;
-        for (int32_t k = f; k <= v; ++k) pre += agg[8 * (int64_t)k];
-        cdf[v] = __double2float_rn(pre / agg[8 * (int64_t)par]);
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    if (((hi >> 20) & 0x7FFu) - 898u > 250u) return ((hi << 1) | lo) == 0u ? __uint_as_float(hi) : __double2float_rn(x);
+    const uint32_t t = (((hi & 0x7FFFFFFFu) - 0x38000000u) << 3) | lo >> 29, rest = lo << 3;  // 24 bits, and the 29 below
+    const uint32_t up = rest > 0x80000000u || (rest == 0x80000000u && (t & 1u)) ? 1u : 0u;
+    return __uint_as_float((hi & 0x80000000u) | (t + up));
+}
+
+constexpr int kAggThreads = 256, kAggWarps = kAggThreads / 32, kAggBlocks = 4;  // blocks resident on an SM
+constexpr int kAggNodes = 4;      // nodes to a warp, eight lanes each
+constexpr int kAggChildren = 64;  // prefix sums kept per node (a leaf of duplicates may have more children)
+
+struct AggScratch {
+    double pre[kAggNodes][kAggChildren];
+    float cdf[kAggNodes][kAggChildren];
+};
+
+struct AggArrays {
+    BuildArrays B;
+    const float4* spw;
+    const float4* snrm;
+    double* agg;
+    float4* pm;
+    float4* dip;
+    float4* pmd;
+    float* cdf;
+    uint8_t* gd;
+    unsigned* barrier;  // blocks that are through with a generation, over all of them; zero at first
+};
+
+// Every block's writes of the generations so far are visible to every block. The grid is a cooperative
+// launch, so all its blocks are running; the wait is bounded all the same.
+__device__ __forceinline__ void grid_barrier(const AggArrays& A, unsigned target)
+{
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(A.barrier, 1u);
+        volatile unsigned* at = A.barrier;
+        int spin = 0;
+        while (*at < target)
+            if (++spin > kSpinLimit) { A.B.ctrl->error = kErrorTimeout; break; }
+        __threadfence();
     }
+    __syncthreads();
 }
 
 // The child pick's guide table (Chen and Asau's method), one entry per child slot: for slot j of
@@ -1039,23 +1049,169 @@ __global__ void k_pack(const double* __restrict__ agg, const int32_t* __restrict
 // children, where u_j = ceil(j 2^24 / nc) 2^-24 is the smallest 24-bit draw whose slot
 // floor(u nc) is j. It is stored at the child's own id (first child + j): every node but the root
 // fills one slot of its parent. That count never decreases with u, so a pick with draw u in slot
-// j that scans up from the entry finds the same child as counting all prefix fractions.
-__global__ void k_guide(const int32_t* __restrict__ fc, const uint32_t* __restrict__ meta,
-                        const int32_t* __restrict__ parent, const float* __restrict__ cdf,
-                        const TreeCtrl* __restrict__ ctrl, uint8_t* __restrict__ gd)
+// j that scans up from the entry finds the same child as counting all prefix fractions. The fractions
+// never decrease, so the count is a bisection.
+__device__ __forceinline__ uint8_t guide_entry(const float* cdf, uint32_t nc, uint32_t j)
 {
-    const int32_t N = ctrl->depth_base[ctrl->max_depth + 1];
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < N; v += (int64_t)gridDim.x * blockDim.x) {
-        if (v == 0) { gd[0] = 0; continue; }
-        const int32_t par = parent[v];
-        const int32_t f = fc[par];
-        const uint32_t nc = meta_nchild(meta[par]);
-        const uint32_t j = (uint32_t)(v - f);
-        const uint32_t mj = (uint32_t)((((uint64_t)j << 24) + nc - 1u) / nc);  // < 2^24: exact in FP32
-        const float uj = (float)mj * 5.9604644775390625e-8f;
-        uint32_t cnt = 0;
-        for (uint32_t i = 0; i + 1u < nc; ++i) cnt += cdf[f + i] <= uj ? 1u : 0u;
-        gd[v] = (uint8_t)cnt;
+    const uint32_t mj = (uint32_t)((((uint64_t)j << 24) + nc - 1u) / nc);  // < 2^24: exact in FP32
+    const float uj = (float)mj * 5.9604644775390625e-8f;
+    uint32_t lo = 0, hi = nc - 1u;
+    while (lo < hi) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (cdf[mid] <= uj) lo = mid + 1u;
+        else hi = mid;
+    }
+    return (uint8_t)lo;
+}
+
+// The records of the node of one group of eight lanes (v < 0: none): its sums in order, then what follows
+// from them. Every lane of the warp comes here.
+__device__ __forceinline__ void aggregate_node(const AggArrays& A, AggScratch& S, int32_t v)
+{
+    const int lane = threadIdx.x & 31, sub = lane & 7, group = lane >> 3, first = lane & 24;
+    int32_t f = 0;
+    int nc = 0;
+    if (v >= 0) {
+        f = A.B.fc[v];
+        nc = A.B.last_child[v] - f + 1;
+    }
+    const int wide = __reduce_max_sync(0xFFFFFFFFu, nc);
+    double sum = 0.0;
+    constexpr int kAhead = 8;
+    double next[kAhead];
+#pragma unroll
+    for (int k = 0; k < kAhead; ++k) next[k] = k < nc ? __ldcg(&A.agg[8 * (int64_t)(f + k) + sub]) : 0.0;
+    for (int c0 = 0; c0 < wide; c0 += kAhead) {
+        double x[kAhead];
+#pragma unroll
+        for (int k = 0; k < kAhead; ++k) {
+            x[k] = next[k];
+            const int c = c0 + kAhead + k;
+            next[k] = c < nc ? __ldcg(&A.agg[8 * (int64_t)(f + c) + sub]) : 0.0;
+        }
+#pragma unroll
+        for (int k = 0; k < kAhead; ++k) {
+            if (c0 + k >= nc) continue;
+            // 0 + x of the first child is x, but for the sign of a zero
+            if (c0 + k == 0) sum = __double_as_longlong(x[0]) == (long long)0x8000000000000000ull ? 0.0 : x[0];
+            else sum += x[k];
+            if (sub == 0 && c0 + k < kAggChildren) S.pre[group][c0 + k] = sum;
+        }
+    }
+    __syncwarp();
+    const double m = __shfl_sync(0xFFFFFFFFu, sum, first);
+    const Split M = split(m);
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(M.h));
+    const float r = v >= 0 && sub >= 1 && sub <= 3 ? quotient_rn(sum, m, M, y) : narrow(sum);
+    float out[7];  // m, centre, dipole
+#pragma unroll
+    for (int k = 0; k < 7; ++k) out[k] = __shfl_sync(0xFFFFFFFFu, r, first + k);
+    if (v >= 0) {
+        A.agg[8 * (int64_t)v + sub] = sub == 7 ? 0.0 : sum;
+        const float4 pm = make_float4(out[1], out[2], out[3], out[0]), dp = make_float4(out[4], out[5], out[6], 0.0f);
+        if (sub == 0) A.pm[v] = pm;
+        if (sub == 1 && A.dip) A.dip[v] = dp;
+        if (sub == 2 && A.pmd) A.pmd[2 * (int64_t)v] = pm;
+        if (sub == 3 && A.pmd) A.pmd[2 * (int64_t)v + 1] = dp;
+        if (sub == 4) {
+            if ((uint32_t)nc > kMaxChildren) A.B.ctrl->error = kErrorChildren;
+            A.B.meta[v] |= (uint32_t)nc & kMaxChildren;
+        }
+        if (nc <= kAggChildren) {
+            for (int c = sub; c < nc; c += 8) {
+                const float q = c == nc - 1 ? 1.0f : quotient_rn(S.pre[group][c], m, M, y);
+                S.cdf[group][c] = q;
+                A.cdf[f + c] = q;
+            }
+        }
+    }
+    __syncwarp();
+    if (v >= 0 && nc <= kAggChildren)
+        for (int j = sub; j < nc; j += 8) A.gd[f + j] = guide_entry(S.cdf[group], (uint32_t)nc, (uint32_t)j);
+    // a leaf of many duplicates: the prefix sums once more, 64 children at a time
+    if (wide > kAggChildren) {
+        const bool mine = v >= 0 && nc > kAggChildren;
+        double pre = 0.0;
+        for (int c0 = 0; c0 < wide; c0 += kAggChildren) {
+            __syncwarp();
+            if (mine && sub == 0)
+                for (int c = c0; c < nc && c < c0 + kAggChildren; ++c) {
+                    pre += __ldcg(&A.agg[8 * (int64_t)(f + c)]);
+                    S.pre[group][c - c0] = pre;
+                }
+            __syncwarp();
+            if (mine)
+                for (int c = c0 + sub; c < nc && c < c0 + kAggChildren; c += 8)
+                    A.cdf[f + c] = c == nc - 1 ? 1.0f : quotient_rn(S.pre[group][c - c0], m, M, y);
+        }
+        __threadfence_block();
+        __syncwarp();
+        if (mine)
+            for (int j = sub; j < nc; j += 8) A.gd[f + j] = guide_entry(A.cdf + f, (uint32_t)nc, (uint32_t)j);
+    }
+    __syncwarp();
+}
+
+__global__ void __launch_bounds__(kAggThreads, kAggBlocks) k_aggregate(AggArrays A)
+{
+    __shared__ AggScratch s_scratch[kAggWarps];
+    AggScratch& S = s_scratch[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    const TreeCtrl* ctrl = A.B.ctrl;
+    const int deepest = ctrl->max_depth;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {  // the root is nobody's child
+        A.cdf[0] = 1.0f;
+        A.gd[0] = 0;
+    }
+    for (int gen = deepest; gen >= 0; --gen) {
+        const int32_t lo = ctrl->depth_base[gen], hi = ctrl->depth_base[gen + 1];
+        // up to 32 ids to a warp, fewer where the generation has fewer than 32 to each warp of the grid:
+        // a warp takes four nodes at a time, one four after the other
+        const int warps = (int)gridDim.x * kAggWarps;
+        int span = 32;
+        while (span > kAggNodes && (int64_t)(hi - lo) * 2 <= (int64_t)span * warps) span >>= 1;
+        for (int64_t b = lo + (int64_t)span * (blockIdx.x * kAggWarps + (threadIdx.x >> 5)); b < hi; b += (int64_t)span * warps) {
+            const int32_t v = (int32_t)b + lane;
+            const bool live = lane < span && b + lane < hi;
+            const bool point = live && meta_kind(A.B.meta[v]) == kPoint;
+            unsigned nodes = __ballot_sync(0xFFFFFFFFu, live && !point);
+            if (point) {
+                const int32_t i = A.B.nb[v];
+                const float4 p = A.spw[i];
+                const double w = widen(p.w);
+                double2* d = reinterpret_cast<double2*>(A.agg + 8 * (int64_t)v);
+                d[0] = make_double2(w, w * widen(p.x));
+                d[1] = make_double2(w * widen(p.y), w * widen(p.z));
+                A.pm[v] = p;
+                float4 q = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                if (A.snrm) {
+                    q = A.snrm[i];
+                    d[2] = make_double2(w * widen(q.x), w * widen(q.y));
+                    d[3] = make_double2(w * widen(q.z), 0.0);
+                } else {
+                    d[2] = d[3] = make_double2(0.0, 0.0);
+                }
+                if (A.dip) {  // m n: one FP32 rounding of the exact product, as the FP64 sum rounded to FP32
+                    const float4 dp = make_float4(__fmul_rn(p.w, q.x), __fmul_rn(p.w, q.y), __fmul_rn(p.w, q.z), 0.0f);
+                    A.dip[v] = dp;
+                    if (A.pmd) {  // the same two records side by side, for one 32-byte load
+                        A.pmd[2 * (int64_t)v] = p;
+                        A.pmd[2 * (int64_t)v + 1] = dp;
+                    }
+                }
+            }
+            while (nodes) {
+                int32_t mine = -1;
+#pragma unroll
+                for (int k = 0; k < kAggNodes; ++k) {
+                    if (nodes && (lane >> 3) == k) mine = (int32_t)b + __ffs(nodes) - 1;
+                    nodes &= nodes - 1u;
+                }
+                aggregate_node(A, S, mine);
+            }
+        }
+        if (gen) grid_barrier(A, (unsigned)(deepest - gen + 1) * gridDim.x);
     }
 }
 
@@ -1170,7 +1326,7 @@ cudaError_t build_tree(sbh_tree* T, DeviceTree& D, const uint8_t* lcp, int max_l
     SBH_TRY(guard.alloc(&B.mask, n * sizeof(uint32_t)));
     SBH_TRY(guard.alloc(&B.last_child, D.cap * sizeof(int32_t)));
     SBH_TRY(guard.alloc(&B.count, (kMaxDepth + 1) * tiles * sizeof(int32_t)));
-    SBH_TRY(guard.alloc(&B.from_left, 2 * tiles * sizeof(uint32_t)));
+    SBH_TRY(guard.alloc(&B.from_left, (2 * tiles + 1) * sizeof(uint32_t)));
     B.from_right = B.from_left + tiles;
 
     k_topo_runs<<<(unsigned)tiles, kTopoThreads, 0, s>>>(B);
@@ -1181,18 +1337,14 @@ cudaError_t build_tree(sbh_tree* T, DeviceTree& D, const uint8_t* lcp, int max_l
     note_launch();
     k_topo_emit<<<(unsigned)tiles, kTopoThreads, 0, s>>>(B);
     note_launch();
-    k_topo_children<<<grid_for(2 * n), kThreads, 0, s>>>(B);
-    note_launch();
-    const int generations = max_level + 2;  // levels strictly increase; points end one below the deepest level
     SBH_TRY(cudaGetLastError());
-    for (int gen = generations; gen >= 0; --gen) {
-        k_aggregate<<<grid_for(n), kThreads, 0, s>>>(D.fc, D.meta, D.nb, T->spw, T->snrm, D.ctrl, gen, D.agg);
-        note_launch();
-    }
-    k_pack<<<grid_for(2 * n), kThreads, 0, s>>>(D.agg, D.fc, D.meta, D.nb, D.parent, T->spw, T->snrm, D.ctrl, D.pm,
-                                                D.dip, D.pmd, D.cdf);
-    note_launch();
-    k_guide<<<grid_for(2 * n), kThreads, 0, s>>>(D.fc, D.meta, D.parent, D.cdf, D.ctrl, D.gd);
+    AggArrays A = {B, T->spw, T->snrm, D.agg, D.pm, D.dip, D.pmd, D.cdf, D.gd, reinterpret_cast<unsigned*>(B.from_right + tiles)};
+    int64_t blocks = (2 * n + kAggThreads - 1) / kAggThreads;
+    const int64_t resident = (int64_t)kAggBlocks * device_sm_count();
+    if (blocks > resident) blocks = resident;
+    void* args[] = {&A};
+    SBH_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_aggregate), dim3((unsigned)blocks),
+                                        dim3(kAggThreads), args, 0, s));
     note_launch();
     SBH_TRY(cudaGetLastError());
     D.built = true;
