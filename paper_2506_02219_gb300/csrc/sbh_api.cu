@@ -909,6 +909,7 @@ sbh_status sbh_tree_export(const sbh_tree* tree, int32_t which, const sbh_tree_e
     cp(buf->guide, D.gd, N * sizeof(uint8_t));
     uint32_t* meta_h = nullptr;
     double* agg_h = nullptr;
+    const int64_t A = D.agg_stride();
     float4* dip_h = nullptr;
     if (buf->nchild || buf->level) {
         meta_h = new (std::nothrow) uint32_t[N];
@@ -916,9 +917,9 @@ sbh_status sbh_tree_export(const sbh_tree* tree, int32_t which, const sbh_tree_e
         cp(meta_h, D.meta, N * sizeof(uint32_t));
     }
     if (buf->com_mass64) {
-        agg_h = new (std::nothrow) double[8 * N];
+        agg_h = new (std::nothrow) double[A * N];
         if (!agg_h) { delete[] meta_h; return fail(SBH_ENOMEM, "host allocation failed"); }
-        cp(agg_h, D.agg, 8 * N * sizeof(double));
+        cp(agg_h, D.agg, A * N * sizeof(double));
     }
     if (buf->dipole && D.dip) {
         dip_h = new (std::nothrow) float4[N];
@@ -931,10 +932,10 @@ sbh_status sbh_tree_export(const sbh_tree* tree, int32_t which, const sbh_tree_e
             if (meta_h && buf->nchild) buf->nchild[v] = (int32_t)sbh::meta_nchild(meta_h[v]);
             if (meta_h && buf->level) buf->level[v] = (int32_t)sbh::meta_level(meta_h[v]);
             if (agg_h) {
-                const double m = agg_h[8 * v];
-                buf->com_mass64[4 * v + 0] = agg_h[8 * v + 1] / m;
-                buf->com_mass64[4 * v + 1] = agg_h[8 * v + 2] / m;
-                buf->com_mass64[4 * v + 2] = agg_h[8 * v + 3] / m;
+                const double m = agg_h[A * v];
+                buf->com_mass64[4 * v + 0] = agg_h[A * v + 1] / m;
+                buf->com_mass64[4 * v + 1] = agg_h[A * v + 2] / m;
+                buf->com_mass64[4 * v + 2] = agg_h[A * v + 3] / m;
                 buf->com_mass64[4 * v + 3] = m;
             }
             if (buf->dipole) {

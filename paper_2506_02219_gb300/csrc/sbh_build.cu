@@ -948,8 +948,8 @@ __global__ void __launch_bounds__(kTopoThreads) k_topo_emit(BuildArrays B)
 //    its children get their prefix mass fractions and the slots of the child pick's guide table.
 //    What bounds it is the FP64 unit, two lanes to an SM: a warp's FP64 instruction holds it for 16
 //    clocks, however few lanes take part. So
-//      - eight lanes work on a node, one to each of the seven sums and the padding (a thread to a
-//        node issued seven additions a child, for the widest of 32 nodes);
+//      - a lane works on one sum of a node, eight lanes to a node with normals (one is padding) and four
+//        without (a thread to a node issued seven additions a child, for the widest of 32 nodes);
 //      - the prefix sums are the running sum of m (each child summed them anew);
 //      - quotients are FP32 pairs (quotient_rn), and conversions integer operations;
 //      - points, three nodes of four, take a lane each and only the products m p, m n.
@@ -1006,12 +1006,19 @@ __device__ __forceinline__ float narrow(double x)
 }
 
 constexpr int kAggThreads = 256, kAggWarps = kAggThreads / 32, kAggBlocks = 4;  // blocks resident on an SM
-constexpr int kAggNodes = 4;      // nodes to a warp, eight lanes each
 constexpr int kAggChildren = 64;  // prefix sums kept per node (a leaf of duplicates may have more children)
 
+template <bool NORMALS>
+struct AggShape {
+    static constexpr int kLanes = NORMALS ? 8 : 4;  // of a node, and doubles of its sums
+    static constexpr int kSums = NORMALS ? 7 : 4;
+    static constexpr int kNodes = 32 / kLanes;      // of a warp at a time
+};
+
+template <bool NORMALS>
 struct AggScratch {
-    double pre[kAggNodes][kAggChildren];
-    float cdf[kAggNodes][kAggChildren];
+    double pre[AggShape<NORMALS>::kNodes][kAggChildren];
+    float cdf[AggShape<NORMALS>::kNodes][kAggChildren];
 };
 
 struct AggArrays {
@@ -1064,11 +1071,13 @@ __device__ __forceinline__ uint8_t guide_entry(const float* cdf, uint32_t nc, ui
     return (uint8_t)lo;
 }
 
-// The records of the node of one group of eight lanes (v < 0: none): its sums in order, then what follows
-// from them. Every lane of the warp comes here.
-__device__ __forceinline__ void aggregate_node(const AggArrays& A, AggScratch& S, int32_t v)
+// The records of the node of one group of lanes (v < 0: none): its sums in order, then what follows from
+// them. Every lane of the warp comes here.
+template <bool NORMALS>
+__device__ __forceinline__ void aggregate_node(const AggArrays& A, AggScratch<NORMALS>& S, int32_t v)
 {
-    const int lane = threadIdx.x & 31, sub = lane & 7, group = lane >> 3, first = lane & 24;
+    constexpr int kLanes = AggShape<NORMALS>::kLanes, kSums = AggShape<NORMALS>::kSums;
+    const int lane = threadIdx.x & 31, sub = lane % kLanes, group = lane / kLanes, first = lane - sub;
     int32_t f = 0;
     int nc = 0;
     if (v >= 0) {
@@ -1080,14 +1089,14 @@ __device__ __forceinline__ void aggregate_node(const AggArrays& A, AggScratch& S
     constexpr int kAhead = 8;
     double next[kAhead];
 #pragma unroll
-    for (int k = 0; k < kAhead; ++k) next[k] = k < nc ? __ldcg(&A.agg[8 * (int64_t)(f + k) + sub]) : 0.0;
+    for (int k = 0; k < kAhead; ++k) next[k] = k < nc ? __ldcg(&A.agg[kLanes * (int64_t)(f + k) + sub]) : 0.0;
     for (int c0 = 0; c0 < wide; c0 += kAhead) {
         double x[kAhead];
 #pragma unroll
         for (int k = 0; k < kAhead; ++k) {
             x[k] = next[k];
             const int c = c0 + kAhead + k;
-            next[k] = c < nc ? __ldcg(&A.agg[8 * (int64_t)(f + c) + sub]) : 0.0;
+            next[k] = c < nc ? __ldcg(&A.agg[kLanes * (int64_t)(f + c) + sub]) : 0.0;
         }
 #pragma unroll
         for (int k = 0; k < kAhead; ++k) {
@@ -1104,22 +1113,25 @@ __device__ __forceinline__ void aggregate_node(const AggArrays& A, AggScratch& S
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(M.h));
     const float r = v >= 0 && sub >= 1 && sub <= 3 ? quotient_rn(sum, m, M, y) : narrow(sum);
-    float out[7];  // m, centre, dipole
+    float out[kSums];  // m, centre, dipole
 #pragma unroll
-    for (int k = 0; k < 7; ++k) out[k] = __shfl_sync(0xFFFFFFFFu, r, first + k);
+    for (int k = 0; k < kSums; ++k) out[k] = __shfl_sync(0xFFFFFFFFu, r, first + k);
     if (v >= 0) {
-        A.agg[8 * (int64_t)v + sub] = sub == 7 ? 0.0 : sum;
-        const float4 pm = make_float4(out[1], out[2], out[3], out[0]), dp = make_float4(out[4], out[5], out[6], 0.0f);
+        A.agg[kLanes * (int64_t)v + sub] = sub == kSums ? 0.0 : sum;
+        const float4 pm = make_float4(out[1], out[2], out[3], out[0]);
         if (sub == 0) A.pm[v] = pm;
-        if (sub == 1 && A.dip) A.dip[v] = dp;
-        if (sub == 2 && A.pmd) A.pmd[2 * (int64_t)v] = pm;
-        if (sub == 3 && A.pmd) A.pmd[2 * (int64_t)v + 1] = dp;
-        if (sub == 4) {
+        if constexpr (NORMALS) {
+            const float4 dp = make_float4(out[4], out[5], out[6], 0.0f);
+            if (sub == 1) A.dip[v] = dp;
+            if (sub == 4 && A.pmd) A.pmd[2 * (int64_t)v] = pm;
+            if (sub == 5 && A.pmd) A.pmd[2 * (int64_t)v + 1] = dp;
+        }
+        if (sub == 2) {
             if ((uint32_t)nc > kMaxChildren) A.B.ctrl->error = kErrorChildren;
             A.B.meta[v] |= (uint32_t)nc & kMaxChildren;
         }
         if (nc <= kAggChildren) {
-            for (int c = sub; c < nc; c += 8) {
+            for (int c = sub; c < nc; c += kLanes) {
                 const float q = c == nc - 1 ? 1.0f : quotient_rn(S.pre[group][c], m, M, y);
                 S.cdf[group][c] = q;
                 A.cdf[f + c] = q;
@@ -1128,7 +1140,7 @@ __device__ __forceinline__ void aggregate_node(const AggArrays& A, AggScratch& S
     }
     __syncwarp();
     if (v >= 0 && nc <= kAggChildren)
-        for (int j = sub; j < nc; j += 8) A.gd[f + j] = guide_entry(S.cdf[group], (uint32_t)nc, (uint32_t)j);
+        for (int j = sub; j < nc; j += kLanes) A.gd[f + j] = guide_entry(S.cdf[group], (uint32_t)nc, (uint32_t)j);
     // a leaf of many duplicates: the prefix sums once more, 64 children at a time
     if (wide > kAggChildren) {
         const bool mine = v >= 0 && nc > kAggChildren;
@@ -1137,26 +1149,28 @@ __device__ __forceinline__ void aggregate_node(const AggArrays& A, AggScratch& S
             __syncwarp();
             if (mine && sub == 0)
                 for (int c = c0; c < nc && c < c0 + kAggChildren; ++c) {
-                    pre += __ldcg(&A.agg[8 * (int64_t)(f + c)]);
+                    pre += __ldcg(&A.agg[kLanes * (int64_t)(f + c)]);
                     S.pre[group][c - c0] = pre;
                 }
             __syncwarp();
             if (mine)
-                for (int c = c0 + sub; c < nc && c < c0 + kAggChildren; c += 8)
+                for (int c = c0 + sub; c < nc && c < c0 + kAggChildren; c += kLanes)
                     A.cdf[f + c] = c == nc - 1 ? 1.0f : quotient_rn(S.pre[group][c - c0], m, M, y);
         }
         __threadfence_block();
         __syncwarp();
         if (mine)
-            for (int j = sub; j < nc; j += 8) A.gd[f + j] = guide_entry(A.cdf + f, (uint32_t)nc, (uint32_t)j);
+            for (int j = sub; j < nc; j += kLanes) A.gd[f + j] = guide_entry(A.cdf + f, (uint32_t)nc, (uint32_t)j);
     }
     __syncwarp();
 }
 
+template <bool NORMALS>
 __global__ void __launch_bounds__(kAggThreads, kAggBlocks) k_aggregate(AggArrays A)
 {
-    __shared__ AggScratch s_scratch[kAggWarps];
-    AggScratch& S = s_scratch[threadIdx.x >> 5];
+    __shared__ AggScratch<NORMALS> s_scratch[kAggWarps];
+    constexpr int kLanes = AggShape<NORMALS>::kLanes, kNodes = AggShape<NORMALS>::kNodes;
+    AggScratch<NORMALS>& S = s_scratch[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     const TreeCtrl* ctrl = A.B.ctrl;
     const int deepest = ctrl->max_depth;
@@ -1167,10 +1181,10 @@ __global__ void __launch_bounds__(kAggThreads, kAggBlocks) k_aggregate(AggArrays
     for (int gen = deepest; gen >= 0; --gen) {
         const int32_t lo = ctrl->depth_base[gen], hi = ctrl->depth_base[gen + 1];
         // up to 32 ids to a warp, fewer where the generation has fewer than 32 to each warp of the grid:
-        // a warp takes four nodes at a time, one four after the other
+        // a warp takes kNodes of them at a time
         const int warps = (int)gridDim.x * kAggWarps;
         int span = 32;
-        while (span > kAggNodes && (int64_t)(hi - lo) * 2 <= (int64_t)span * warps) span >>= 1;
+        while (span > kNodes && (int64_t)(hi - lo) * 2 <= (int64_t)span * warps) span >>= 1;
         for (int64_t b = lo + (int64_t)span * (blockIdx.x * kAggWarps + (threadIdx.x >> 5)); b < hi; b += (int64_t)span * warps) {
             const int32_t v = (int32_t)b + lane;
             const bool live = lane < span && b + lane < hi;
@@ -1180,19 +1194,15 @@ __global__ void __launch_bounds__(kAggThreads, kAggBlocks) k_aggregate(AggArrays
                 const int32_t i = A.B.nb[v];
                 const float4 p = A.spw[i];
                 const double w = widen(p.w);
-                double2* d = reinterpret_cast<double2*>(A.agg + 8 * (int64_t)v);
+                double2* d = reinterpret_cast<double2*>(A.agg + kLanes * (int64_t)v);
                 d[0] = make_double2(w, w * widen(p.x));
                 d[1] = make_double2(w * widen(p.y), w * widen(p.z));
                 A.pm[v] = p;
-                float4 q = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                if (A.snrm) {
-                    q = A.snrm[i];
+                if constexpr (NORMALS) {
+                    const float4 q = A.snrm[i];
                     d[2] = make_double2(w * widen(q.x), w * widen(q.y));
                     d[3] = make_double2(w * widen(q.z), 0.0);
-                } else {
-                    d[2] = d[3] = make_double2(0.0, 0.0);
-                }
-                if (A.dip) {  // m n: one FP32 rounding of the exact product, as the FP64 sum rounded to FP32
+                    // m n: one FP32 rounding of the exact product, as the FP64 sum rounded to FP32
                     const float4 dp = make_float4(__fmul_rn(p.w, q.x), __fmul_rn(p.w, q.y), __fmul_rn(p.w, q.z), 0.0f);
                     A.dip[v] = dp;
                     if (A.pmd) {  // the same two records side by side, for one 32-byte load
@@ -1204,11 +1214,11 @@ __global__ void __launch_bounds__(kAggThreads, kAggBlocks) k_aggregate(AggArrays
             while (nodes) {
                 int32_t mine = -1;
 #pragma unroll
-                for (int k = 0; k < kAggNodes; ++k) {
-                    if (nodes && (lane >> 3) == k) mine = (int32_t)b + __ffs(nodes) - 1;
+                for (int k = 0; k < kNodes; ++k) {
+                    if (nodes && lane / kLanes == k) mine = (int32_t)b + __ffs(nodes) - 1;
                     nodes &= nodes - 1u;
                 }
-                aggregate_node(A, S, mine);
+                aggregate_node<NORMALS>(A, S, mine);
             }
         }
         if (gen) grid_barrier(A, (unsigned)(deepest - gen + 1) * gridDim.x);
@@ -1267,7 +1277,7 @@ cudaError_t alloc_tree(DeviceTree& D, int64_t n, bool with_dip, bool with_skip, 
     SBH_TRY(dalloc((void**)&D.ne, cap * sizeof(int32_t), s));
     SBH_TRY(dalloc((void**)&D.parent, cap * sizeof(int32_t), s));
     if (with_skip) SBH_TRY(dalloc((void**)&D.skip, cap * sizeof(int32_t), s));
-    SBH_TRY(dalloc((void**)&D.agg, cap * 8 * sizeof(double), s));
+    SBH_TRY(dalloc((void**)&D.agg, cap * D.agg_stride() * sizeof(double), s));
     if (!D.ctrl) SBH_TRY(dalloc((void**)&D.ctrl, sizeof(TreeCtrl), s));
     return cudaSuccess;
 }
@@ -1343,7 +1353,8 @@ cudaError_t build_tree(sbh_tree* T, DeviceTree& D, const uint8_t* lcp, int max_l
     const int64_t resident = (int64_t)kAggBlocks * device_sm_count();
     if (blocks > resident) blocks = resident;
     void* args[] = {&A};
-    SBH_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_aggregate), dim3((unsigned)blocks),
+    const void* kernel = T->snrm ? reinterpret_cast<const void*>(k_aggregate<true>) : reinterpret_cast<const void*>(k_aggregate<false>);
+    SBH_TRY(cudaLaunchCooperativeKernel(kernel, dim3((unsigned)blocks),
                                         dim3(kAggThreads), args, 0, s));
     note_launch();
     SBH_TRY(cudaGetLastError());

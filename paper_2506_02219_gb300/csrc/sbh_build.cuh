@@ -25,9 +25,11 @@ struct DeviceTree {
     int32_t* parent = nullptr;
     int32_t* skip = nullptr;
     float4* rec = nullptr;   // [cap][2]: the walk records (8-ary tree; optional, see add_walk_records)
-    double* agg = nullptr;   // [cap][8] FP64: m, m p (3), m n (3), 0
+    double* agg = nullptr;   // [cap][4] FP64: m, m p (3); with normals [cap][8]: and m n (3), 0
     TreeCtrl* ctrl = nullptr;
     bool built = false;
+
+    int agg_stride() const { return dip ? 8 : 4; }
 
     TreeView view() const
     {
