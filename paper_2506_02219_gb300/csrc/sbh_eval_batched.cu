@@ -56,10 +56,10 @@ constexpr int multi_min_blocks() { return KIND == SBH_SMOOTHDIST ? SBH_SMOOTH_MI
 #endif
 // A subdomain's depth-0 decisions are taken in place by the warp (every lane at the same node)
 // when more than this many of its lanes may continue, else queued as decision tasks. Measured on
-// the estimator: 20 (16 to 24 within 1%). The smooth-distance, adjoint and learned instances
-// always queue them (32): their larger code ran slower with the decision inlined twice (smooth
-// distance 2.55 against 2.29 ms, adjoint 32.7 against 31.3), and queueing let the learned one keep
-// its state in registers.
+// the estimator: 20 (16 to 24 within 1%; smooth distance, multi-set: 8.67 ms against 8.98 with every
+// one queued, since its terms no longer carry the code for subnormal exponentials). The adjoint and learned
+// instances always queue them (32): their larger code ran slower with the decision inlined twice
+// (adjoint 32.7 against 31.3 ms), and queueing let the learned one keep its state in registers.
 #ifndef SBH_DEPTH0_QUEUE_MAX
 #define SBH_DEPTH0_QUEUE_MAX 20
 #endif
@@ -67,14 +67,8 @@ constexpr int multi_min_blocks() { return KIND == SBH_SMOOTHDIST ? SBH_SMOOTH_MI
 #ifndef SBH_GRAD_MIN_BLOCKS
 #define SBH_GRAD_MIN_BLOCKS 4
 #endif
-#ifndef SBH_DEPTH0_QUEUE_MAX_SMOOTH
-#define SBH_DEPTH0_QUEUE_MAX_SMOOTH 32
-#endif
-template <int KIND, bool LEARNED, bool GRAD>
-constexpr int depth0_queue_max()
-{
-    return (LEARNED || GRAD) ? 32 : (KIND == SBH_SMOOTHDIST ? SBH_DEPTH0_QUEUE_MAX_SMOOTH : SBH_DEPTH0_QUEUE_MAX);
-}
+template <bool LEARNED, bool GRAD>
+constexpr int depth0_queue_max() { return (LEARNED || GRAD) ? 32 : SBH_DEPTH0_QUEUE_MAX; }
 // resident blocks per SM of the learned-proposal instance: four (64 registers) fit its shared
 // memory without a stage and with 64-row scoring groups; 8-16% faster than three blocks of 80
 // registers with the stage and 128-row groups
@@ -643,11 +637,11 @@ __device__ __forceinline__ void smooth_vg(float4 pm, float3 q, float alpha, floa
     const float ir = rsqrt_ftz(fmaxf(r2, 1e-37f));
     const float d = r2 * ir;
     if (d < ref) {
-        const float f = __expf(-alpha * (ref - d));
+        const float f = exp_ftz(-alpha * (ref - d));
         v *= f; g[0] *= f; g[1] *= f; g[2] *= f;
         ref = d;
     }
-    const float t = wm * __expf(-alpha * (d - ref));
+    const float t = wm * exp_ftz(-alpha * (d - ref));
     v += t;
     if (r2 > 0.0f) {
         const float c = alpha * t * ir;  // alpha m exp(-alpha d) / d
@@ -712,13 +706,14 @@ __device__ __forceinline__ void swap_terms(const Params& P, const Stage& S, int3
         g[0] = w * (g[0] - go[0]); g[1] = w * (g[1] - go[1]); g[2] = w * (g[2] - go[2]);
     } else if constexpr (KIND == SBH_SMOOTHDIST) {
         const float a = P.kp.alpha;
+        // one child at a time: two, their distances formed first, ran 13% slower (multi-set 8.98 -> 10.17 ms)
         r = dist_fast(pT, q);
         v = -w * pT.w;
         for (int k = 0; k < nc; ++k) {
             const float4 pc = cp[k];
             const float d = dist_fast(pc, q);
-            if (d < r) { v *= __expf(-a * (r - d)); r = d; }
-            v = fmaf(w * pc.w, __expf(-a * (d - r)), v);
+            if (d < r) { v *= exp_ftz(-a * (r - d)); r = d; }
+            v = fmaf(w * pc.w, exp_ftz(-a * (d - r)), v);
         }
     } else {
         // two independent partial sums: two children in flight per iteration. Winding: each
@@ -769,12 +764,12 @@ __device__ __forceinline__ void add_to_query(const Params& P, WarpState<KIND>& W
         const float a = P.kp.alpha;
         float qr = W.ref[slot], qa = W.acc[slot];
         if (tr < qr) {
-            const float f = __expf(-a * (qr - tr));
+            const float f = exp_ftz(-a * (qr - tr));
             qa = qa * f + tot;
             if (GRAD) for (int c = 0; c < 3; ++c) qg[c] = qg[c] * f + tg[c];
             qr = tr;
         } else {
-            const float f = __expf(-a * (tr - qr));
+            const float f = exp_ftz(-a * (tr - qr));
             qa = fmaf(tot, f, qa);
             if (GRAD) for (int c = 0; c < 3; ++c) qg[c] = fmaf(tg[c], f, qg[c]);
         }
@@ -825,12 +820,12 @@ __device__ __forceinline__ void swap_batch(const Params& P, const Stage& S, Warp
             const float rs = __shfl_sync(peers, r, src);
             const float a = P.kp.alpha;
             if (rs < tr) {
-                const float f = __expf(-a * (tr - rs));
+                const float f = exp_ftz(-a * (tr - rs));
                 tot = tot * f + vs;
                 if (GRAD) for (int c = 0; c < 3; ++c) tg[c] = tg[c] * f + gs[c];
                 tr = rs;
             } else {
-                const float f = __expf(-a * (rs - tr));
+                const float f = exp_ftz(-a * (rs - tr));
                 tot = fmaf(vs, f, tot);
                 if (GRAD) for (int c = 0; c < 3; ++c) tg[c] = fmaf(gs[c], f, tg[c]);
             }
@@ -911,7 +906,7 @@ __device__ __forceinline__ void run_tile(const Params& P, const PhiloxRoundKeys&
                 live = !certain_stop(P.rr, unit24(x.y), da, Ba, W.slack);
             }
             const unsigned push = __ballot_sync(0xFFFFFFFFu, live);
-            constexpr int kQueueMax = depth0_queue_max<KIND, LEARNED, GRAD>();
+            constexpr int kQueueMax = depth0_queue_max<LEARNED, GRAD>();
             if (kQueueMax < 0 || (kQueueMax < 32 && __popc(push) > kQueueMax)) {
                 decide<KIND, LEARNED, true>(P, K, S, W, sdiam, live, a, x.x, x.y, x.z, x.w, tag, 1.0f, da, wa, wa,
                                             d_tail, s_tail);
@@ -954,12 +949,12 @@ __device__ __forceinline__ void run_tile(const Params& P, const PhiloxRoundKeys&
             if (GRAD) { sg[0] = qg[0]; sg[1] = qg[1]; sg[2] = qg[2]; }
             // merge the swap sum into the control-variate sum
             if (r < ex.ref) {
-                const float f = __expf(-a * (ex.ref - r));
+                const float f = exp_ftz(-a * (ex.ref - r));
                 ex.acc = ex.acc * f + v;
                 if (GRAD) for (int c = 0; c < 3; ++c) cg[c] = cg[c] * f + sg[c];
                 ex.ref = r;
             } else {
-                const float f = __expf(-a * (r - ex.ref));
+                const float f = exp_ftz(-a * (r - ex.ref));
                 ex.acc = fmaf(v, f, ex.acc);
                 if (GRAD) for (int c = 0; c < 3; ++c) cg[c] = fmaf(sg[c], f, cg[c]);
             }
