@@ -1108,6 +1108,8 @@ static cudaError_t launch_batched_impl(const TreeView& T, const TreeCtrl& host_c
     P.sampling = o.sampling; P.rr = o.rr; P.coherent = o.seed_mode; P.raw_sum = o.raw_sum; P.out = out;
     P.mlpw = (const __half*)mlp_half; P.near = near;
     const int64_t tiles = (nq + 31) / 32;
+    // (fewer warps to a block, to spread a few tiles over more SMs, is slower: the warps of a block find in
+    // L1 what the others read. 4,096 queries in 128 blocks of one warp: 214 us against 156 in 16 of eight)
     int64_t blocks = (tiles + kWarpsPerBlock - 1) / kWarpsPerBlock;
     const int64_t grid_cap = (int64_t)device_sm_count() * SBH_GRID_BLOCKS_PER_SM;
     if (blocks > grid_cap) blocks = grid_cap;
