@@ -287,6 +287,10 @@ __global__ void __launch_bounds__(32 * kTrainWarps, 3) k_loss_grad(const float* 
     __shared__ float s_d[kTrainWarps][kMaxLearnedChildren];   // exp(score), then d loss / d score
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (threadIdx.x < kH) s_w3[threadIdx.x] = wg[ow3 + threadIdx.x];
+    // W2 through shared memory (rows of 33: a row to a lane without bank conflicts), where the activations
+    // go later
+    float* s_w2 = reinterpret_cast<float*>(s_act);
+    for (int i = threadIdx.x; i < kH * kH; i += blockDim.x) s_w2[(i / kH) * (kH + 1) + i % kH] = wg[oW2 + i];
     __syncthreads();
     float4* h1s = s_act + (size_t)warp * 2 * (kActFloats / 4);
     float4* h2s = h1s + kActFloats / 4;  // of the second layer, then its gradient
@@ -300,9 +304,10 @@ __global__ void __launch_bounds__(32 * kTrainWarps, 3) k_loss_grad(const float* 
 #pragma unroll
     for (int k = 0; k < kH; ++k) {
         gW2[k] = 0.0f;
-        w2row[k] = wg[oW2 + lane * kH + k];
-        w2col[k] = wg[oW2 + k * kH + lane];
+        w2row[k] = s_w2[lane * (kH + 1) + k];
+        w2col[k] = s_w2[k * (kH + 1) + lane];
     }
+    __syncthreads();
     const float b1 = wg[ob1 + lane], b2 = wg[ob2 + lane], w3 = wg[ow3 + lane], b3 = wg[ob3];
     const int mine = lane & 3;  // this lane's unit within its group of four
 
