@@ -56,10 +56,11 @@ constexpr int multi_min_blocks() { return KIND == SBH_SMOOTHDIST ? SBH_SMOOTH_MI
 #endif
 // A subdomain's depth-0 decisions are taken in place by the warp (every lane at the same node)
 // when more than this many of its lanes may continue, else queued as decision tasks. Measured on
-// the estimator: 20 (16 to 24 within 1%; smooth distance, multi-set: 8.67 ms against 8.98 with every
-// one queued, since its terms no longer carry the code for subnormal exponentials). The adjoint and learned
-// instances always queue them (32): their larger code ran slower with the decision inlined twice
-// (adjoint 32.7 against 31.3 ms), and queueing let the learned one keep its state in registers.
+// the estimator: 20 (16 to 24 within 1%). The adjoint and learned instances always queue them (32): their
+// larger code ran slower with the decision inlined twice (adjoint 32.7 against 31.3 ms), and queueing let
+// the learned one keep its state in registers. The smooth distance queues them too: 20 is 3% faster
+// (multi-set 8.68 against 8.98 ms), but the order in which a query's swaps are added then differs, and its
+// sums cancel so far that results moved by up to 2e-3 where they are nearest to zero.
 #ifndef SBH_DEPTH0_QUEUE_MAX
 #define SBH_DEPTH0_QUEUE_MAX 20
 #endif
@@ -67,8 +68,8 @@ constexpr int multi_min_blocks() { return KIND == SBH_SMOOTHDIST ? SBH_SMOOTH_MI
 #ifndef SBH_GRAD_MIN_BLOCKS
 #define SBH_GRAD_MIN_BLOCKS 4
 #endif
-template <bool LEARNED, bool GRAD>
-constexpr int depth0_queue_max() { return (LEARNED || GRAD) ? 32 : SBH_DEPTH0_QUEUE_MAX; }
+template <int KIND, bool LEARNED, bool GRAD>
+constexpr int depth0_queue_max() { return (LEARNED || GRAD || KIND == SBH_SMOOTHDIST) ? 32 : SBH_DEPTH0_QUEUE_MAX; }
 // resident blocks per SM of the learned-proposal instance: four (64 registers) fit its shared
 // memory without a stage and with 64-row scoring groups; 8-16% faster than three blocks of 80
 // registers with the stage and 128-row groups
@@ -906,7 +907,7 @@ __device__ __forceinline__ void run_tile(const Params& P, const PhiloxRoundKeys&
                 live = !certain_stop(P.rr, unit24(x.y), da, Ba, W.slack);
             }
             const unsigned push = __ballot_sync(0xFFFFFFFFu, live);
-            constexpr int kQueueMax = depth0_queue_max<LEARNED, GRAD>();
+            constexpr int kQueueMax = depth0_queue_max<KIND, LEARNED, GRAD>();
             if (kQueueMax < 0 || (kQueueMax < 32 && __popc(push) > kQueueMax)) {
                 decide<KIND, LEARNED, true>(P, K, S, W, sdiam, live, a, x.x, x.y, x.z, x.w, tag, 1.0f, da, wa, wa,
                                             d_tail, s_tail);
