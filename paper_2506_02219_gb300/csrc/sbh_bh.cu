@@ -10,9 +10,13 @@
 //
 // What bounds the walk is the instructions of a step and the chain from one node's record to the
 // next one's address, so a step is kept short:
-//   - one 32-byte record per node holds its centre, mass, first child, skip and level
-//     (k_walk_records): one load, where position, meta word and link were three, the last of them
-//     behind the test;
+//   - one 32-byte record per node (k_walk_records) holds its centre, mass, first child, skip and level, where
+//     position, meta word and link were three loads, the last of them behind the test. All lanes of a
+//     warp read one node, and each word delivered to 32 lanes is a wavefront of the L1 data path, which ran
+//     at 83% with that record and the dipole: in trees with normals the record is the winding walk's,
+//     with the dipole sum for the mass, and the first child is read when a node is opened, one in
+//     eight (5.06 -> 4.85 ms; without normals, where the record is one load, that was slower). The
+//     other kernels walk a tree with normals by its arrays;
 //   - the far-field ratio is a correctly rounded root and quotient, and monotone in the squared
 //     distance, so the test is one comparison with the smallest squared distance that passes it at
 //     the node's level (open_limit): the same decisions without either operation.
@@ -33,9 +37,8 @@
 namespace sbh {
 
 // The node's term from d = p - q; r2 is its squared length as the test has it (every operation rounded),
-// which the Coulomb term takes too. The other two are singular at a source, or alpha times as
-// sensitive, and take the fused sum. The winding term is times 4 pi (the sum is scaled once), with the
-// squared length clamped as in term_winding_4pi.
+// which the Coulomb term takes too. The winding term is singular at a source and the smooth distance's
+// alpha times as sensitive: they take the fused sum, as before.
 template <int KIND>
 __device__ __forceinline__ void bh_add(float4 p, float4 dp, float3 d, float r2, const KernelParams& kp, float& acc,
                                        ExpAcc& ex)
@@ -43,8 +46,10 @@ __device__ __forceinline__ void bh_add(float4 p, float4 dp, float3 d, float r2, 
     if constexpr (KIND == SBH_COULOMB) {
         acc = fmaf(p.w, rsqrt_ftz(__fadd_rn(r2, kp.eps2)), acc);
     } else if constexpr (KIND == SBH_WINDING) {
-        const float ir = rsqrt_ftz(fmaxf(fmaf(d.x, d.x, fmaf(d.y, d.y, d.z * d.z)), kMinNormal));
-        acc = fmaf(fmaf(d.x, dp.x, fmaf(d.y, dp.y, d.z * dp.z)) * ir, ir * ir, acc);
+        const float f2 = fmaf(d.x, d.x, fmaf(d.y, d.y, d.z * d.z));
+        const float ir = rsqrt_ftz(f2);
+        const float t = fmaf(d.x, dp.x, fmaf(d.y, dp.y, d.z * dp.z)) * (ir * ir * ir) * kInv4Pi;
+        acc += f2 >= kMinNormal ? t : 0.0f;
     } else if constexpr (KIND == SBH_AFFINE) {
         acc = fmaf(p.w, 1.0f + fmaf(kp.g[0], d.x, fmaf(kp.g[1], d.y, kp.g[2] * d.z)), acc);
     } else {
@@ -95,7 +100,7 @@ __device__ float open_limit(float B, float beta)
 //              each other (sorted), whose nodes are mostly the same.
 enum { kAlone = 0, kVote = 1, kTogether = 2 };
 
-// REC: the walk records are there (without the memory for them a node is read from its three arrays)
+// REC: the kernel's walk records are there (else a node is read from the tree's arrays)
 template <int KIND, int MODE, bool REC>
 __global__ void __launch_bounds__(256) k_bh_eval(TreeView T, const float4* __restrict__ rec,
                                                  const float* __restrict__ Q, int64_t nq, KernelParams kp, float beta,
@@ -125,18 +130,31 @@ __global__ void __launch_bounds__(256) k_bh_eval(TreeView T, const float4* __res
         if (MODE != kAlone || active) {
             while (v >= 0 && budget-- > 0) {
                 float4 p;
-                int32_t first = 0, skip = 0;
+                int32_t skip = 0, first = 0;
                 float limit;
                 bool point;
+                float4 dp;
                 if constexpr (REC) {
-                    float4 r;
-                    ld_pmd(rec, v, p, r);
-                    first = __float_as_int(r.x);
-                    skip = __float_as_int(r.y);
-                    limit = *reinterpret_cast<const float*>(reinterpret_cast<const char*>(s_limit) + __float_as_int(r.z));
-                    point = first < 0;
+                    const float4* at = rec + 2 * (int64_t)v;
+                    int lvl;
+                    if constexpr (KIND == SBH_WINDING) {
+                        p = __ldg(at);
+                        dp = __ldg(at + 1);
+                        lvl = __float_as_int(p.w);
+                        skip = __float_as_int(dp.w);
+                        point = lvl == kWalkPoint;
+                    } else {
+                        float4 r;
+                        ld_pmd(rec, v, p, r);
+                        first = __float_as_int(r.x);
+                        skip = __float_as_int(r.y);
+                        lvl = __float_as_int(r.z);
+                        point = first < 0;
+                    }
+                    limit = *reinterpret_cast<const float*>(reinterpret_cast<const char*>(s_limit) + lvl);
                 } else {
                     p = __ldg(&T.pm[v]);
+                    if constexpr (KIND == SBH_WINDING) dp = __ldg(&T.dip[v]);
                     const uint32_t m = __ldg(&T.meta[v]);
                     limit = s_limit[meta_level(m)];
                     point = meta_kind(m) == kPoint;
@@ -147,22 +165,19 @@ __global__ void __launch_bounds__(256) k_bh_eval(TreeView T, const float4* __res
                 bool use = point || r2 >= limit;
                 if (MODE == kVote) use = __all_sync(0xFFFFFFFFu, use || !active);
                 const bool mine = MODE == kTogether ? own == v : active;
-                if (use && mine) bh_add<KIND>(p, KIND == SBH_WINDING ? __ldg(&T.dip[v]) : p, d, r2, kp, acc, ex);
-                if constexpr (MODE == kTogether) {
-                    if (mine) own = use ? skip : first;
-                    v = __any_sync(0xFFFFFFFFu, mine && !use) ? first : skip;
-                } else if (use) {
-                    v = REC ? skip : __ldg(&T.skip[v]);
-                } else {
-                    v = REC ? first : __ldg(&T.fc[v]);
-                }
+                if (use && mine) bh_add<KIND>(p, KIND == SBH_WINDING ? dp : p, d, r2, kp, acc, ex);
+                if constexpr (!REC) skip = use ? __ldg(&T.skip[v]) : 0;
+                const bool open = MODE == kTogether ? __any_sync(0xFFFFFFFFu, mine && !use) : !use;
+                if (!REC || KIND == SBH_WINDING) first = open ? __ldg(&T.fc[v]) : 0;
+                if (MODE == kTogether && mine) own = use ? skip : first;
+                v = open ? first : skip;
             }
         }
         if (v >= 0) acc = ex.acc = __int_as_float(0x7FC00000);  // walk did not finish: NaN
         if (active) {
             if constexpr (KIND == SBH_SMOOTHDIST)
                 out[j] = ex.acc > 0.0f ? ex.ref - __logf(ex.acc) / kp.alpha : __int_as_float(0x7F800000);
-            else out[j] = KIND == SBH_WINDING ? acc * kInv4Pi : acc;
+            else out[j] = acc;
         }
     }
 }
@@ -209,9 +224,11 @@ cudaError_t launch_bh_eval(const DeviceTree& D, const float* Q, int64_t nq, cons
     int64_t blocks = (nq + 255) / 256;
     const int64_t cap = (int64_t)device_sm_count() * 64;
     if (blocks > cap) blocks = cap;
-    BhLaunch L = {D.view(), D.rec, Q, nq, kp, beta, nullptr, nullptr, out, s, (unsigned)blocks};
+    // the walk records of a tree with normals are the winding walk's
+    const float4* rec = (kp.kind == SBH_WINDING) == (D.dip != nullptr) ? D.rec : nullptr;
+    BhLaunch L = {D.view(), rec, Q, nq, kp, beta, nullptr, nullptr, out, s, (unsigned)blocks};
     void* scratch = nullptr;
-    if (!warp_vote && D.rec && nq >= kSortFrom) {
+    if (!warp_vote && rec && nq >= kSortFrom) {
         const cudaError_t e = sort_queries(Q, nq, D.ctrl, &scratch, &L.order, &L.sort_error, s);
         if (e != cudaSuccess) return e;
     }

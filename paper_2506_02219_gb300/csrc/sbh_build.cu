@@ -1447,16 +1447,26 @@ cudaError_t build_tree(sbh_tree* T, DeviceTree& D, const uint8_t* lcp, int max_l
     return cudaSuccess;
 }
 
-// Node v's walk record: centre of mass and mass; first child (-1: a point), skip, level times 4, nothing
+// Node v's walk record: centre of mass and mass; first child (-1: a point), skip, level times 4, nothing. In
+// trees with normals: centre of mass and level times 4 (kWalkPoint: a point); dipole sum and skip.
 __global__ void __launch_bounds__(kThreads) k_walk_records(TreeView T, float4* __restrict__ rec)
 {
     const int32_t N = T.ctrl->n_nodes;
     for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < N; v += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t m = T.meta[v];
         const bool point = meta_kind(m) == kPoint;
-        rec[2 * v] = T.pm[v];
-        rec[2 * v + 1] = make_float4(__int_as_float(point ? -1 : T.fc[v]), __int_as_float(T.skip[v]),
-                                     __int_as_float(4 * (int)meta_level(m)), 0.0f);
+        const int lvl = 4 * (int)meta_level(m);
+        float4 p = T.pm[v];
+        float4 r;
+        if (T.dip) {
+            r = T.dip[v];
+            r.w = __int_as_float(T.skip[v]);
+            p.w = __int_as_float(point ? kWalkPoint : lvl);
+        } else {
+            r = make_float4(__int_as_float(point ? -1 : T.fc[v]), __int_as_float(T.skip[v]), __int_as_float(lvl), 0.0f);
+        }
+        rec[2 * v] = p;
+        rec[2 * v + 1] = r;
     }
 }
 

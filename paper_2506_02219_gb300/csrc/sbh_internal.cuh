@@ -64,6 +64,9 @@ struct TreeCtrl {
 constexpr int32_t kErrorChildren = 1;  // a node with more than kMaxChildren children
 constexpr int32_t kErrorTimeout = 2;   // a bounded wait gave up
 
+// A walk record's level field (level times 4) of a single point: past every level, in the opening limits' table
+constexpr int kWalkPoint = 4 * (kDiamLevels - 1);
+
 // Structure-of-arrays node storage of one tree (device pointers). Children of node v are the
 // contiguous ids fc[v] .. fc[v] + nchild - 1, in Morton order; generations are contiguous.
 struct TreeView {

@@ -65,6 +65,18 @@ def test_without_memory_for_the_records(sbh, vote):
     assert torch.equal(got, want)
 
 
+@pytest.mark.parametrize("vote", [False, True])
+@pytest.mark.parametrize("nq", [1000, 70001])
+def test_trees_with_normals_walk_alike(sbh, nq, vote):
+    """Normals change a tree's walk records, not its nodes or its masses."""
+    import torch
+    plain, p, _, _ = _tree(sbh)
+    other, _, _, v = _tree(sbh, normals=True)
+    Q = dev(np.random.default_rng(2).random((nq, 3), dtype=np.float32))
+    for kind in ("coulomb", "smoothdist"):
+        assert torch.equal(sbh.sbh_eval_bh(plain, Q, kind, 0.7, vote), sbh.sbh_eval_bh(other, Q, kind, 0.7, vote))
+
+
 @pytest.mark.parametrize("theta", [0.3, 0.5, 0.777, 1.0, 40.0])
 def test_opening_rule_is_the_rounded_quotient(sbh, theta):
     tree, p, _, _ = _tree(sbh, n=500, seed=3)
