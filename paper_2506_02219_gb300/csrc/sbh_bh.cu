@@ -183,9 +183,14 @@ __global__ void __launch_bounds__(256) k_bh_eval(TreeView T, const float4* __res
 }
 
 namespace {
-// Queries from which a walk without voting is worth the sort: it takes 45 us of launches and 20 us
-// per million queries.
-constexpr int64_t kSortFrom = 1 << 16;
+// Queries from which a walk without voting is sorted and walked together. The sort takes 30 us and 20 us per
+// million queries, and the fewer the queries, the further apart a warp's 32 are and the more nodes they
+// visit between them. theta 0.8, us sorted / not:
+//   2^18 sources, random queries   2^16: 440 / 167   2^18: 377 / 325   2^20: 658 / 1194
+//   2^20 sources, random queries   2^16: 549 / 179   2^18: 493 / 347   2^20: 791 / 1250
+//   2^18 sources, grid             2^16: 469 / 152   2^18: 352 / 245   2^20: 632 / 693
+//   2^14 sources, random queries   2^16: 192 / 113   2^18: 211 / 233   2^20: 463 / 935
+constexpr int64_t kSortFrom = 1 << 19;
 
 struct BhLaunch {
     TreeView T;

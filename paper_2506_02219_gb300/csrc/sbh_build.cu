@@ -4,14 +4,14 @@
 //   1. bounds + validation   per-axis min/max of the points (the root cube), counts of NaN/Inf
 //                            coordinates and of non-positive weights
 //   2. Morton codes          20-bit FP32 quantisation per axis, interleaved to 60 bits
-//   3. stable LSD radix sort (code, index), 8 passes of 8 bits, one kernel each
+//   3. stable LSD radix sort (code, index), 8 passes of 8 bits, one kernel each (one for all up to a tile)
 //   4. gather                points, weights and normals into Morton order
-//   5. topology              generation by generation: a node whose points span several cells one
-//                            level down has those runs as children; a run that stays inside one
-//                            cell collapses into its deepest split; a run of <= leaf_size points
-//                            (or at the deepest level) is a leaf whose children are its points
-//   6. aggregates            FP64 bottom-up sums of m, m p, m n per node, then packed to FP32
-//                            with the children's prefix mass fractions
+//   5. topology              a node whose points span several cells one level down has those runs
+//                            as children; a run that stays inside one cell collapses into its
+//                            deepest split; a run of <= leaf_size points (or at the deepest level)
+//                            is a leaf whose children are its points
+//   6. aggregates            FP64 bottom-up sums of m, m p, m n per node, FP32 records, the children's
+//                            prefix mass fractions and the child pick's guide table
 //
 // Node ids are generation-major (breadth-first): every node's children are contiguous, in
 // Morton order, and the top generations that every query reads sit at the front of each array.
@@ -1041,8 +1041,8 @@ __global__ void __launch_bounds__(kTopoThreads) k_topo_emit(BuildArrays B)
 //      - the prefix sums are the running sum of m (each child summed them anew);
 //      - quotients are FP32 pairs (quotient_rn), and conversions integer operations;
 //      - points, three nodes of four, take a lane each and only the products m p, m n.
-//    2^22 points: 1,090 us in 16 kernels -> 534 us; 4,096 points: 137 -> 39 us; the 8-ary and 64-ary
-//    trees of 2^18: 434 us in 42 kernels -> 190 us.
+//    2^22 points: 1,090 us in 16 kernels -> 389 us; 4,096 points: 137 -> 39 us; the 8-ary and 64-ary
+//    trees of 2^18: 434 us in 42 kernels -> 168 us (without normals).
 // ----------------------------------------------------------------------------------------------
 struct Split {
     float h, l;

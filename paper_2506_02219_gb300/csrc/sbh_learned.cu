@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(32 * kScoreWarps) k_scores(const __half* __res
 // the order (subdomain, sample, depth).
 //   A block is a query and a thread one of its paths: a path is a chain of dependent reads of a few
 // levels, and paths are all there is to run side by side. One thread to a query walked a few hundred
-// such chains one after the other: 650 us a pass for 256 queries, now 10.
+// such chains one after the other: 650 us a pass for 256 queries, now 8.
 // ------------------------------------------------------------------------------------------------
 constexpr int kVisitThreads = 256;
 
@@ -199,7 +199,7 @@ constexpr double value64_factor() { return KIND == SBH_WINDING ? 1.0 / (4.0 * 3.
 
 // A block to a decision set s = (query set_q[s], node set_node[s]), a warp to each of its children in
 // turn: rows set_off[s] .. (sets near the root hold thousands of points a child, so a warp to a whole
-// set left most of the chip waiting for the last of them). With rsqrt64: 1,183 -> 300 us for the 256
+// set left most of the chip waiting for the last of them). With rsqrt64 and widen: 1,183 -> 458 us for the 256
 // training queries of 2^17 winding sources.
 constexpr int kDatasetWarps = 4;
 
@@ -257,10 +257,10 @@ __global__ void __launch_bounds__(32 * kDatasetWarps) k_dataset(TreeView T, cons
 // softmax have a row to a lane. Each warp keeps its partial gradient, the block adds its warps'
 // partials in warp order and writes one row per block; k_sum_blocks adds the rows in block order.
 // No atomics, and every sum in a fixed order: the training is the same bit for bit on every run.
-//   It takes 96 multiply-adds per row and lane and half as many other instructions: bound by their
-// issue, with 12 warps to an SM (registers and shared memory). Reading W2 from shared memory with a
+//   It takes 96 multiply-adds per row and lane and half as many other instructions: bound by the latency
+// of their chains, with 12 warps to an SM (registers and shared memory) that issue 37% of the time. Reading W2 from shared memory with a
 // row to a lane (every lane in the same bank) and passing activations by shuffles took 534 us a step
-// for 2,220 sets, now 16.
+// for 2,219 sets, now 40: 555 blocks are 1.2 waves, so a part of it is the second wave's.
 // ------------------------------------------------------------------------------------------------
 constexpr int kTrainWarps = 4;
 constexpr int kTrainRows = 4;                // rows worked on together
@@ -473,7 +473,7 @@ __global__ void __launch_bounds__(32 * kTrainWarps, 3) k_loss_grad(const float* 
 
 // grad[i] = sum over blocks b (in order) of part[b][i]; loss likewise from the last column. ADAM: and
 // the Adam step with that gradient. One warp to a block, and kSumAhead rows asked for before the first
-// is added: the chain of additions is kept, the waits for the rows are not (25 -> 7 us for 555 rows).
+// is added: the chain of additions is kept, the waits for the rows are not (25 -> 11 us for 555 rows, with the Adam step).
 constexpr int kSumThreads = 32, kSumAhead = 64;
 
 template <bool ADAM>

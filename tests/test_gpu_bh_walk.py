@@ -27,7 +27,7 @@ def _tree(sbh, n=3000, normals=False, seed=0):
 
 
 @pytest.mark.parametrize("kind", ["coulomb", "winding", "smoothdist"])
-@pytest.mark.parametrize("nq", [(1 << 16), (1 << 16) + 1, 100003])
+@pytest.mark.parametrize("nq", [(1 << 16), (1 << 16) + 1, 100003, 1 << 19, (1 << 19) + 1, 600011])
 def test_order_of_queries_changes_nothing(sbh, kind, nq):
     import torch
     tree, p, _, _ = _tree(sbh, normals=kind == "winding")
@@ -44,10 +44,11 @@ def test_order_of_queries_changes_nothing(sbh, kind, nq):
 
 
 @pytest.mark.parametrize("vote", [False, True])
-def test_without_memory_for_the_records(sbh, vote):
+@pytest.mark.parametrize("nq", [70001, 600011])
+def test_without_memory_for_the_records(sbh, nq, vote):
     import torch
     tree, p, w, _ = _tree(sbh, n=20000)
-    Q = dev(np.random.default_rng(1).random((70001, 3), dtype=np.float32))
+    Q = dev(np.random.default_rng(1).random((nq, 3), dtype=np.float32))
     want = sbh.sbh_eval_bh(tree, Q, "coulomb", 0.7, vote)
     other = sbh.sbh_build(dev(p), dev(w), leaf_size=3)
     used = sbh.sbh_memory_in_use()
@@ -66,7 +67,7 @@ def test_without_memory_for_the_records(sbh, vote):
 
 
 @pytest.mark.parametrize("vote", [False, True])
-@pytest.mark.parametrize("nq", [1000, 70001])
+@pytest.mark.parametrize("nq", [1000, 70001, 600011])
 def test_trees_with_normals_walk_alike(sbh, nq, vote):
     """Normals change a tree's walk records, not its nodes or its masses."""
     import torch
