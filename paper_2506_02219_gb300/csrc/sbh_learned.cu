@@ -160,21 +160,10 @@ __global__ void k_set_rows(TreeView T, const int32_t* __restrict__ set_node, int
 // set = the children of a, features and |exact residual| targets (FP64 sums over the child's
 // points, in Morton order)
 // ------------------------------------------------------------------------------------------------
-// 1 / sqrt(x) in FP64: the FP32 approximation of relative error below 2^-21 and one step of the
-// cubically convergent y (1 + e/2 + 3 e^2 / 8), e = 1 - x y^2 (the binomial series of (1 - e)^(-1/2)),
-// which leaves the FP64 roundings. Seven FP64 instructions for the some forty of a root and a
-// division: they are what the training set's sums cost on a chip with two FP64 lanes to an SM.
-__device__ __forceinline__ double rsqrt64(double x)
-{
-    const float xf = (float)x;
-    if (!(xf >= 1e-36f && xf <= 1e36f)) return 1.0 / sqrt(x);  // zero, not a number, or outside FP32's range
-    const double y = widen(rsqrt_ftz(xf));
-    const double e = fma(-(x * y), y, 1.0);
-    return fma(y * e, fma(0.375, e, 0.5), y);
-}
-
-// m f(p, q) in FP64, without the factor of value64_factor (p: position and mass, N: m n of a node or a
-// unit normal, whose m is then scale)
+// m f(p, q) in FP64 (p: position and mass, N: m n of a node or a unit normal, whose m is then scale), by
+// correctly rounded roots and quotients: a child that is one point has the residual zero exactly, and a
+// set of such children uniform targets. (A reciprocal root refined from FP32's takes a third off the
+// kernel, but leaves such sets the noise of its last places as targets.)
 struct Query64 {
     double x, y, z;
 };
@@ -183,23 +172,19 @@ __device__ __forceinline__ double value64(float4 p, float4 N, double scale, cons
 {
     const double dx = widen(p.x) - q.x, dy = widen(p.y) - q.y, dz = widen(p.z) - q.z;
     const double r2 = dx * dx + dy * dy + dz * dz;
-    if constexpr (KIND == SBH_COULOMB) return widen(p.w) * rsqrt64(r2 + (double)kp.eps2);
+    if constexpr (KIND == SBH_COULOMB) return widen(p.w) / sqrt(r2 + (double)kp.eps2);
     else if constexpr (KIND == SBH_WINDING) {
         if (r2 == 0.0) return 0.0;
-        const double ir = rsqrt64(r2);
-        return scale * (dx * widen(N.x) + dy * widen(N.y) + dz * widen(N.z)) * (ir * ir * ir);
+        return scale * (dx * widen(N.x) + dy * widen(N.y) + dz * widen(N.z)) / (4.0 * 3.141592653589793 * r2 * sqrt(r2));
     } else if constexpr (KIND == SBH_SMOOTHDIST) {
-        return widen(p.w) * exp(-(double)kp.alpha * (r2 > 0.0 ? r2 * rsqrt64(r2) : 0.0));
+        return widen(p.w) * exp(-(double)kp.alpha * sqrt(r2));
     } else {
         return widen(p.w) * (1.0 + kp.g[0] * dx + kp.g[1] * dy + kp.g[2] * dz);
     }
 }
-template <int KIND>
-constexpr double value64_factor() { return KIND == SBH_WINDING ? 1.0 / (4.0 * 3.141592653589793) : 1.0; }
-
 // A block to a decision set s = (query set_q[s], node set_node[s]), a warp to each of its children in
 // turn: rows set_off[s] .. (sets near the root hold thousands of points a child, so a warp to a whole
-// set left most of the chip waiting for the last of them). With rsqrt64 and widen: 1,183 -> 458 us for the 256
+// set left most of the chip waiting for the last of them). With widen for the conversions: 1,183 -> 616 us for the 256
 // training queries of 2^17 winding sources.
 constexpr int kDatasetWarps = 4;
 
@@ -239,7 +224,7 @@ __global__ void __launch_bounds__(32 * kDatasetWarps) k_dataset(TreeView T, cons
             if (lane == 0) {
                 const float4 pc = __ldg(&T.pm[ch]);
                 const double r = sum - value64<KIND>(pc, KIND == SBH_WINDING ? __ldg(&T.dip[ch]) : none, 1.0, q64, kp);
-                targets[r0 + c] = (float)fabs(r * value64_factor<KIND>());
+                targets[r0 + c] = (float)fabs(r);
                 float x[6];
                 child_features(T, diam, ma, pa, ch, pc, __ldg(&T.meta[ch]), q, KIND == SBH_WINDING, x);
                 for (int k = 0; k < 6; ++k) feats[6 * (r0 + c) + k] = x[k];

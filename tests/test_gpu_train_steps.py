@@ -48,3 +48,26 @@ def test_training_repeats(sbh, nq, steps):
     assert got[0][0].shape == (steps,) and np.all(np.isfinite(got[0][0]))
     assert np.array_equal(got[0][0], got[1][0]) and np.array_equal(got[0][1], got[1][1])
     assert np.array_equal(got[0][0][:-1], got[2][0]) and not np.array_equal(got[0][1], got[2][1])
+
+
+@pytest.mark.parametrize("kind", ["coulomb", "winding"])
+def test_single_points_have_no_residual(sbh, kind):
+    """A child that is one source is its own centre of mass: its target is zero exactly (with normals along
+    an axis, so that the dipole m n is exact), and a set of such children then has uniform targets."""
+    import torch
+    rng = np.random.default_rng(9)
+    n = 5000
+    p = rng.random((n, 3)).astype(np.float32)
+    w = (rng.random(n) + 0.5).astype(np.float32)
+    v = np.zeros((n, 3), np.float32)
+    v[np.arange(n), rng.integers(0, 3, n)] = 1.0
+    tree = sbh.sbh_build(dev(p), dev(w), dev(v) if kind == "winding" else None)
+    ex = sbh.sbh_tree_export(tree, 0)
+    nodes = [u for u in range(len(ex["nchild"])) if 2 <= ex["nchild"][u] <= 64
+             and np.all(ex["nchild"][ex["first_child"][u]:ex["first_child"][u] + ex["nchild"][u]] == 0)][:300]
+    assert len(nodes) > 50
+    q = rng.random((len(nodes), 3)).astype(np.float32)
+    off = np.concatenate([[0], np.cumsum(ex["nchild"][nodes])]).astype(np.int64)
+    _, targets = sbh.sbh_mlp_dataset(tree, dev(q), torch.arange(len(nodes), dtype=torch.int32, device="cuda"),
+                                     torch.tensor(nodes, dtype=torch.int32, device="cuda"), torch.from_numpy(off).cuda(), kind)
+    assert bool((targets == 0).all())
