@@ -128,10 +128,11 @@ typedef struct {
  *   leaf_size 1 <= leaf_size <= 64: nodes with at most this many points are leaves
  * Builds the 64-ary estimator tree now; the 8-ary Barnes-Hut tree is built from the same sorted
  * codes on the first sbh_eval_bh call. The input buffers are not retained. On success *out owns
- * device memory until sbh_tree_free. Validation of the inputs synchronises the stream once; the
- * build itself is enqueued on `stream` and the call synchronises once more at its end. Returns
+ * device memory until sbh_tree_free. The build is enqueued on `stream` and the call synchronises it
+ * once, at its end, which is also where the check of the inputs is read. Returns
  * SBH_EINVAL for a bad size, NaN/Inf coordinates or a non-positive weight, SBH_ENOMEM when
- * device memory runs out, SBH_EUNSUPPORTED when more than 2^24 - 1 points share one cell of the
+ * device memory runs out, SBH_ETIMEOUT when a bounded wait between the build's blocks gave up (its
+ * limit is seconds without any progress), SBH_EUNSUPPORTED when more than 2^24 - 1 points share one cell of the
  * deepest level (2^-20 of the root cube per axis). */
 SBH_API sbh_status sbh_build(const float* points, const float* weights, const float* normals, int64_t n,
                      int32_t leaf_size, void* stream, sbh_tree** out);
@@ -334,7 +335,9 @@ SBH_API const char* sbh_last_error(void);
  * be ordered by the caller. Every call looks up the array's device address in the current
  * device's context (cudaGetSymbolAddress, no allocation), so the address is never stale after a
  * device reset; the first call on a device also loads the library's device code there, so make
- * that first call before any stream capture. Enqueued on `stream`, no synchronisation. */
+ * that first call before any stream capture. Enqueued on `stream`, no synchronisation. The blocks of
+ * the sort wait for each other, with a limit of seconds: should a wait ever give up, perm[0] is -1 and
+ * the rest of codes and perm is undefined. */
 #define SBH_NOALLOC_MAX_POINTS 65536
 SBH_API sbh_status sbh_morton_sort_noalloc(const float* points, int64_t n, uint64_t* codes, int32_t* perm,
                                            void* stream);

@@ -177,7 +177,7 @@ sbh_status sbh_build(const float* points, const float* weights, const float* nor
     if (c.error) {
         const int32_t why = c.error;
         release(T, s);
-        if (why == sbh::kErrorTimeout) return fail(SBH_ETIMEOUT, "sbh_build: a wait of the sort gave up");
+        if (why == sbh::kErrorTimeout) return fail(SBH_ETIMEOUT, "sbh_build: a bounded wait between the build's blocks gave up");
         return fail(SBH_EUNSUPPORTED, "sbh_build: more than 2^24 - 1 points share one deepest-level cell");
     }
     *out = T;

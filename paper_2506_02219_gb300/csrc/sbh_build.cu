@@ -319,8 +319,11 @@ __global__ void __launch_bounds__(kMortonThreads) k_morton(const float* __restri
 //    Parallel Prefix Scan with Decoupled Look-back", 2016; as a sort: Adinets and Merrill,
 //    "Onesweep", 2022): a status word per (tile, digit) says nothing yet, the tile's own count, or
 //    the count of it and all before it. A tile number is drawn when a block starts, so every tile
-//    waited for is already running; each wait is bounded all the same, and one that runs out sets
-//    H->error, which ends the build with SBH_ETIMEOUT.
+//    waited for is already running; each wait is bounded all the same. One that runs out sets H->error
+//    and hands on what it has: keys may then be missing from the sorted arrays and their places hold
+//    what was in memory before, which nothing may use as an index. k_gather leaves the points in the
+//    caller's order and sets the tree's error, no records are made, and sbh_build returns SBH_ETIMEOUT;
+//    the walk drops the order of its queries; sbh_morton_sort_noalloc marks its output (`report`).
 //    What bounds it: the latency of a tile's steps (load, rank, look back, write) with two blocks of
 //    512 threads to an SM; the 24 bytes a key moves take a quarter of the time. It replaces a count, a
 //    scan of up to three kernels and a scatter that sorted its tile by nine one-bit splits: 40 kernels
@@ -328,7 +331,10 @@ __global__ void __launch_bounds__(kMortonThreads) k_morton(const float* __restri
 //    digits come with the codes.
 // ----------------------------------------------------------------------------------------------
 constexpr uint32_t kStatusOwn = 1u << 30, kStatusAll = 2u << 30, kStatusMask = (1u << 30) - 1;
-constexpr int kSpinLimit = 1 << 22;  // polls before a wait gives up (seconds)
+#ifndef SBH_SPIN_LIMIT
+#define SBH_SPIN_LIMIT (1 << 22)
+#endif
+constexpr int kSpinLimit = SBH_SPIN_LIMIT;  // polls before a wait gives up (seconds); below 0: all do, at once (for tests)
 constexpr int kLook = 4;             // status words a digit's thread has in flight
 
 // The lanes of the warp whose 8-bit digit equals the caller's, by one ballot per bit: about 40 cycles
@@ -346,14 +352,16 @@ __device__ __forceinline__ unsigned same_digit(int d)
     return peers;
 }
 
-template <int ITEMS>
-__global__ void __launch_bounds__(kSortThreads, 2) k_radix_pass(const uint64_t* __restrict__ kin,
+// REPORT (of the last pass): *report = -1 if a wait of any pass gave up
+template <bool REPORT>
+__global__ void __launch_bounds__(kSortThreads, REPORT ? 1 : 2) k_radix_pass(const uint64_t* __restrict__ kin,
                                                              const int32_t* __restrict__ vin, int64_t n, int pass,
                                                              SortHead* __restrict__ H, uint32_t* status,
                                                              uint32_t* __restrict__ next_status,
-                                                             uint64_t* __restrict__ kout, int32_t* __restrict__ vout)
+                                                             uint64_t* __restrict__ kout, int32_t* __restrict__ vout,
+                                                             int32_t* report)
 {
-    constexpr int kTile = kSortThreads * ITEMS, kWarps = kSortThreads / 32;
+    constexpr int ITEMS = kSortItems, kTile = kSortTile, kWarps = kSortThreads / 32;
     extern __shared__ __align__(16) unsigned char s_sort[];
     uint64_t* s_key = reinterpret_cast<uint64_t*>(s_sort);
     int32_t* s_val = reinterpret_cast<int32_t*>(s_key + kTile);
@@ -428,6 +436,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_radix_pass(const uint64_t* 
     if (tile > 0 && t < 256) {
         int spin = 0;
         for (int p = tile - 1; p >= 0;) {
+            if (kSpinLimit < 0) { H->error = 1; break; }
             uint32_t v[kLook];
 #pragma unroll
             for (int k = 0; k < kLook; ++k) v[k] = p - k >= 0 ? st[(int64_t)(p - k) * 256 + t] : (uint32_t)kStatusAll;
@@ -459,6 +468,9 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_radix_pass(const uint64_t* 
             kout[dst] = k;
             vout[dst] = s_val[i];
         }
+    }
+    if constexpr (REPORT) {
+        if (last_block(&H->done[2]) && t == 0 && *(volatile int32_t*)&H->error) *report = -1;
     }
 }
 
@@ -549,28 +561,27 @@ int64_t sort_tiles(int64_t n) { return (n + kSortTile - 1) / kSortTile; }
 
 size_t sort_status_bytes(int64_t n) { return (size_t)sort_tiles(n) * 256 * sizeof(uint32_t); }
 
-template <int ITEMS>
+constexpr size_t kPassSmem = kSortTile * (sizeof(uint64_t) + sizeof(int32_t)) + (kSortThreads / 32) * 256 * sizeof(uint16_t);
+
 static cudaError_t radix_passes(uint64_t* const k[2], int32_t* const v[2], int64_t n, int passes, SortHead* H,
-                                uint32_t* status, cudaStream_t s)
+                                uint32_t* status, int32_t* report, cudaStream_t s)
 {
-    constexpr int kTile = kSortThreads * ITEMS;
-    constexpr size_t kBytes = (size_t)kTile * (sizeof(uint64_t) + sizeof(int32_t)) + (kSortThreads / 32) * 256 * sizeof(uint16_t);
-    const cudaError_t e = cudaFuncSetAttribute(k_radix_pass<ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBytes);
-    if (e != cudaSuccess) return e;
-    const unsigned tiles = (unsigned)((n + kTile - 1) / kTile);
-    const size_t words = (size_t)sort_tiles(n) * 256;
+    const unsigned tiles = (unsigned)sort_tiles(n);
+    const size_t words = (size_t)tiles * 256;
     for (int pass = 0; pass < passes; ++pass) {
         const int a = pass & 1;
-        k_radix_pass<ITEMS><<<tiles, kSortThreads, kBytes, s>>>(k[a], pass ? v[a] : nullptr, n, pass, H,
-                                                                status + a * words, status + (a ^ 1) * words, k[a ^ 1],
-                                                                v[a ^ 1]);
+        const auto kernel = report && pass == passes - 1 ? k_radix_pass<true> : k_radix_pass<false>;
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPassSmem);
+        if (e != cudaSuccess) return e;
+        kernel<<<tiles, kSortThreads, kPassSmem, s>>>(k[a], pass ? v[a] : nullptr, n, pass, H, status + a * words,
+                                                      status + (a ^ 1) * words, k[a ^ 1], v[a ^ 1], report);
         note_launch();
     }
     return cudaGetLastError();
 }
 
 cudaError_t sort_codes(const float* pts, const float* w, int64_t n, uint64_t* const k[2], int32_t* const v[2],
-                       SortHead* H, uint32_t* status, TreeCtrl* c4, TreeCtrl* c2, cudaStream_t s)
+                       SortHead* H, uint32_t* status, TreeCtrl* c4, TreeCtrl* c2, int32_t* report, cudaStream_t s)
 {
     const bool one_tile = n <= kSortTile;
     cudaError_t e = cudaMemsetAsync(H, 0, sizeof(SortHead), s);
@@ -587,7 +598,7 @@ cudaError_t sort_codes(const float* pts, const float* w, int64_t n, uint64_t* co
         note_launch();
         return cudaGetLastError();
     }
-    return radix_passes<kSortItems>(k, v, n, kPasses, H, status, s);
+    return radix_passes(k, v, n, kPasses, H, status, report, s);
 }
 
 cudaError_t sort_queries(const float* q, int64_t n, const TreeCtrl* ctrl, void** scratch, const int32_t** order,
@@ -615,7 +626,7 @@ cudaError_t sort_queries(const float* q, int64_t n, const TreeCtrl* ctrl, void**
     if (e == cudaSuccess) {
         k_morton<kQueryPasses><<<grid_for(n, kMortonThreads, 2u * (unsigned)device_sm_count()), kMortonThreads, 0, s>>>(q, n, ctrl, k[0], H);
         note_launch();
-        e = radix_passes<kSortItems>(k, v, n, kQueryPasses, H, status, s);
+        e = radix_passes(k, v, n, kQueryPasses, H, status, nullptr, s);
     }
     if (e != cudaSuccess) {
         dfree(*scratch, s);
@@ -689,12 +700,15 @@ __global__ void __launch_bounds__(kTopoThreads) k_gather(const float* __restrict
                                                          uint8_t* __restrict__ lcp4, uint8_t* __restrict__ lcp2,
                                                          const SortHead* __restrict__ H, TreeCtrl* ctrl)
 {
-    if (blockIdx.x == 0 && threadIdx.x == 0 && H->error) ctrl->error = kErrorTimeout;  // of the sort
+    // Where a wait of the sort gave up, perm and code hold anything: the points stay where they are, and
+    // the shared digits are kept in range, for which any values make a tree
+    const bool sorted = H->error == 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0 && !sorted) ctrl->error = kErrorTimeout;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t j = perm[i];
+        const int64_t j = sorted ? perm[i] : i;
         spw[i] = make_float4(pts[3 * j], pts[3 * j + 1], pts[3 * j + 2], w[j]);
         if (nrm) snrm[i] = make_float4(nrm[3 * j], nrm[3 * j + 1], nrm[3 * j + 2], 0.0f);
-        const int same = i ? __clzll((long long)(code[i] ^ code[i - 1])) - 4 : 0;  // codes use 60 bits
+        const int same = i ? max(__clzll((long long)(code[i] ^ code[i - 1])) - 4, 0) : 0;  // codes use 60 bits
         lcp4[i] = (uint8_t)min(same / 6, kMaxLevel4);
         lcp2[i] = (uint8_t)min(same / 3, kMaxLevel2);
     }
@@ -1132,7 +1146,7 @@ __device__ __forceinline__ void grid_barrier(const AggArrays& A, unsigned target
         atomicAdd(A.barrier, 1u);
         volatile unsigned* at = A.barrier;
         int spin = 0;
-        while (*at < target)
+        while (*at < target || kSpinLimit < 0)
             if (++spin > kSpinLimit) { A.B.ctrl->error = kErrorTimeout; break; }
         __threadfence();
     }
@@ -1262,6 +1276,7 @@ __global__ void __launch_bounds__(kAggThreads, kAggBlocks) k_aggregate(AggArrays
     const int lane = threadIdx.x & 31;
     const TreeCtrl* ctrl = A.B.ctrl;
     const int deepest = ctrl->max_depth;
+    if (ctrl->error) return;  // found before this kernel (another block's give-up makes it end all the sooner)
     if (blockIdx.x == 0 && threadIdx.x == 0) {  // the root is nobody's child
         A.cdf[0] = 1.0f;
         A.gd[0] = 0;
@@ -1391,7 +1406,7 @@ cudaError_t build_sorted(sbh_tree* T, const float* pts, const float* w, const fl
         SBH_TRY(guard.alloc(&k[a], n * sizeof(uint64_t)));
         SBH_TRY(guard.alloc(&v[a], n * sizeof(int32_t)));
     }
-    SBH_TRY(sort_codes(pts, w, n, k, v, head, status, T->t4.ctrl, T->t2.ctrl, s));
+    SBH_TRY(sort_codes(pts, w, n, k, v, head, status, T->t4.ctrl, T->t2.ctrl, nullptr, s));
     T->code = k[0];  // an even number of passes ends where it began
     T->perm = v[0];
     guard.keep(k[0]);

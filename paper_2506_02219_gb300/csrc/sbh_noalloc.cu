@@ -71,11 +71,12 @@ sbh_status sbh_morton_sort_noalloc(const float* points, int64_t n, uint64_t* cod
     TreeCtrl* ctrl = (TreeCtrl*)(base + kOffCtrl);
     // the sort goes back and forth between the caller's outputs and the scratch copy and ends in the
     // outputs. The count of bad weights is not used here; the points array stands in for the weights
-    // (it has 3n floats, so the n reads stay inside it)
+    // (it has 3n floats, so the n reads stay inside it). There is no status to return later: a sort whose
+    // bounded wait gave up says so in perm[0].
     uint64_t* const k[2] = {codes, (uint64_t*)(base + kOffKeys)};
     int32_t* const v[2] = {perm, (int32_t*)(base + kOffVals)};
     e = sort_codes(points, points, n, k, v, (SortHead*)(base + kOffHead), (uint32_t*)(base + kOffStatus), ctrl,
-                   ctrl + 1, s);
+                   ctrl + 1, perm, s);
     if (e != cudaSuccess) {
         set_error_message("sbh_morton_sort_noalloc: kernel launch failed: %s", cudaGetErrorString(e));
         return SBH_ECUDA;

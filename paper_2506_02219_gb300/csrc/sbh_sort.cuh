@@ -18,7 +18,7 @@ constexpr int kQueryPasses = 3;
 // Zeroed before each sort
 struct SortHead {
     uint32_t bounds[8];          // ordered-integer maxima of -x, -y, -z, x, y, z; bad coordinates, bad weights
-    unsigned done[2];            // blocks of k_bounds, k_morton that are through
+    unsigned done[3];            // blocks of k_bounds, k_morton, the last pass that are through
     uint32_t next_tile[kPasses]; // tiles drawn in each pass
     int32_t error;               // nonzero: a bounded wait gave up
     int32_t hist[kPasses][256];  // counts of each digit, then where its run starts
@@ -29,8 +29,10 @@ size_t sort_status_bytes(int64_t n);
 
 // Enqueue the root cube (c4, c2), the codes and their stable sort: k[0], v[0] get the sorted codes and
 // the input index of each; k[1], v[1] are scratch of the same size, status 2 x sort_status_bytes(n).
+// Where a bounded wait gave up, H->error is set when the sort has run, k[0] and v[0] are damaged, and
+// *report (unless it is null) is -1.
 cudaError_t sort_codes(const float* pts, const float* w, int64_t n, uint64_t* const k[2], int32_t* const v[2],
-                       SortHead* H, uint32_t* status, TreeCtrl* c4, TreeCtrl* c2, cudaStream_t s);
+                       SortHead* H, uint32_t* status, TreeCtrl* c4, TreeCtrl* c2, int32_t* report, cudaStream_t s);
 
 // Order of n queries by their Morton codes in twice the tree's root cube (24 bits, three passes): order[i]
 // is the query to take at place i, unless *error is set when the sort has run. Both are in *scratch,
