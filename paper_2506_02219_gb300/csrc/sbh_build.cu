@@ -222,9 +222,10 @@ __global__ void __launch_bounds__(kThreads) k_bounds(const float* __restrict__ p
         for (int a = 0; a < 3; ++a) { c4->lo[a] = lo[a]; c2->lo[a] = lo[a]; }
         c4->side = side;
         c2->side = side;
-        c4->error = c2->error = 0;
         c4->bad_points = (int32_t)__ldcg(&H->bounds[6]);
         c4->bad_weights = (int32_t)__ldcg(&H->bounds[7]);
+        c4->error = c4->bad_points || c4->bad_weights ? kErrorInput : 0;
+        c2->error = 0;
     }
 }
 
@@ -711,6 +712,8 @@ __global__ void __launch_bounds__(kTopoThreads) k_gather(const float* __restrict
         const int same = i ? max(__clzll((long long)(code[i] ^ code[i - 1])) - 4, 0) : 0;  // codes use 60 bits
         lcp4[i] = (uint8_t)min(same / 6, kMaxLevel4);
         lcp2[i] = (uint8_t)min(same / 3, kMaxLevel2);
+        // equal codes are the points of one cell of the deepest level
+        if (sorted && i >= (int64_t)kMaxChildren && code[i] == code[i - kMaxChildren]) ctrl->error = kErrorChildren;
     }
 }
 
@@ -1228,10 +1231,7 @@ __device__ __forceinline__ void aggregate_node(const AggArrays& A, AggScratch<NO
             if (sub == 4 && A.pmd) A.pmd[2 * (int64_t)v] = pm;
             if (sub == 5 && A.pmd) A.pmd[2 * (int64_t)v + 1] = dp;
         }
-        if (sub == 2) {
-            if ((uint32_t)nc > kMaxChildren) A.B.ctrl->error = kErrorChildren;
-            A.B.meta[v] |= (uint32_t)nc & kMaxChildren;
-        }
+        if (sub == 2) A.B.meta[v] |= (uint32_t)nc & kMaxChildren;
         if (nc <= kAggChildren) {
             for (int c = sub; c < nc; c += kLanes) {
                 const float q = c == nc - 1 ? 1.0f : quotient_rn(S.pre[group][c], m, M, y);
@@ -1276,7 +1276,9 @@ __global__ void __launch_bounds__(kAggThreads, kAggBlocks) k_aggregate(AggArrays
     const int lane = threadIdx.x & 31;
     const TreeCtrl* ctrl = A.B.ctrl;
     const int deepest = ctrl->max_depth;
-    if (ctrl->error) return;  // found before this kernel (another block's give-up makes it end all the sooner)
+    // Input that is refused has no records made: points that are not numbers, say, are one leaf of all of
+    // them, a single warp's work (2^18: the refusal took 128 ms). Errors of this kernel itself end it too.
+    if (ctrl->error) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) {  // the root is nobody's child
         A.cdf[0] = 1.0f;
         A.gd[0] = 0;

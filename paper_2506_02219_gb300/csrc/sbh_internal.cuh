@@ -57,12 +57,13 @@ struct TreeCtrl {
     float lo[3];
     float side;
     float diam[kDiamLevels];  // |B| at each level: sqrt(3) * side * d^-level (FP32, exact scaling)
-    int32_t error;        // kErrorChildren, kErrorTimeout: a build step failed
+    int32_t error;        // kError...: why there is no tree
     int32_t bad_points;   // non-finite coordinates among the points
     int32_t bad_weights;  // weights not finite or not > 0
 };
 constexpr int32_t kErrorChildren = 1;  // a node with more than kMaxChildren children
 constexpr int32_t kErrorTimeout = 2;   // a bounded wait gave up
+constexpr int32_t kErrorInput = 3;     // bad coordinates or weights
 
 // A walk record's level field (level times 4) of a single point: past every level, in the opening limits' table
 constexpr int kWalkPoint = 4 * (kDiamLevels - 1);
