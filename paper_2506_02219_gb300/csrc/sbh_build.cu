@@ -771,7 +771,7 @@ __global__ void __launch_bounds__(kTopoThreads) k_topo_runs(BuildArrays B)
     const int64_t i = (int64_t)blockIdx.x * kTopoTile + 8 * threadIdx.x;
     int have;
     const uint64_t l8 = lcp8(B, i, have);
-    if (i == 0) B.from_right[B.tiles] = 0u;  // k_aggregate's barrier
+    if (i == 0) B.from_right[B.tiles] = B.from_right[B.tiles + 1] = 0u;  // k_aggregate's barrier
     tile_runs(l8, have, i == 0, B.from_left, B.from_right, s_run);
 }
 
@@ -1136,11 +1136,19 @@ struct AggArrays {
     float4* pmd;
     float* cdf;
     uint8_t* gd;
-    unsigned* barrier;  // blocks that are through with a generation, over all of them; zero at first
+    unsigned* barrier;  // [0] blocks that are through with a generation, over all of them; [1] signs of life
 };
 
+// A leaf of many coincident points is one warp's work for 0.5 us a point, while every other block waits
+// for it: the warp gives a sign of life after at most so many children, and a wait gives up only where
+// there was none for its whole limit. (By the count of polls alone, some three million points in one
+// cell, of 2^24 - 1 that are allowed, ended the build with SBH_ETIMEOUT.)
+constexpr int kBeat = 4096;
+__device__ __forceinline__ void beat(const AggArrays& A) { atomicAdd(A.barrier + 1, 1u); }
+
 // Every block's writes of the generations so far are visible to every block. The grid is a cooperative
-// launch, so all its blocks are running; the wait is bounded all the same.
+// launch, so all its blocks are running; the wait is bounded all the same, by kSpinLimit polls without a
+// sign of life.
 __device__ __forceinline__ void grid_barrier(const AggArrays& A, unsigned target)
 {
     __syncthreads();
@@ -1149,8 +1157,17 @@ __device__ __forceinline__ void grid_barrier(const AggArrays& A, unsigned target
         atomicAdd(A.barrier, 1u);
         volatile unsigned* at = A.barrier;
         int spin = 0;
-        while (*at < target || kSpinLimit < 0)
-            if (++spin > kSpinLimit) { A.B.ctrl->error = kErrorTimeout; break; }
+        unsigned seen = 0;
+        while (*at < target || kSpinLimit < 0) {
+            if (++spin <= kSpinLimit) continue;
+            const unsigned beats = at[1];
+            if (kSpinLimit < 0 || beats == seen) {
+                atomicCAS(&A.B.ctrl->error, 0, kErrorTimeout);
+                break;
+            }
+            seen = beats;
+            spin = 0;
+        }
         __threadfence();
     }
     __syncthreads();
@@ -1196,6 +1213,7 @@ __device__ __forceinline__ void aggregate_node(const AggArrays& A, AggScratch<NO
 #pragma unroll
     for (int k = 0; k < kAhead; ++k) next[k] = k < nc ? __ldcg(&A.agg[kLanes * (int64_t)(f + k) + sub]) : 0.0;
     for (int c0 = 0; c0 < wide; c0 += kAhead) {
+        if (c0 && c0 % kBeat == 0 && lane == 0) beat(A);
         double x[kAhead];
 #pragma unroll
         for (int k = 0; k < kAhead; ++k) {
@@ -1249,6 +1267,7 @@ __device__ __forceinline__ void aggregate_node(const AggArrays& A, AggScratch<NO
         double pre = 0.0;
         for (int c0 = 0; c0 < wide; c0 += kAggChildren) {
             __syncwarp();
+            if (c0 % kBeat == 0 && lane == 0) beat(A);
             if (mine && sub == 0)
                 for (int c = c0; c < nc && c < c0 + kAggChildren; ++c) {
                     pre += __ldcg(&A.agg[kLanes * (int64_t)(f + c)]);
@@ -1262,7 +1281,10 @@ __device__ __forceinline__ void aggregate_node(const AggArrays& A, AggScratch<NO
         __threadfence_block();
         __syncwarp();
         if (mine)
-            for (int j = sub; j < nc; j += kLanes) A.gd[f + j] = guide_entry(A.cdf + f, (uint32_t)nc, (uint32_t)j);
+            for (int j = sub; j < nc; j += kLanes) {
+                if (j && j % kBeat == 0) beat(A);
+                A.gd[f + j] = guide_entry(A.cdf + f, (uint32_t)nc, (uint32_t)j);
+            }
     }
     __syncwarp();
 }
@@ -1438,7 +1460,7 @@ cudaError_t build_tree(sbh_tree* T, DeviceTree& D, const uint8_t* lcp, int max_l
     SBH_TRY(guard.alloc(&B.mask, n * sizeof(uint32_t)));
     SBH_TRY(guard.alloc(&B.last_child, D.cap * sizeof(int32_t)));
     SBH_TRY(guard.alloc(&B.count, (kMaxDepth + 1) * tiles * sizeof(int32_t)));
-    SBH_TRY(guard.alloc(&B.from_left, (2 * tiles + 1) * sizeof(uint32_t)));
+    SBH_TRY(guard.alloc(&B.from_left, (2 * tiles + 2) * sizeof(uint32_t)));
     B.from_right = B.from_left + tiles;
 
     k_topo_runs<<<(unsigned)tiles, kTopoThreads, 0, s>>>(B);
