@@ -1473,11 +1473,13 @@ cudaError_t build_tree(sbh_tree* T, DeviceTree& D, const uint8_t* lcp, int max_l
     note_launch();
     SBH_TRY(cudaGetLastError());
     AggArrays A = {B, T->spw, T->snrm, D.agg, D.pm, D.dip, D.pmd, D.cdf, D.gd, reinterpret_cast<unsigned*>(B.from_right + tiles)};
-    int64_t blocks = (2 * n + kAggThreads - 1) / kAggThreads;
-    const int64_t resident = (int64_t)kAggBlocks * device_sm_count();
-    if (blocks > resident) blocks = resident;
     void* args[] = {&A};
     const void* kernel = T->snrm ? reinterpret_cast<const void*>(k_aggregate<true>) : reinterpret_cast<const void*>(k_aggregate<false>);
+    int per_sm = 0;  // blocks of a cooperative launch must all be resident: as many as fit, at most kAggBlocks
+    SBH_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kAggThreads, 0));
+    int64_t blocks = (2 * n + kAggThreads - 1) / kAggThreads;
+    const int64_t resident = (int64_t)(per_sm < kAggBlocks ? per_sm : kAggBlocks) * device_sm_count();
+    if (blocks > resident) blocks = resident;
     SBH_TRY(cudaLaunchCooperativeKernel(kernel, dim3((unsigned)blocks),
                                         dim3(kAggThreads), args, 0, s));
     note_launch();
