@@ -1,12 +1,14 @@
 // sbh_brute.cu -- the exact kernel sum F(q) = sum_i m_i f(p_i, q) (Madan et al. 2025, Eq. 1) and its
 // query gradient by tiled brute force (the paper's ground truth, Sec. 4.3).
 //
-// A block of eight warps works on one group of 32 x QPT queries, QPT to a lane, and every warp of it on
-// another eighth of each source tile; a cluster of up to eight blocks splits the sources further. So
-// a few thousand queries fill the chip (5,001 queries: 79 groups of 64 make 632 blocks instead of
-// the 20 that one query per thread makes), and a source read from shared memory serves QPT queries.
-// Partial sums meet in shared memory, then across the cluster's distributed shared memory, always in
-// the same order: no scratch memory, no atomics, results reproducible.
+// Where queries are few for the chip, a block of eight warps works on one group of 32 x QPT queries, QPT to
+// a lane, and every warp of it on another eighth of each source tile; a cluster of up to eight blocks
+// splits the sources further. So a few thousand queries fill the chip (5,001 queries: 79 groups of 64
+// make 632 blocks instead of the 20 that one query per thread makes), and a source read from shared
+// memory serves QPT queries. Partial sums meet in shared memory, then across the cluster's
+// distributed shared memory, always in the same order: no scratch memory, no atomics, results
+// reproducible. Where queries are many or sources few, each warp has queries of its own and goes
+// through all sources, and there is nothing to join (launch_kind).
 //
 // Sources are staged two by two, so that the packed FP32 instructions take both of a pair at once.
 // What bounds it: the FP32 pipe's register reads. A winding term is 12 FMA-pipe operations, most of them on
@@ -14,7 +16,7 @@
 // repeated operand; measured, packed or scalar alike): 19 cycles a term, of which the reciprocal root's 8.4
 // run beside. The Coulomb term takes 9.7 cycles, near the root's own rate.
 // 65,536 queries against 2^20 sources, winding: 49.1 -> 32.2 ms; smooth distance and gradient, 5,001
-// queries against 2^19 sources: 47.3 -> 2.5 ms (one query per thread ran on 20 of 152 SMs, and the FP64
+// queries against 2^19 sources: 47.3 -> 2.3 ms (one query per thread ran on 20 of 152 SMs, and the FP64
 // sums were rescaled with every new smallest distance).
 //
 // With fp64_accum every FP32 partial sum of at most 256 terms is added into an FP64 accumulator, which
@@ -38,7 +40,7 @@ constexpr int kBruteWarps = 8;
 constexpr int kBruteThreads = 32 * kBruteWarps;
 constexpr int kWarpTile = 128;                       // sources of a tile that one warp takes
 constexpr int kBruteTile = kWarpTile * kBruteWarps;  // sources staged at a time
-constexpr int kFlushTiles = 2;                       // tiles per FP32 partial: 256 terms at most
+constexpr int kOwnTile = 256;                        // the same where each warp takes all of them
 constexpr int kMaxCluster = 8;
 
 __device__ __forceinline__ float ex2_ftz(float x)
@@ -88,8 +90,14 @@ struct Sums {
             for (int c = 0; c < 3; ++c) { g[c] = f2_dup(0.0f); ag[c] = 0; }
         ref = aref = 3.0e38f;
     }
+    // SPLIT as in k_brute; where a query has few terms the conversions count, and integer operations do them
+    template <bool SPLIT>
     __device__ __forceinline__ void flush(float c2)
     {
+        const auto acc = [](float x) -> Acc {
+            if constexpr (FP64 && !SPLIT) return widen(x);
+            else return (Acc)x;
+        };
         if constexpr (KIND == SBH_SMOOTHDIST) {
             if (ref < aref) {
                 const Acc f = (Acc)ex2_ftz(c2 * (aref - ref));
@@ -99,10 +107,10 @@ struct Sums {
                 aref = ref;
             }
         }
-        av += (Acc)(f2_lo(v) + f2_hi(v));
+        av += acc(f2_lo(v) + f2_hi(v));
         v = f2_dup(0.0f);
         if constexpr (GRAD)
-            for (int c = 0; c < 3; ++c) { ag[c] += (Acc)(f2_lo(g[c]) + f2_hi(g[c])); g[c] = f2_dup(0.0f); }
+            for (int c = 0; c < 3; ++c) { ag[c] += acc(f2_lo(g[c]) + f2_hi(g[c])); g[c] = f2_dup(0.0f); }
     }
     // the frame moves down to distance d (rare: about ln n times a query)
     __device__ __forceinline__ void lower(float d, float c2)
@@ -229,27 +237,52 @@ __device__ __forceinline__ Part<FP64, GRAD> sum_parts(int count, float alpha, Ge
     return s;
 }
 
-template <int KIND, bool FP64, bool GRAD, int QPT>
-__global__ void __launch_bounds__(kBruteThreads) k_brute(const float* __restrict__ P, const float* __restrict__ W,
-                                                         const float* __restrict__ N, int64_t n,
-                                                         const float* __restrict__ Q, int64_t nq, KernelParams kp,
-                                                         float* __restrict__ out, float* __restrict__ grad)
+// The results of query j from its sums over all sources
+template <int KIND, bool GRAD, class Acc>
+__device__ __forceinline__ void write_query(int64_t j, Acc sum, const Acc* g, float ref, const KernelParams& kp,
+                                            float* __restrict__ out, float* __restrict__ grad)
+{
+    const double v = (double)sum;
+    if constexpr (KIND == SBH_SMOOTHDIST) {
+        const bool pos = v > 0.0;
+        out[j] = pos ? (float)((double)ref - log(v) / (double)kp.alpha) : __int_as_float(0x7F800000);
+        if constexpr (GRAD)  // d = ref - log(acc) / alpha: grad d = -grad acc / (alpha acc); alpha cancels
+            for (int c = 0; c < 3; ++c)
+                grad[3 * j + c] = pos ? (float)(-(double)g[c] / v) : __int_as_float(0x7FC00000);
+    } else {
+        const double f = KIND == SBH_WINDING ? 0.07957747154594766788 : 1.0;  // 1 / (4 pi)
+        out[j] = (float)(v * f);
+        if constexpr (GRAD)
+            for (int c = 0; c < 3; ++c) grad[3 * j + c] = (float)((double)g[c] * f);
+    }
+}
+
+// blocks to an SM asked for (0: as it comes): three of the smooth distance's gradient, 2.52 -> 2.32 ms for 5,001
+// queries against 2^19 sources (at 80 registers either way)
+template <int KIND, bool GRAD, bool SPLIT>
+constexpr int brute_blocks() { return KIND == SBH_SMOOTHDIST && GRAD && SPLIT ? 3 : 0; }
+
+// SPLIT: the warps of a block work on the same queries, else each on its own
+template <int KIND, bool FP64, bool GRAD, int QPT, bool SPLIT>
+__global__ void __launch_bounds__(kBruteThreads, brute_blocks<KIND, GRAD, SPLIT>()) k_brute(
+    const float* __restrict__ P, const float* __restrict__ W, const float* __restrict__ N, int64_t n,
+    const float* __restrict__ Q, int64_t nq, KernelParams kp, float* __restrict__ out, float* __restrict__ grad)
 {
     constexpr int kQuads = Pair<KIND>::kQuads;
     constexpr int kGroup = 32 * QPT;
+    constexpr int kTile = SPLIT ? kBruteTile : kOwnTile, kShare = SPLIT ? kBruteWarps : 1;
     using PartT = Part<FP64, GRAD>;
-    constexpr size_t kTileBytes = (size_t)(kBruteTile / 2) * kQuads * sizeof(float4);
-    constexpr size_t kPartBytes = sizeof(PartT) * kGroup * kBruteWarps;
+    constexpr size_t kTileBytes = (size_t)(kTile / 2) * kQuads * sizeof(float4);
+    constexpr size_t kPartBytes = SPLIT ? sizeof(PartT) * kGroup * kBruteWarps : 0;
     __shared__ __align__(16) unsigned char s_buf[kTileBytes > kPartBytes ? kTileBytes : kPartBytes];
-    __shared__ PartT s_block[kGroup];
     float4* tile = reinterpret_cast<float4*>(s_buf);
     cg::cluster_group cluster = cg::this_cluster();
-    const int rank = (int)cluster.block_rank(), ranks = (int)cluster.num_blocks();
+    const int rank = SPLIT ? (int)cluster.block_rank() : 0, ranks = SPLIT ? (int)cluster.num_blocks() : 1;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t q0 = (int64_t)(blockIdx.x / ranks) * kGroup;
-    // this block's sources: whole tiles, as evenly as they go
-    const int64_t tiles = (n + kBruteTile - 1) / kBruteTile;
-    const int64_t t_lo = tiles * rank / ranks, t_hi = tiles * (rank + 1) / ranks;
+    const int64_t q0 = (SPLIT ? (int64_t)(blockIdx.x / ranks) : (int64_t)blockIdx.x * kBruteWarps + warp) * kGroup;
+    // this block's sources, as evenly as whole pairs go
+    const int64_t s_lo = (n * rank / ranks) & ~(int64_t)1;
+    const int64_t s_hi = rank == ranks - 1 ? n : (n * (rank + 1) / ranks) & ~(int64_t)1;
 
     Sums<KIND, FP64, GRAD> S[QPT];
 #pragma unroll
@@ -258,12 +291,13 @@ __global__ void __launch_bounds__(kBruteThreads) k_brute(const float* __restrict
         S[k].init(j < nq ? make_float3(Q[3 * j], Q[3 * j + 1], Q[3 * j + 2]) : make_float3(0.f, 0.f, 0.f));
     }
     const float c2 = -kp.alpha * 1.44269504088896341f;  // exp(-alpha x) = 2^(c2 x)
-    for (int64_t t = t_lo; t < t_hi; ++t) {
-        const int64_t base = t * kBruteTile;
-        const int cnt = (n - base) < kBruteTile ? (int)(n - base) : kBruteTile;
+    const int tiles = (int)((s_hi - s_lo + kTile - 1) / kTile);
+    for (int t = 0; t < tiles; ++t) {
+        const int64_t base = s_lo + (int64_t)t * kTile;
+        const int cnt = (s_hi - base) < kTile ? (int)(s_hi - base) : kTile;
         __syncthreads();
         for (int k = threadIdx.x; k < (cnt + 1) / 2; k += kBruteThreads) {
-            const int64_t i = base + 2 * k, i1 = i + 1 < n ? i + 1 : i;
+            const int64_t i = base + 2 * k, i1 = i + 1 < s_hi ? i + 1 : i;
             float4* d = tile + kQuads * k;
             const float w0 = W[i], w1 = W[i1];
             d[0] = make_float4(P[3 * i], P[3 * i1], P[3 * i + 1], P[3 * i1 + 1]);
@@ -275,9 +309,9 @@ __global__ void __launch_bounds__(kBruteThreads) k_brute(const float* __restrict
             }
         }
         __syncthreads();
-        // the warp's eighth of the tile, in whole pairs; only the last pair of all may hold padding
-        const int per = cnt == kBruteTile ? kWarpTile / 2 : ((cnt + 1) / 2 + kBruteWarps - 1) / kBruteWarps;
-        const int lo = warp * per, full = cnt / 2;
+        // the warp's part of the tile, in whole pairs; only the last pair of all may hold padding
+        const int per = cnt == kTile ? kTile / 2 / kShare : ((cnt + 1) / 2 + kShare - 1) / kShare;
+        const int lo = SPLIT ? warp * per : 0, full = cnt / 2;
         const int hi = lo + per < full ? lo + per : full;
         // measured per kernel: 20.3 / 18.9 cycles a winding term at 2 / 4, 21.7 / 21.0 / 23.7 a smooth-distance
         // one at 2 / 1 / 4, its gradient 2.51 / 2.58 ms (5,001 queries, 2^19 sources) at 2 / 1
@@ -295,95 +329,122 @@ __global__ void __launch_bounds__(kBruteThreads) k_brute(const float* __restrict
 #pragma unroll
             for (int u = 0; u < QPT; ++u) S[u].template add<false>(p, kp, c2);
         }
-        if (((t - t_lo) % kFlushTiles) == kFlushTiles - 1) {
+        if (!SPLIT || (t & 1)) {  // 256 terms at most
 #pragma unroll
-            for (int u = 0; u < QPT; ++u) S[u].flush(c2);
+            for (int u = 0; u < QPT; ++u) S[u].template flush<SPLIT>(c2);
         }
     }
-    __syncthreads();  // the tile's memory becomes the warps' parts
-    PartT* parts = reinterpret_cast<PartT*>(s_buf);
+    if constexpr (!SPLIT) {
 #pragma unroll
-    for (int u = 0; u < QPT; ++u) {
-        S[u].flush(c2);
-        PartT p;
-        p.v = S[u].av;
-        if (GRAD) for (int c = 0; c < 3; ++c) p.g[c] = S[u].ag[c];
-        p.ref = S[u].ref;
-        parts[warp * kGroup + 32 * u + lane] = p;
-    }
-    __syncthreads();
-    if (threadIdx.x < kGroup)
-        s_block[threadIdx.x] = sum_parts<KIND, FP64, GRAD>(kBruteWarps, kp.alpha,
-                                                           [&](int k) { return parts[k * kGroup + threadIdx.x]; });
-    cluster.sync();
-    const int64_t j = q0 + threadIdx.x;
-    if (rank == 0 && threadIdx.x < kGroup && j < nq) {
-        const PartT s = sum_parts<KIND, FP64, GRAD>(
-            ranks, kp.alpha, [&](int k) { return *cluster.map_shared_rank(&s_block[threadIdx.x], k); });
-        const double v = (double)s.v;
-        if constexpr (KIND == SBH_SMOOTHDIST) {
-            const bool pos = v > 0.0;
-            out[j] = pos ? (float)((double)s.ref - log(v) / (double)kp.alpha) : __int_as_float(0x7F800000);
-            if constexpr (GRAD)  // d = ref - log(acc) / alpha: grad d = -grad acc / (alpha acc); alpha cancels
-                for (int c = 0; c < 3; ++c)
-                    grad[3 * j + c] = pos ? (float)(-(double)s.g[c] / v) : __int_as_float(0x7FC00000);
-        } else {
-            const double f = KIND == SBH_WINDING ? 0.07957747154594766788 : 1.0;  // 1 / (4 pi)
-            out[j] = (float)(v * f);
-            if constexpr (GRAD)
-                for (int c = 0; c < 3; ++c) grad[3 * j + c] = (float)((double)s.g[c] * f);
+        for (int u = 0; u < QPT; ++u) {
+            const int64_t j = q0 + 32 * u + lane;
+            if (j < nq) write_query<KIND, GRAD>(j, S[u].av, S[u].ag, S[u].ref, kp, out, grad);
         }
+    } else {
+        __shared__ PartT s_block[kGroup];
+        __syncthreads();  // the tile's memory becomes the warps' parts
+        PartT* parts = reinterpret_cast<PartT*>(s_buf);
+#pragma unroll
+        for (int u = 0; u < QPT; ++u) {
+            S[u].template flush<SPLIT>(c2);
+            PartT p;
+            p.v = S[u].av;
+            if (GRAD) for (int c = 0; c < 3; ++c) p.g[c] = S[u].ag[c];
+            p.ref = S[u].ref;
+            parts[warp * kGroup + 32 * u + lane] = p;
+        }
+        __syncthreads();
+        if (threadIdx.x < kGroup)
+            s_block[threadIdx.x] = sum_parts<KIND, FP64, GRAD>(kBruteWarps, kp.alpha,
+                                                               [&](int k) { return parts[k * kGroup + threadIdx.x]; });
+        cluster.sync();
+        const int64_t j = q0 + threadIdx.x;
+        if (rank == 0 && threadIdx.x < kGroup && j < nq) {
+            const PartT s = sum_parts<KIND, FP64, GRAD>(
+                ranks, kp.alpha, [&](int k) { return *cluster.map_shared_rank(&s_block[threadIdx.x], k); });
+            write_query<KIND, GRAD>(j, s.v, s.g, s.ref, kp, out, grad);
+        }
+        cluster.sync();  // no block leaves while its sums are being read
     }
-    cluster.sync();  // no block leaves while its sums are being read
 }
 
-template <int KIND, bool FP64, bool GRAD, int QPT>
-cudaError_t launch_group(const float* P, const float* W, const float* N, int64_t n, const float* Q, int64_t nq,
-                         const KernelParams& kp, float* out, float* grad, cudaStream_t s)
+struct BruteCall {
+    const float *P, *W, *N;
+    int64_t n;
+    const float* Q;
+    int64_t nq;
+    KernelParams kp;
+    float *out, *grad;
+    cudaStream_t s;
+};
+
+template <int KIND, bool FP64, bool GRAD, int QPT, bool SPLIT>
+cudaError_t launch_group(const BruteCall& B)
 {
-    // as many blocks to a cluster as there are tiles for, at most eight
-    int ranks = kMaxCluster;
-    while (ranks > 1 && (int64_t)ranks * kBruteTile > n) ranks /= 2;
-    const int64_t groups = (nq + 32 * QPT - 1) / (32 * QPT);
+    const int64_t per_block = 32 * QPT * (SPLIT ? 1 : kBruteWarps);
+    const int64_t groups = (B.nq + per_block - 1) / per_block;
+    // as many blocks to a cluster as fill the chip several times over, a tile to each at least, eight at most
+    int ranks = 1;
+    while (SPLIT && ranks < kMaxCluster && groups * ranks < 16 * (int64_t)device_sm_count() &&
+           2 * (int64_t)ranks * kBruteTile <= B.n)
+        ranks *= 2;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(groups * ranks));
     cfg.blockDim = dim3(kBruteThreads);
-    cfg.stream = s;
+    cfg.stream = B.s;
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeClusterDimension;
     attr.val.clusterDim.x = (unsigned)ranks;
     attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_brute<KIND, FP64, GRAD, QPT>, P, W, N, n, Q, nq, kp, out, grad);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_brute<KIND, FP64, GRAD, QPT, SPLIT>, B.P, B.W, B.N, B.n, B.Q, B.nq,
+                                             B.kp, B.out, B.grad);
     if (e == cudaSuccess) note_launch();
     return e;
 }
 
-// Queries to a lane: four (the shared-memory reads of a source then cost a quarter each) where that
-// still leaves several blocks to every SM, else two; the gradient's sums have registers for two
+// Which way a call goes. Joining the parts of a query that was split costs about as much as 200 to 800 of
+// its terms (FP64 additions, and for the smooth distance an FP64 exponential for each part), so
+// queries are split over warps only where that is what fills the chip, and over blocks only as
+// far. 10^6 queries, us: one query a thread and no packed pairs (the kernel before this one) / every call
+// split over eight warps and up to eight blocks / as now:
+//   sources             10                100               1000                 10^4
+//   Coulomb             29 / 85 / 26      53 / 85 / 48      304 / 264 / 247      2,800 / 3,615 / 2,250
+//   smooth distance    141 / 499 / 109   306 / 482 / 115    775 / 596 / 548      6,440 / 8,398 / 5,106
+//   its gradient       240 / 783 / 186   660 / 818 / 187  1,430 / 1,224 / 711    8,840 / 18,081 / 6,410
+// Queries to a lane: four split (a shared-memory read of a source then costs each a quarter) where that
+// still leaves several blocks to every SM, else two; two unsplit, one where two would leave too few
+// blocks. The gradient's sums have registers for two, the smooth distance's are faster with one (5,270 / 5,459 us for
+// 2 10^6 queries against 4,096 sources). Sums kept in FP32 stay split over the warps where sources are many:
+// it is as fast, and their chains of additions are shorter.
 template <int KIND, bool FP64, bool GRAD>
-cudaError_t launch_kind(const float* P, const float* W, const float* N, int64_t n, const float* Q, int64_t nq,
-                        const KernelParams& kp, float* out, float* grad, cudaStream_t s)
+cudaError_t launch_kind(const BruteCall& B)
 {
-    if constexpr (!GRAD) {
-        if (nq >= (int64_t)128 * device_sm_count())
-            return launch_group<KIND, FP64, GRAD, 4>(P, W, N, n, Q, nq, kp, out, grad, s);
+    constexpr bool kSmoothGrad = GRAD && KIND == SBH_SMOOTHDIST;
+    const bool many = B.nq >= (kSmoothGrad ? 1 << 18 : 5 << 17) && (FP64 || B.n <= 4096);
+    if (many || B.n < (B.nq >= 1 << 16 ? 1024 : 128)) {
+        if constexpr (!kSmoothGrad) {
+            if (many) return launch_group<KIND, FP64, GRAD, 2, false>(B);
+        }
+        return launch_group<KIND, FP64, GRAD, 1, false>(B);
     }
-    return launch_group<KIND, FP64, GRAD, 2>(P, W, N, n, Q, nq, kp, out, grad, s);
+    if constexpr (!GRAD) {
+        if (B.nq >= (int64_t)128 * device_sm_count()) return launch_group<KIND, FP64, GRAD, 4, true>(B);
+    }
+    return launch_group<KIND, FP64, GRAD, 2, true>(B);
 }
 
 template <bool FP64, bool GRAD>
-cudaError_t launch_any(const float* P, const float* W, const float* N, int64_t n, const float* Q, int64_t nq,
-                       const KernelParams& kp, float* out, float* grad, cudaStream_t s)
+cudaError_t launch_any(const BruteCall& B)
 {
-    if (nq <= 0) return cudaSuccess;
+    if (B.nq <= 0) return cudaSuccess;
     cudaError_t e;
-    switch (kp.kind) {
-    case SBH_COULOMB: e = launch_kind<SBH_COULOMB, FP64, GRAD>(P, W, N, n, Q, nq, kp, out, grad, s); break;
-    case SBH_WINDING: e = launch_kind<SBH_WINDING, FP64, GRAD>(P, W, N, n, Q, nq, kp, out, grad, s); break;
-    case SBH_SMOOTHDIST: e = launch_kind<SBH_SMOOTHDIST, FP64, GRAD>(P, W, N, n, Q, nq, kp, out, grad, s); break;
-    case SBH_AFFINE: e = launch_kind<SBH_AFFINE, FP64, GRAD>(P, W, N, n, Q, nq, kp, out, grad, s); break;
+    switch (B.kp.kind) {
+    case SBH_COULOMB: e = launch_kind<SBH_COULOMB, FP64, GRAD>(B); break;
+    case SBH_WINDING: e = launch_kind<SBH_WINDING, FP64, GRAD>(B); break;
+    case SBH_SMOOTHDIST: e = launch_kind<SBH_SMOOTHDIST, FP64, GRAD>(B); break;
+    case SBH_AFFINE: e = launch_kind<SBH_AFFINE, FP64, GRAD>(B); break;
     default: return cudaErrorInvalidValue;
     }
     return e != cudaSuccess ? e : cudaGetLastError();
@@ -394,14 +455,14 @@ cudaError_t launch_any(const float* P, const float* W, const float* N, int64_t n
 cudaError_t launch_brute(const float* P, const float* W, const float* N, int64_t n, const float* Q, int64_t nq,
                          const KernelParams& kp, int fp64_accum, float* out, cudaStream_t s)
 {
-    return fp64_accum ? launch_any<true, false>(P, W, N, n, Q, nq, kp, out, nullptr, s)
-                      : launch_any<false, false>(P, W, N, n, Q, nq, kp, out, nullptr, s);
+    const BruteCall B = {P, W, N, n, Q, nq, kp, out, nullptr, s};
+    return fp64_accum ? launch_any<true, false>(B) : launch_any<false, false>(B);
 }
 
 cudaError_t launch_brute_grad(const float* P, const float* W, const float* N, int64_t n, const float* Q, int64_t nq,
                               const KernelParams& kp, float* out, float* grad, cudaStream_t s)
 {
-    return launch_any<true, true>(P, W, N, n, Q, nq, kp, out, grad, s);
+    return launch_any<true, true>({P, W, N, n, Q, nq, kp, out, grad, s});
 }
 
 }  // namespace sbh
