@@ -68,3 +68,18 @@ def test_uneven_shares_are_balanced(sbh):
         p, w = torch.rand(n, 3, device="cuda"), torch.ones(n, device="cuda")
         t.append(_time(lambda: sbh.sbh_eval_brute(p, w, q, "coulomb", out=out)))
     assert t[0] < 0.85 * t[1]
+
+
+@pytest.mark.parametrize("nq", [100, 70000])
+def test_the_largest_alpha_gives_the_nearest_source(sbh, nq):
+    """alpha only has to be finite: the smooth distance is then the smallest distance, a rounded root."""
+    rng = np.random.default_rng(nq)
+    p, q = rng.random((300, 3)).astype(np.float32), rng.random((nq, 3)).astype(np.float32)
+    w = np.ones(300, np.float32)
+    want = np.sqrt(((p[None].astype(np.float64) - q[:100, None]) ** 2).sum(2).min(1))
+    for alpha in (2.0e38, 3.0e38):
+        out, grad = sbh.sbh_eval_brute_grad(dev(p), dev(w), dev(q), "smoothdist", alpha=alpha)
+        for f in (out, sbh.sbh_eval_brute(dev(p), dev(w), dev(q), "smoothdist", alpha=alpha),
+                  sbh.sbh_eval_brute(dev(p), dev(w), dev(q), "smoothdist", fp64_accum=False, alpha=alpha)):
+            assert np.all(np.abs(f.cpu().numpy()[:100] - want) <= 1e-6 * want)
+        assert np.all(np.abs(np.linalg.norm(grad.cpu().numpy(), axis=1) - 1) < 1e-6)
