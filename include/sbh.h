@@ -54,6 +54,8 @@ typedef enum {
  *                   uses its dipole sum_j m_j n_j at its centre of mass. Needs normals.
  *   SBH_SMOOTHDIST  f = exp(-alpha |p - q|); the output is the smooth distance
  *                   -log(F) / alpha (Sec. 4.3.3), +inf where the estimate of F is <= 0.
+ *                   Sums are kept relative to the nearest source met: exponentials below 2^-126
+ *                   of its own count as 0.
  *   SBH_AFFINE      f = 1 + g . (p - q) with g = affine[0..2]: a test kernel, affine in p, for
  *                   which every contribution swap is zero and the estimator is exact. */
 typedef enum { SBH_COULOMB = 0, SBH_WINDING = 1, SBH_SMOOTHDIST = 2, SBH_AFFINE = 3 } sbh_kernel_kind;
