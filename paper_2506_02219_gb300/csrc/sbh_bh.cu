@@ -26,7 +26,8 @@
 // walk or its sum.
 //   2^20 winding sources, 2^21 grid queries, voting, theta 0.5: 8.04 -> 6.04 ms with the record and the
 // comparison, 5.06 ms with the term taken from the test's differences. 2^18 Coulomb sources, 10^6 random
-// queries, theta 0.8, no voting: 1.68 -> 0.67 ms sorted, lanes alone, 0.58 ms together.
+// queries, theta 0.8, no voting: 1.68 -> 0.67 ms sorted, lanes alone, 0.58 ms together
+// (0.60 with the fused sum of the Coulomb term; the call with its sort 0.69 ms).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -184,11 +185,15 @@ __global__ void __launch_bounds__(256) k_bh_eval(TreeView T, const float4* __res
 namespace {
 // Queries from which a walk without voting is sorted and walked together. The sort takes 30 us and 20 us per
 // million queries, and the fewer the queries, the further apart a warp's 32 are and the more nodes they
-// visit between them. theta 0.8, us sorted / not:
-//   2^18 sources, random queries   2^16: 440 / 167   2^18: 377 / 325   2^20: 658 / 1194
-//   2^20 sources, random queries   2^16: 549 / 179   2^18: 493 / 347   2^20: 791 / 1250
-//   2^18 sources, grid             2^16: 469 / 152   2^18: 352 / 245   2^20: 632 / 693
-//   2^14 sources, random queries   2^16: 192 / 113   2^18: 211 / 233   2^20: 463 / 935
+// visit between them; the larger theta, the less there is to gain. us sorted / not, at theta 0.5, 0.8, 1.2:
+//                                              2^18 queries                        2^19                                2^20
+//   Coulomb, 2^12 sources, grid         489/645   257/261   161/119     794/1211   387/466   221/206    1335/2277   622/840   331/342
+//   Coulomb, 2^18 sources, random      2268/3185  853/987   389/363    3316/6787  1226/2072  523/791   5029/12472 1870/3852  768/1365
+//   winding, 2^20 sources, grid        4508/5896 1722/1679  743/551    6889/11982 2526/3365 1033/1132 10471/22698 3779/6053 1539/1873
+//   smooth distance, 2^14, random      1170/1496  523/533   263/219    1766/2910   788/1010  378/400   3021/5830  1245/1982  576/785
+//   smooth distance, 2^20, grid        4666/3940 1736/1138  777/380    6983/8161  2491/2281 1044/783  10253/14920 3762/4064 1550/1303
+// At 2^19 the smooth distance, whose terms cost most beside the reads, is the one that can lose, on a
+// grid at large theta; below, all of them do.
 constexpr int64_t kSortFrom = 1 << 19;
 
 struct BhLaunch {
