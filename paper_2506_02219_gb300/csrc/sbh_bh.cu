@@ -25,9 +25,10 @@
 // warp going through the nodes that any of its queries visits (kTogether): neither changes a query's
 // walk or its sum.
 //   2^20 winding sources, 2^21 grid queries, voting, theta 0.5: 8.04 -> 6.04 ms with the record and the
-// comparison, 5.06 ms with the term taken from the test's differences. 2^18 Coulomb sources, 10^6 random
-// queries, theta 0.8, no voting: 1.68 -> 0.67 ms sorted, lanes alone, 0.58 ms together
-// (0.60 with the fused sum of the Coulomb term; the call with its sort 0.69 ms).
+// comparison, 5.06 ms with the term taken from the test's differences, 3% less with the term formed
+// after the link to the next node. 2^18 Coulomb sources, 10^6 random queries, theta 0.8, no voting:
+// 1.68 -> 0.67 ms sorted, lanes alone, 0.58 ms together (0.60 with the fused sum of the Coulomb term;
+// the call with its sort 0.69 ms).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -100,13 +101,51 @@ __device__ float open_limit(float B, float beta)
 //              each other (sorted), whose nodes are mostly the same.
 enum { kAlone = 0, kVote = 1, kTogether = 2 };
 
-// REC: the kernel's walk records are there (else a node is read from the tree's arrays)
-template <int KIND, int MODE, bool REC>
+// What a step of the walk reads of node v, from the kernel's walk records (REC) or the tree's arrays
+template <int KIND, bool REC>
+struct Node {
+    float4 p, dp;         // (dp: the winding kernel's dipole)
+    int32_t skip, first;  // (first: where the record has it)
+    int lvl;              // level times 4
+    bool point;
+};
+template <int KIND, bool REC>
+__device__ __forceinline__ Node<KIND, REC> load_node(const TreeView& T, const float4* __restrict__ rec, int32_t v)
+{
+    Node<KIND, REC> n;
+    n.first = 0;
+    if constexpr (REC && KIND == SBH_WINDING) {
+        n.p = __ldg(rec + 2 * (int64_t)v);
+        n.dp = __ldg(rec + 2 * (int64_t)v + 1);
+        n.lvl = __float_as_int(n.p.w);
+        n.skip = __float_as_int(n.dp.w);
+        n.point = n.lvl == kWalkPoint;
+    } else if constexpr (REC) {
+        float4 r;
+        ld_pmd(rec, v, n.p, r);
+        n.first = __float_as_int(r.x);
+        n.skip = __float_as_int(r.y);
+        n.lvl = __float_as_int(r.z);
+        n.point = n.first < 0;
+    } else {
+        n.p = __ldg(&T.pm[v]);
+        if constexpr (KIND == SBH_WINDING) n.dp = __ldg(&T.dip[v]);
+        const uint32_t m = __ldg(&T.meta[v]);
+        n.skip = __ldg(&T.skip[v]);
+        n.lvl = 4 * (int)meta_level(m);
+        n.point = meta_kind(m) == kPoint;
+    }
+    return n;
+}
+
+// AHEAD: the next node is asked for before the node's term is formed (kAheadTo)
+template <int KIND, int MODE, bool REC, bool AHEAD>
 __global__ void __launch_bounds__(256) k_bh_eval(TreeView T, const float4* __restrict__ rec,
                                                  const float* __restrict__ Q, int64_t nq, KernelParams kp, float beta,
                                                  const int32_t* __restrict__ order, const int32_t* sort_error,
                                                  float* __restrict__ out)
 {
+    constexpr bool kLate = AHEAD || MODE == kVote;  // the term after the link (voting 3% faster, together 2% slower)
     __shared__ float s_limit[kDiamLevels];
     if (threadIdx.x < kDiamLevels) s_limit[threadIdx.x] = open_limit(T.ctrl->diam[threadIdx.x], beta);
     __syncthreads();
@@ -128,49 +167,27 @@ __global__ void __launch_bounds__(256) k_bh_eval(TreeView T, const float4* __res
         // a depth-first walk enters every node at most once; the bound only guards a damaged tree
         int32_t budget = n_nodes + 1;
         if (MODE != kAlone || active) {
+            Node<KIND, REC> node;
+            if constexpr (AHEAD) node = load_node<KIND, REC>(T, rec, 0);
             while (v >= 0 && budget-- > 0) {
-                float4 p;
-                int32_t skip = 0, first = 0;
-                float limit;
-                bool point;
-                float4 dp;
-                if constexpr (REC) {
-                    const float4* at = rec + 2 * (int64_t)v;
-                    int lvl;
-                    if constexpr (KIND == SBH_WINDING) {
-                        p = __ldg(at);
-                        dp = __ldg(at + 1);
-                        lvl = __float_as_int(p.w);
-                        skip = __float_as_int(dp.w);
-                        point = lvl == kWalkPoint;
-                    } else {
-                        float4 r;
-                        ld_pmd(rec, v, p, r);
-                        first = __float_as_int(r.x);
-                        skip = __float_as_int(r.y);
-                        lvl = __float_as_int(r.z);
-                        point = first < 0;
-                    }
-                    limit = *reinterpret_cast<const float*>(reinterpret_cast<const char*>(s_limit) + lvl);
-                } else {
-                    p = __ldg(&T.pm[v]);
-                    if constexpr (KIND == SBH_WINDING) dp = __ldg(&T.dip[v]);
-                    const uint32_t m = __ldg(&T.meta[v]);
-                    limit = s_limit[meta_level(m)];
-                    point = meta_kind(m) == kPoint;
-                }
+                if constexpr (!AHEAD) node = load_node<KIND, REC>(T, rec, v);
+                const Node<KIND, REC> at = node;
+                const float4 p = at.p;
+                const float limit = *reinterpret_cast<const float*>(reinterpret_cast<const char*>(s_limit) + at.lvl);
                 // dist2_rn, its differences kept
                 const float3 d = make_float3(__fsub_rn(p.x, q.x), __fsub_rn(p.y, q.y), __fsub_rn(p.z, q.z));
                 const float r2 = __fadd_rn(__fadd_rn(__fmul_rn(d.x, d.x), __fmul_rn(d.y, d.y)), __fmul_rn(d.z, d.z));
-                bool use = point || r2 >= limit;
+                bool use = at.point || r2 >= limit;
                 if (MODE == kVote) use = __all_sync(0xFFFFFFFFu, use || !active);
                 const bool mine = MODE == kTogether ? own == v : active;
-                if (use && mine) bh_add<KIND>(p, KIND == SBH_WINDING ? dp : p, d, kp, acc, ex);
-                if constexpr (!REC) skip = use ? __ldg(&T.skip[v]) : 0;
+                if (!kLate && use && mine) bh_add<KIND>(p, KIND == SBH_WINDING ? at.dp : p, d, kp, acc, ex);
                 const bool open = MODE == kTogether ? __any_sync(0xFFFFFFFFu, mine && !use) : !use;
+                int32_t first = at.first;
                 if (!REC || KIND == SBH_WINDING) first = open ? __ldg(&T.fc[v]) : 0;
-                if (MODE == kTogether && mine) own = use ? skip : first;
-                v = open ? first : skip;
+                if (MODE == kTogether && mine) own = use ? at.skip : first;
+                v = open ? first : at.skip;
+                if constexpr (AHEAD) node = load_node<KIND, REC>(T, rec, v < 0 ? 0 : v);
+                if (kLate && use && mine) bh_add<KIND>(p, KIND == SBH_WINDING ? at.dp : p, d, kp, acc, ex);
             }
         }
         if (v >= 0) acc = ex.acc = __int_as_float(0x7FC00000);  // walk did not finish: NaN
@@ -196,6 +213,14 @@ namespace {
 // grid at large theta; below, all of them do.
 constexpr int64_t kSortFrom = 1 << 19;
 
+// Queries up to which a walk asks for the next node before it forms a node's term, to an SM: the wait for a
+// node is then all that a step takes, where few warps share an SM, but it takes 5 to 13 registers more,
+// and warps where there are many. 16 warps to an SM; times with / without, over three kernels, 5,000 to 2^20
+// sources, theta 0.5 and 0.9: 20,000 queries 0.76 to 0.95, 78,000 0.77 to 1.04, 155,000 0.88 to 1.16, 310,000
+// 0.98 to 1.29. (Without it a walk that opens every node, at theta 0, took up to a quarter longer from
+// the records, a 32-byte sector each, than from the arrays, which hold neighbours in one sector.)
+constexpr int64_t kAheadTo = 512;
+
 struct BhLaunch {
     TreeView T;
     const float4* rec;
@@ -210,19 +235,26 @@ struct BhLaunch {
     unsigned blocks;
 };
 
-template <int KIND, int MODE, bool REC>
+template <int KIND, int MODE, bool REC, bool AHEAD>
 void launch_bh(const BhLaunch& L)
 {
-    k_bh_eval<KIND, MODE, REC><<<L.blocks, 256, 0, L.s>>>(L.T, L.rec, L.Q, L.nq, L.kp, L.beta, L.order, L.sort_error, L.out);
+    k_bh_eval<KIND, MODE, REC, AHEAD><<<L.blocks, 256, 0, L.s>>>(L.T, L.rec, L.Q, L.nq, L.kp, L.beta, L.order, L.sort_error, L.out);
     note_launch();
+}
+
+template <int KIND, int MODE>
+void launch_bh_mode(const BhLaunch& L)
+{
+    if (L.nq <= kAheadTo * device_sm_count()) L.rec ? launch_bh<KIND, MODE, true, true>(L) : launch_bh<KIND, MODE, false, true>(L);
+    else L.rec ? launch_bh<KIND, MODE, true, false>(L) : launch_bh<KIND, MODE, false, false>(L);
 }
 
 template <int KIND>
 void launch_bh_kind(const BhLaunch& L, bool vote)
 {
-    if (vote) L.rec ? launch_bh<KIND, kVote, true>(L) : launch_bh<KIND, kVote, false>(L);
-    else if (L.rec) L.order ? launch_bh<KIND, kTogether, true>(L) : launch_bh<KIND, kAlone, true>(L);
-    else launch_bh<KIND, kAlone, false>(L);
+    if (vote) launch_bh_mode<KIND, kVote>(L);
+    else if (L.order) launch_bh<KIND, kTogether, true, false>(L);
+    else launch_bh_mode<KIND, kAlone>(L);
 }
 }  // namespace
 

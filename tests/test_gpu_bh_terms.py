@@ -20,3 +20,26 @@ def test_coulomb_term(sbh, nq, normals, vote):
     for softening in (0.0, 1e-3, 0.3):
         assert torch.equal(sbh.sbh_eval_bh(tree, q, "coulomb", 0.5, vote, softening=softening),
                            sbh.sbh_eval_brute(p, w, q, "coulomb", softening=softening))
+
+
+@pytest.mark.parametrize("vote", [False, True])
+@pytest.mark.parametrize("kind,normals", [("coulomb", False), ("coulomb", True), ("winding", True), ("smoothdist", False),
+                                          ("affine", True)])
+def test_few_queries_walk_as_many_do(sbh, kind, normals, vote):
+    """Up to 512 queries to an SM a walk asks for its nodes ahead: the same sums as in a larger call."""
+    import torch
+    rng = np.random.default_rng(8)
+    n = 20000
+    p = rng.random((n, 3)).astype(np.float32)
+    p[15000:] = p[15000]  # a leaf of 5,000 points
+    w, v = rng.random(n) + 0.5, rng.normal(size=(n, 3))
+    tree = sbh.sbh_build(dev(p), dev(w), dev(v) if normals else None, leaf_size=3)
+    few = 512 * torch.cuda.get_device_properties(0).multi_processor_count
+    q = dev(rng.random((few + 32, 3)) * 3 - 1)
+    for theta in (0.0, 0.4, 1.1):
+        m = 2048 if theta == 0.0 else few
+        many = sbh.sbh_eval_bh(tree, q if m == few else q[:m].repeat(41, 1), kind, theta, vote)
+        for a, b in ((0, 1), (0, 33), (0, m)):
+            if vote and b % 32:  # a vote's queries are a warp's: none left out of the last one
+                continue
+            assert torch.equal(sbh.sbh_eval_bh(tree, q[a:b], kind, theta, vote), many[a:b])
