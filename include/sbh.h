@@ -290,7 +290,8 @@ SBH_API uint64_t sbh_memory_in_use(void);
  * single point or ||q - p_a|| / |B_a| >= beta = 1 / theta (theta = 0 gives the exact sum).
  * warp_vote = 1 takes the decision jointly for the 32 queries of a warp (a node is opened when
  * any of them needs it); 0 decides per query, exactly as Algorithm 1. The first call builds the
- * 8-ary tree (enqueued on `stream`). */
+ * 8-ary tree (enqueued on `stream`); should a bounded wait of that build ever give up, every
+ * result of the tree is NaN. */
 SBH_API sbh_status sbh_eval_bh(sbh_tree* tree, const float* queries, int64_t nq, sbh_kernel kernel,
                        float theta, int32_t warp_vote, float* out, void* stream);
 

@@ -25,10 +25,9 @@
 // warp going through the nodes that any of its queries visits (kTogether): neither changes a query's
 // walk or its sum.
 //   2^20 winding sources, 2^21 grid queries, voting, theta 0.5: 8.04 -> 6.04 ms with the record and the
-// comparison, 5.06 ms with the term taken from the test's differences, 3% less with the term formed
-// after the link to the next node. 2^18 Coulomb sources, 10^6 random queries, theta 0.8, no voting:
-// 1.68 -> 0.67 ms sorted, lanes alone, 0.58 ms together (0.60 with the fused sum of the Coulomb term;
-// the call with its sort 0.69 ms).
+// comparison, 5.06 ms with the term taken from the test's differences. 2^18 Coulomb sources, 10^6 random
+// queries, theta 0.8, no voting: 1.68 -> 0.67 ms sorted, lanes alone, 0.58 ms together (0.60 with the
+// fused sum of the Coulomb term; the call with its sort 0.69 ms).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -105,11 +104,11 @@ enum { kAlone = 0, kVote = 1, kTogether = 2 };
 template <int KIND, bool REC>
 struct Node {
     float4 p, dp;         // (dp: the winding kernel's dipole)
-    int32_t skip, first;  // (first: where the record has it)
+    int32_t skip, first;  // (first: where the record has it; skip: there, or asked for ahead)
     int lvl;              // level times 4
     bool point;
 };
-template <int KIND, bool REC>
+template <int KIND, bool REC, bool AHEAD>
 __device__ __forceinline__ Node<KIND, REC> load_node(const TreeView& T, const float4* __restrict__ rec, int32_t v)
 {
     Node<KIND, REC> n;
@@ -131,7 +130,7 @@ __device__ __forceinline__ Node<KIND, REC> load_node(const TreeView& T, const fl
         n.p = __ldg(&T.pm[v]);
         if constexpr (KIND == SBH_WINDING) n.dp = __ldg(&T.dip[v]);
         const uint32_t m = __ldg(&T.meta[v]);
-        n.skip = __ldg(&T.skip[v]);
+        n.skip = AHEAD ? __ldg(&T.skip[v]) : 0;
         n.lvl = 4 * (int)meta_level(m);
         n.point = meta_kind(m) == kPoint;
     }
@@ -145,7 +144,6 @@ __global__ void __launch_bounds__(256) k_bh_eval(TreeView T, const float4* __res
                                                  const int32_t* __restrict__ order, const int32_t* sort_error,
                                                  float* __restrict__ out)
 {
-    constexpr bool kLate = AHEAD || MODE == kVote;  // the term after the link (voting 3% faster, together 2% slower)
     __shared__ float s_limit[kDiamLevels];
     if (threadIdx.x < kDiamLevels) s_limit[threadIdx.x] = open_limit(T.ctrl->diam[threadIdx.x], beta);
     __syncthreads();
@@ -168,9 +166,9 @@ __global__ void __launch_bounds__(256) k_bh_eval(TreeView T, const float4* __res
         int32_t budget = n_nodes + 1;
         if (MODE != kAlone || active) {
             Node<KIND, REC> node;
-            if constexpr (AHEAD) node = load_node<KIND, REC>(T, rec, 0);
+            if constexpr (AHEAD) node = load_node<KIND, REC, AHEAD>(T, rec, 0);
             while (v >= 0 && budget-- > 0) {
-                if constexpr (!AHEAD) node = load_node<KIND, REC>(T, rec, v);
+                if constexpr (!AHEAD) node = load_node<KIND, REC, AHEAD>(T, rec, v);
                 const Node<KIND, REC> at = node;
                 const float4 p = at.p;
                 const float limit = *reinterpret_cast<const float*>(reinterpret_cast<const char*>(s_limit) + at.lvl);
@@ -180,14 +178,16 @@ __global__ void __launch_bounds__(256) k_bh_eval(TreeView T, const float4* __res
                 bool use = at.point || r2 >= limit;
                 if (MODE == kVote) use = __all_sync(0xFFFFFFFFu, use || !active);
                 const bool mine = MODE == kTogether ? own == v : active;
-                if (!kLate && use && mine) bh_add<KIND>(p, KIND == SBH_WINDING ? at.dp : p, d, kp, acc, ex);
+                if (!AHEAD && use && mine) bh_add<KIND>(p, KIND == SBH_WINDING ? at.dp : p, d, kp, acc, ex);
+                int32_t skip = at.skip;
+                if constexpr (!REC && !AHEAD) skip = use ? __ldg(&T.skip[v]) : 0;
                 const bool open = MODE == kTogether ? __any_sync(0xFFFFFFFFu, mine && !use) : !use;
                 int32_t first = at.first;
                 if (!REC || KIND == SBH_WINDING) first = open ? __ldg(&T.fc[v]) : 0;
-                if (MODE == kTogether && mine) own = use ? at.skip : first;
-                v = open ? first : at.skip;
-                if constexpr (AHEAD) node = load_node<KIND, REC>(T, rec, v < 0 ? 0 : v);
-                if (kLate && use && mine) bh_add<KIND>(p, KIND == SBH_WINDING ? at.dp : p, d, kp, acc, ex);
+                if (MODE == kTogether && mine) own = use ? skip : first;
+                v = open ? first : skip;
+                if constexpr (AHEAD) node = load_node<KIND, REC, AHEAD>(T, rec, v < 0 ? 0 : v);
+                if (AHEAD && use && mine) bh_add<KIND>(p, KIND == SBH_WINDING ? at.dp : p, d, kp, acc, ex);
             }
         }
         if (v >= 0) acc = ex.acc = __int_as_float(0x7FC00000);  // walk did not finish: NaN

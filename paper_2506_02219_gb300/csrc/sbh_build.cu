@@ -731,7 +731,7 @@ __global__ void __launch_bounds__(kTopoThreads) k_gather(const float* __restrict
 //    many points are dropped from A_i (kSmallLeaf marks that ancestor).
 //    What bounds it: a few passes over the positions, one for each generation in the last kernel. It
 //    replaces seven kernels over all positions for every generation: 84 kernels and 1,180 us for 2^22
-//    points, now 5 and 174 us (2^20: 470 -> 58 us)
+//    points, now four and 155 us (2^20: 470 -> 54 us)
 // ----------------------------------------------------------------------------------------------
 constexpr uint32_t kSmallLeaf = 1u << 31;  // in a mask: its last level is a leaf for its size
 

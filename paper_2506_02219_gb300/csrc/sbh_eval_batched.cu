@@ -203,7 +203,7 @@ __device__ __forceinline__ float node_value(const TreeView& T, const Stage& S, i
 
 // child index (0-based) picked by the 24-bit draw x: mass -> the number of prefix fractions <= u
 // among all but the last child; count -> the child holding point floor(u * |T|) of the node's
-// range. Mass: the scan starts at the guide entry of u's slot floor(u nc) (k_guide), a lower bound
+// range. Mass: the scan starts at the guide entry of u's slot floor(u nc) (guide_entry), a lower bound
 // of that number, and steps up while the prefix fractions (nondecreasing) are <= u: the same
 // index as counting, in one or two reads on average. Count: binary search over the child ranges.
 __device__ __forceinline__ int pick_child(const TreeView& T, const Stage& S, int32_t node, int32_t f, int nc, uint32_t x,

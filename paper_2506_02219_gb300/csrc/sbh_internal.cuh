@@ -75,7 +75,7 @@ struct TreeView {
     const float4* dip;    // (sum_j m_j n_j; 0) or nullptr
     const float4* pmd;    // [2 v], [2 v + 1]: pm[v] and dip[v] as one 32-byte record, or nullptr
     const float* cdf;     // prefix fraction of the node's mass among its siblings (last = 1)
-    const uint8_t* gd;    // the parent's child-pick guide entry for this node's slot (k_guide)
+    const uint8_t* gd;    // the parent's child-pick guide entry for this node's slot (guide_entry)
     const int32_t* fc;    // first child, -1 for a point
     const uint32_t* meta; // nchild | level << 24 | kind << 30
     const int32_t* nb;    // first sorted point
