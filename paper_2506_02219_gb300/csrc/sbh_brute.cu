@@ -258,14 +258,21 @@ __device__ __forceinline__ void write_query(int64_t j, Acc sum, const Acc* g, fl
     }
 }
 
-// blocks to an SM asked for (0: as it comes): three of the smooth distance's gradient, 2.52 -> 2.29 ms for 5,001
-// queries against 2^19 sources (at 80 registers either way)
-template <int KIND, bool GRAD, bool SPLIT>
-constexpr int brute_blocks() { return KIND == SBH_SMOOTHDIST && GRAD && SPLIT ? 3 : 0; }
+// Blocks to an SM that a split kernel is compiled for (0: as it comes). Left alone, some get a few registers
+// more than a block more would allow, others fewer than they could use. With these, against without:
+// the smooth distance 0.92 of the time (28 sizes), its gradient 2.52 -> 2.29 ms (5,001 queries, 2^19 sources),
+// winding gradients 0.93 to 1.00 (two blocks either way, at 90 registers without).
+template <int KIND, bool FP64, bool GRAD, bool SPLIT>
+constexpr int brute_blocks()
+{
+    if (!SPLIT) return 0;
+    if (GRAD) return KIND == SBH_WINDING ? 2 : 3;
+    return KIND == SBH_SMOOTHDIST && FP64 ? 4 : 0;
+}
 
 // SPLIT: the warps of a block work on the same queries, else each on its own
 template <int KIND, bool FP64, bool GRAD, int QPT, bool SPLIT>
-__global__ void __launch_bounds__(kBruteThreads, brute_blocks<KIND, GRAD, SPLIT>()) k_brute(
+__global__ void __launch_bounds__(kBruteThreads, brute_blocks<KIND, FP64, GRAD, SPLIT>()) k_brute(
     const float* __restrict__ P, const float* __restrict__ W, const float* __restrict__ N, int64_t n,
     const float* __restrict__ Q, int64_t nq, KernelParams kp, float c2, float* __restrict__ out, float* __restrict__ grad)
 {
@@ -281,9 +288,9 @@ __global__ void __launch_bounds__(kBruteThreads, brute_blocks<KIND, GRAD, SPLIT>
     const int rank = SPLIT ? (int)cluster.block_rank() : 0, ranks = SPLIT ? (int)cluster.num_blocks() : 1;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t q0 = (SPLIT ? (int64_t)(blockIdx.x / ranks) : (int64_t)blockIdx.x * kBruteWarps + warp) * kGroup;
-    // this block's sources, as evenly as whole pairs go
-    const int64_t s_lo = (n * rank / ranks) & ~(int64_t)1;
-    const int64_t s_hi = rank == ranks - 1 ? n : (n * (rank + 1) / ranks) & ~(int64_t)1;
+    // this block's sources: as even shares as whole 128s go, so that loads start on a line
+    const int64_t s_lo = (n * rank / ranks) & ~(int64_t)127;
+    const int64_t s_hi = rank == ranks - 1 ? n : (n * (rank + 1) / ranks) & ~(int64_t)127;
 
     Sums<KIND, FP64, GRAD> S[QPT];
 #pragma unroll
